@@ -152,12 +152,16 @@ __device__ __forceinline__ void store_w(uint8_t* planes, uint32_t wplane, int K,
   for (int pl = 0; pl < P::planes; ++pl) *reinterpret_cast<__nv_bfloat16*>(planes + pl * wplane + off) = e[pl];
 }
 
-// D[128][N] (+)= A[128][K] * B[N][K]^T over the part products i + j < planes, one thread
+// D[128][N] (+)= A[128][K] * B[N][K]^T over the part products i + j < planes, one thread.  The
+// operand descriptors of the series are the first one's plus constants: built from their
+// addresses each, the issuing thread spent about 15 instructions per MMA, which the whole
+// group waits for.
 template <class P, int N, int K>
 __device__ __forceinline__ void issue_mma(uint32_t d, uint32_t a0, uint32_t b0, uint32_t wplane) {
   constexpr uint32_t sbo = (uint32_t)(K * P::es / 16) * 128u;
   constexpr uint32_t idesc = tc::instr_desc(P::kind, 128, N);
   constexpr uint32_t aplane = 128u * 32u * P::es;
+  const uint32_t alo = tc::desc_lo(a0, 128u), blo = tc::desc_lo(b0, 128u);
   bool first = true;
 #pragma unroll
   for (int s = 0; s < K / P::kmma; ++s) {
@@ -168,8 +172,8 @@ __device__ __forceinline__ void issue_mma(uint32_t d, uint32_t a0, uint32_t b0, 
 #pragma unroll
       for (int i = 0; i <= sum; ++i) {
         const int jj = sum - i;
-        tc::mma_bf16(d, tc::smem_desc(a0 + i * aplane + off, 128u, sbo),
-                     tc::smem_desc(b0 + jj * wplane + off, 128u, sbo), idesc, first ? 0u : 1u);
+        tc::mma_bf16(d, tc::desc_of(alo + ((i * aplane + off) >> 4), tc::desc_hi(sbo)),
+                     tc::desc_of(blo + ((jj * wplane + off) >> 4), tc::desc_hi(sbo)), idesc, first ? 0u : 1u);
         first = false;
       }
   }
@@ -183,19 +187,21 @@ template <int APL, int BPL, int SUM, int N>
 __device__ __forceinline__ void issue_mma_dw(uint32_t d, uint32_t a0, uint32_t a_plane, uint32_t a_kstride,
                                              uint32_t b0, uint32_t b_plane, uint32_t b_kstride, bool acc) {
   constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 64, N) | (1u << 15) | (1u << 16);
-#pragma unroll 1
+  uint32_t alo = tc::desc_lo(a0, a_kstride), blo = tc::desc_lo(b0, b_kstride);
+#pragma unroll 2
   for (int s = 0; s < 8; ++s) {  // K = 128 samples, 16 per MMA
-    const uint32_t oa = (uint32_t)s * 2u * a_kstride, ob = (uint32_t)s * 2u * b_kstride;
 #pragma unroll
     for (int sum = SUM - 1; sum >= 0; --sum)
 #pragma unroll
       for (int i = 0; i <= sum; ++i) {
         const int j = sum - i;
         if (i >= APL || j >= BPL) continue;
-        tc::mma_bf16(d, tc::smem_desc(a0 + i * a_plane + oa, a_kstride, 128u),
-                     tc::smem_desc(b0 + j * b_plane + ob, b_kstride, 128u), idesc, acc ? 1u : 0u);
+        tc::mma_bf16(d, tc::desc_of(alo + ((i * a_plane) >> 4), tc::desc_hi(128u)),
+                     tc::desc_of(blo + ((j * b_plane) >> 4), tc::desc_hi(128u)), idesc, acc ? 1u : 0u);
         acc = true;
       }
+    alo += (2u * a_kstride) >> 4;
+    blo += (2u * b_kstride) >> 4;
   }
 }
 

@@ -33,6 +33,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;
 }
 
+// The same descriptor in halves, for a series of operands that differ only in their start
+// address: the high word holds no address bits, and an operand `bytes` further on (bytes a
+// multiple of 16, inside shared memory) has the low word + bytes / 16.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo) { return (saddr >> 4) | ((lbo >> 4) << 16); }
+__host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
+
 enum Kind { KIND_TF32 = 0, KIND_BF16 = 1 };
 
 // Instruction descriptor for kind::tf32 / kind::f16: D = F32, A and B K-major,
@@ -98,6 +105,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* mbar, uint32_t parity, u
       : "r"(smem_u32(mbar)), "r"(parity), "r"(hint_ns)
       : "memory");
   return ok != 0;
+}
+// one look at the barrier, without suspending
+__device__ __forceinline__ bool mbar_test(uint64_t* mbar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(mbar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 // bounded wait: false after `limit` tries of up to 2 us each (the caller records an error and leaves)
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint32_t limit) {
