@@ -134,8 +134,7 @@ gs_status gs_create(const gs_config* cfg, gs_ctx** out) {
   long long off = 0;
   for (int l = 0; l < GS_LEVELS; ++l) {
     for (int a = 0; a < 3; ++a) g.dims[l][a] = cfg->dims[l][a];
-    g.voxel[l] = cfg->voxel[l];
-    g.inv_voxel[l] = 1.0f / cfg->voxel[l];
+    gs::set_voxel(g, l, cfg->voxel[l]);
     g.off[l] = off;
     off += level_floats(cfg, l);
   }

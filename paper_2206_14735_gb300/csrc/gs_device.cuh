@@ -1,6 +1,7 @@
 // Device-side building blocks of the GO-Surf step shared by the kernels of this library.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "gosurf.h"
@@ -27,6 +28,9 @@ struct GridDesc {
   int dims[kLevels][3];
   float voxel[kLevels];
   float inv_voxel[kLevels];
+  // x / voxel as the correctly rounded quotient without a division (cell_coord): a power of two
+  // that brings the voxel edge into [1, 2), the edge times it, and that product's reciprocal
+  float div_scale[kLevels], div_voxel[kLevels], div_recip[kLevels];
   float origin[3];
   long long off[kLevels];  // float offset of each level in theta
   long long n_grid;
@@ -58,6 +62,34 @@ struct Cell {
   int idx[3];     // base vertex per axis
 };
 
+// Host: the voxel edge of level l and the constants that go with it.
+inline void set_voxel(GridDesc& g, int l, float voxel) {
+  g.voxel[l] = voxel;
+  g.inv_voxel[l] = 1.0f / voxel;
+  int e = 0;
+  frexpf(voxel, &e);                   // voxel = m 2^e, m in [1/2, 1)
+  if (e < -125) e = -125;              // subnormal edges: the scale stays finite
+  g.div_scale[l] = ldexpf(1.0f, 1 - e);
+  g.div_voxel[l] = voxel * g.div_scale[l];  // exact
+  g.div_recip[l] = 1.0f / g.div_voxel[l];
+}
+
+// d / voxel_l rounded to nearest, by Markstein's scheme (P. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990): with y the correctly
+// rounded reciprocal, one residual step makes q faithful and a second one, on a faithful q,
+// correctly rounded.  The divisor is a constant of the level, so y comes with it: 6 operations
+// and a select in place of a division's reciprocal, its own steps and its range check with the
+// branch behind it; a sample needs 24 of them.  The power of two is exact, and keeps the
+// products clear of overflow; a quotient beyond 2^100 (or not finite) is left as it is: the
+// caller clamps it to the grid.
+__host__ __device__ __forceinline__ float cell_coord(float d, float scale, float voxel, float recip) {
+  const float a = d * scale;
+  const float q0 = a * recip;
+  const float q1 = fmaf(fmaf(-q0, voxel, a), recip, q0);
+  const float q2 = fmaf(fmaf(-q1, voxel, a), recip, q1);
+  return fabsf(q0) < 0x1p100f ? q2 : q0;
+}
+
 // Cell of x at level l: u = (x - origin) / v decided in binary32 (round-to-nearest),
 // clamped to [0, n-1], base = min(floor(u), n-2), f = u - base.
 __device__ __forceinline__ Cell locate(const GridDesc& g, int l, const float x[3]) {
@@ -67,7 +99,7 @@ __device__ __forceinline__ Cell locate(const GridDesc& g, int l, const float x[3
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int n = g.dims[l][a];
-    float u = __fdiv_rn(__fsub_rn(x[a], g.origin[a]), g.voxel[l]);
+    float u = cell_coord(__fsub_rn(x[a], g.origin[a]), g.div_scale[l], g.div_voxel[l], g.div_recip[l]);
     if (u < 0.0f) {
       u = 0.0f;
       c.clamped |= 1u << a;

@@ -87,8 +87,7 @@ extern "C" gs_status gs_forward_backward_noalloc(const gs_config* cfg, const flo
   long long off = 0;
   for (int l = 0; l < GS_LEVELS; ++l) {
     for (int a = 0; a < 3; ++a) c.grid.dims[l][a] = cfg->dims[l][a];
-    c.grid.voxel[l] = cfg->voxel[l];
-    c.grid.inv_voxel[l] = 1.0f / cfg->voxel[l];
+    gs::set_voxel(c.grid, l, cfg->voxel[l]);
     c.grid.off[l] = off;
     off += (long long)cfg->dims[l][0] * cfg->dims[l][1] * cfg->dims[l][2] * GS_FEAT;
   }
