@@ -13,7 +13,7 @@ constexpr int kSmoothCtas = 128;  // CTAs of the smoothness kernel (fixed, so pa
 constexpr int kRenderCtasPerSm = 1;  // persistent render CTAs per SM
 constexpr int kStoreFloatsPerSample = 100;  // stored activations: z 16, a1 32, (phi, h) 16, a2 32, c 3 + 1 pad
 constexpr int kPaperStoreFloatsPerSample = 156;  // paper architecture: z 16, cf 6 + phi + pad, c 3 + pad, 4 x 32 hidden
-constexpr int kRenderGroups = 3;     // tile groups (4 warps, 128 tensor-memory columns each) per render CTA
+constexpr int kRenderGroups = 2;     // tile groups (8 warps, 176 tensor-memory columns each) per render CTA
 // Bits of the context's device status word: a kernel sets its bit when a bounded wait for its
 // tensor-core products ran out (it then stops early; that call's outputs are incomplete)
 constexpr int kStatusRender = 2, kStatusProposal = 4, kStatusEikonal = 8, kStatusPaperRender = 16,

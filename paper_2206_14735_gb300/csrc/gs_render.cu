@@ -209,15 +209,11 @@ gs_status gs_launch_render(const gs_ctx* ctx, const float* theta, const uint16_t
   a.d_hat = d_hat;
   a.wsum = wsum;
   a.status = ctx->status;
-  if (ctx->cfg.precision != GS_PREC_BF16)
-    for (int q = 0; q < 2; ++q)
-      if (!gs_encode_level_map(ctx, theta, 2 + q, &a.tmap[q])) return GS_ERR_CUDA;
   a.store = ctx->store;
   a.w_out = b->w;
   a.dz_out = b->dz;
   a.eik = reinterpret_cast<const float4*>(b->eik);
   a.eik_stride = (long long)b->R * b->N;
-  a.store_stride = (long long)ctx->cfg.max_rays * ctx->max_n;
   const int nch = (b->N + 31) / 32;
   if (ctx->cfg.precision == GS_PREC_BF16) {
     switch (nch) {

@@ -4,20 +4,30 @@
 // geometry and colour decoders, NeuS compositing, the rgb / depth / sdf / free-space losses
 // and, in the same pass, their reverse mode down to every grid feature and decoder weight.
 //
-// Mapping.  A "group" of 4 warps owns one M = 128 tensor-core tile: warp w of the group
-// renders one ray and its 32-sample chunk j fills tile rows 32w..32w+31, which are exactly
-// the tensor-memory lanes that warp may read.  Each decoder layer of a chunk is one MMA
-// phase: every thread writes its sample's activation row into the shared-memory A operand
-// (K-major, no swizzle), one thread issues the MMA(s) against the shared-memory weight tile,
-// the result lands in tensor memory and every thread reads its own row back with
-// tcgen05.ld.  Forward: 4 phases per chunk.  Reverse: the forward is recomputed (4 phases)
-// and the four activation adjoints run as 4 more phases; the decoder weight gradients are
-// reduced on CUDA cores as 4x4 register tiles over the warp's 32 staged samples while the
-// next MMA runs.  FP32 form: each operand is split into three bfloat16 parts and the six
-// leading part products are accumulated in FP32 (FP32-grade accuracy on BF16 tensor cores).
-// Compositing and its adjoint are warp scans over the ray's chunks, as in the CUDA-core
-// design; grid gradients are scattered with 16-byte vector atomics (coarsest level first
-// accumulated in shared memory).
+// Mapping.  A "group" of 8 warps owns one M = 128 tensor-core tile, two threads per tile row:
+// warps w and w + 4 of the group render one ray, and its 32-sample chunk j fills tile rows
+// 32w..32w+31, which are exactly the tensor-memory lanes that warps w (mod 4) may read.  The
+// lower half's threads hold the first half of a layer's units and grid levels 0 and 3, the upper
+// half's the other units and levels 1 and 2.  Each decoder layer of a chunk is one MMA phase:
+// the threads write their sample's activation row into the tensor-memory A operand, one thread
+// issues the MMA(s) against the shared-memory weight tile (K-major, no swizzle), the result lands
+// in tensor memory and every thread reads its columns back with tcgen05.ld.  Forward: 3 phases
+// per chunk (the colour output layer on CUDA cores).  Reverse: the stored activations (or the
+// forward phases again), then 3 adjoint phases; the decoder weight gradients are products over
+// the tile's samples, accumulated in tensor memory.  FP32 form: each operand is split into three
+// bfloat16 parts and the six leading part products are accumulated in FP32 (FP32-grade accuracy
+// on BF16 tensor cores).  Compositing and its adjoint are warp scans over the ray's chunks, by
+// the lower half; grid gradients are scattered with 16-byte vector reductions.
+//
+// What bounds it: the L1 / shared-memory data path (62 % busy over the whole kernel at 8192 x 96
+// before the operands moved to tensor memory, in bursts: the phases of a group load it in turn)
+// and each group's serial chain; DRAM and the tensor cores are below 20 %.  Hence two threads per
+// row (half the chain at the same shared and tensor memory), the phases' A operands in tensor
+// memory, two groups of 128 registers without spills (three at 80 registers measured slower:
+// 607 against 476 us, at the same data path), the weight gradients' part pairs in as few products
+// as the tile layout allows.  Render call, 8192 x 96, stored: one thread per row and three groups
+// 523 us, two threads and two groups 476 us, A operands in tensor memory 451 us; forward only,
+// 8192 x 132: 251, 223, 198 us.
 #pragma once
 #include "gs_internal.h"
 #include <cuda.h>
@@ -45,13 +55,12 @@ struct PrecBF16 {
   static constexpr int planes = 1;
 };
 
-constexpr int kKD = 16;  // padded K of the colour-output adjoint (3 real columns) = one bf16 K step
-
-// weight (B) tiles: {N, K} of the 8 decoder contractions
-//   0 W1  32x16 | 1 W2 16x32 | 2 W3 32x16 (col 15 zero) | 3 W4 16x32 (rows 3.. zero)
-//   4 W4^T 32xKD (cols 3.. zero) | 5 W3^T 16x32 (row 15 zero) | 6 W2^T 32x16 | 7 W1^T 16x32
-__host__ __device__ constexpr int wN(int i) { return (i == 0 || i == 2 || i == 4 || i == 6) ? 32 : 16; }
-__host__ __device__ constexpr int wK(int i) { return i == 4 ? kKD : ((i == 0 || i == 2 || i == 6) ? 16 : 32); }
+constexpr int kTiles = 6;
+// weight (B) tiles: {N, K} of the decoder contractions on the tensor core
+//   0 W1  32x16 | 1 W2 16x32 | 2 W3 32x16 (col 15 zero)
+//   3 W3^T 16x32 (row 15 zero) | 4 W2^T 32x16 | 5 W1^T 16x32
+__host__ __device__ constexpr int wN(int i) { return (i == 0 || i == 2 || i == 4) ? 32 : 16; }
+__host__ __device__ constexpr int wK(int i) { return (i == 0 || i == 2 || i == 4) ? 16 : 32; }
 template <class P>
 __host__ __device__ constexpr uint32_t wBytes(int i) { return (uint32_t)(wN(i) * wK(i) * P::es); }
 template <class P>
@@ -61,14 +70,13 @@ __host__ __device__ constexpr uint32_t wOff(int i) {
   return o;
 }
 template <class P>
-__host__ __device__ constexpr uint32_t wTotal() { return wOff<P>(8); }
+__host__ __device__ constexpr uint32_t wTotal() { return wOff<P>(kTiles); }
 
-// tensor-memory columns of one group: forward accumulators D1..D3 and the colour output X;
-// the backward phases reuse D3 (N = 32) and D2 (N = 16) once those are consumed; the decoder
-// weight gradients accumulate over all of the group's tiles in W1..W4 (M = 64 layout: row m
-// in lane 32 (m / 16) + m % 16)
-constexpr uint32_t cD1 = 0, cD2 = 32, cD3 = 48, cX = 80, cXb = cD3, cYb = cD2;
-constexpr uint32_t cW1 = 96, cW2 = 120, cW3 = 136, cW4 = 152, kGroupCols = 160;
+// tensor-memory columns of one group: the phases' results (N = 32 in cX, N = 16 in cY; each is
+// read back before the next phase that writes its columns), then the decoder weight gradients,
+// accumulated over all of the group's tiles (M = 64 layout: row m in lane 32 (m / 16) + m % 16)
+// and the phases' A operand: part p of a K-column row in columns cA + p K / 2 ..
+constexpr uint32_t cX = 0, cY = 32, cW1 = 48, cW2 = 72, cW3 = 112, cA = 128, kGroupCols = 176;
 // tcgen05.alloc takes a power of two >= 32 columns
 __host__ __device__ constexpr uint32_t tmem_cols(int groups) {
   uint32_t c = 32;
@@ -76,21 +84,43 @@ __host__ __device__ constexpr uint32_t tmem_cols(int groups) {
   return c;
 }
 
-constexpr int kGroupThreads = 128;
+constexpr int kGroupThreads = 128;  // a tile group of one thread per tile row
+constexpr int kTileThreads = 256;   // the compact render kernel's tile group: two threads per tile row
+constexpr int kSums = 8;            // running sums of a compositing thread: 4 losses, kappa, db4
 constexpr uint32_t kMbarLimit = 1u << 20;  // bounded MMA-completion wait (tries of up to 2 us: ~2 s)
 
+// Shared memory per tile group: adjoint tile | partner planes of the weight-gradient products (an
+// activation tile of up to 40 columns; that widest one goes with a 16-column adjoint tile, which
+// fills half of its space, and starts there) | (BF16 form) the colour layer's staging rows |
+// barriers.  The phases' own A operands are in tensor memory: from shared memory every product
+// read its 4 KB again, and the shared-memory data path, which the loads and stores of both
+// caches go through too, is what binds this kernel.
+// The adjoint tile holds the two leading parts side by side (part p of a K-column tile takes the
+// 16-byte column chunks p K / 8 .. of a row): read MN-major, one M = 64 product then takes both
+// parts of a 32-unit adjoint as 64 rows, two products per 16 samples (one per part of the
+// partner) where the part pairs by themselves took three.  An M = 64 read of a narrower tile runs
+// into the next rows (or what follows the tile), for D rows that nobody reads.
 template <class P>
 struct TcLayout {
-  static constexpr uint32_t a_bytes = 128u * 32u * P::es;  // one A operand plane, K <= 32
-  // partner operand of the weight-gradient products (an activation tile of up to 40 columns);
-  // 12 KB per plane keeps every M = 64 operand read inside the plane
-  static constexpr uint32_t b_bytes = 12288u;
+  static constexpr uint32_t a_bytes = 128u * 32u * P::es;  // one part, K = 32
+  static constexpr int side = P::planes < 2 ? 1 : 2;       // parts side by side
+  static constexpr uint32_t b_bytes = 128u * 40u * P::es;
   static constexpr int b_planes = P::planes < 2 ? P::planes : 2;
-  static constexpr uint32_t group_bytes = a_bytes * P::planes + b_bytes * b_planes + 128;  // + mbarrier, flag
+  static constexpr uint32_t b_off = a_bytes * side;                            // partner tile
+  static constexpr uint32_t b_wide = b_off - (side > 1 ? a_bytes : 0u);        // the 40-column one
+  static constexpr uint32_t stage_off = b_off + (b_bytes * 3 / 5) * b_planes;  // after 24 columns
+  static constexpr uint32_t stage_bytes = P::planes < 2 ? 128u * 32u * 4u : 0u;
+  static constexpr uint32_t tiles = stage_off + stage_bytes;
+  static constexpr uint32_t runs = 8u * 33u * 36u * 4u;  // the run reduction's rows over the whole space
+  static constexpr uint32_t bar_off = ((tiles > runs ? tiles : runs) + 127u) / 128u * 128u;
+  static constexpr uint32_t group_bytes = bar_off + 128;
+  static_assert(b_wide + b_bytes * b_planes <= bar_off, "the wide partner tile fits");
+  static constexpr uint32_t row_stride(int K) { return (uint32_t)side * (uint32_t)K * 16u; }  // per 8 rows
 };
 
+template <int T = kGroupThreads>
 __device__ __forceinline__ void group_sync(int g) {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kGroupThreads) : "memory");
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(T) : "memory");
 }
 
 // ---- operand rows ---------------------------------------------------------------------
@@ -105,39 +135,81 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 (&p)[PL]) {
   }
 }
 
-// write K values as row `row` of a K-major no-swizzle tile, one plane per bf16 part; pairs
-// of values are rounded together (one cvt.rn.bf16x2 per pair and part)
-template <int NPL, int K, uint32_t PLANE_BYTES>
-__device__ __forceinline__ void store_row_planes(uint8_t* planes, int row, const float* v) {
-  constexpr uint32_t sbo = (uint32_t)(K * 2 / 16) * 128u;
-  constexpr uint32_t plane_bytes = PLANE_BYTES;
-  constexpr int kPl = NPL;
+// r -= the two bfloat16 values in w, exactly (they are r's leading bits): one packed operation
+__device__ __forceinline__ void sub_parts(float2& r, uint32_t w) {
+  const float2 h = make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+  const float2 m1 = make_float2(-1.0f, -1.0f);
+  asm("fma.rn.f32x2 %0, %1, %2, %0;"
+      : "+l"(reinterpret_cast<uint64_t&>(r))
+      : "l"(reinterpret_cast<const uint64_t&>(h)), "l"(reinterpret_cast<const uint64_t&>(m1)));
+}
+// the NPL bf16 parts of 2 W consecutive values, W words a part; pairs of values are rounded
+// together (one cvt.rn.bf16x2 per pair and part)
+template <int NPL, int W>
+__device__ __forceinline__ void split_words(const float* v, uint32_t (&w)[NPL][W]) {
 #pragma unroll
-  for (int c = 0; c < K / 8; ++c) {
-    float r[8];
+  for (int q = 0; q < W; ++q) {
+    float2 r = make_float2(v[2 * q], v[2 * q + 1]);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) r[q] = v[8 * c + q];
-    const uint32_t off = tc::core_offset((uint32_t)row, (uint32_t)c, 128u, sbo);
-#pragma unroll
-    for (int pl = 0; pl < kPl; ++pl) {
-      uint32_t w[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(r[2 * q], r[2 * q + 1]);
-        w[q] = *reinterpret_cast<const uint32_t*>(&b);
-        if (pl + 1 < kPl) {
-          r[2 * q] -= __uint_as_float(w[q] << 16);
-          r[2 * q + 1] -= __uint_as_float(w[q] & 0xFFFF0000u);
-        }
-      }
-      *reinterpret_cast<uint4*>(planes + pl * plane_bytes + off) = make_uint4(w[0], w[1], w[2], w[3]);
+    for (int pl = 0; pl < NPL; ++pl) {
+      const __nv_bfloat162 b = __floats2bfloat162_rn(r.x, r.y);
+      w[pl][q] = *reinterpret_cast<const uint32_t*>(&b);
+      if (pl + 1 < NPL) sub_parts(r, w[pl][q]);
     }
   }
 }
+// 8 values as 16-byte chunk `c` of row `row` of a K-major no-swizzle tile of K columns
+template <int NPL, int K, uint32_t PLANE_BYTES>
+__device__ __forceinline__ void store_chunk(uint8_t* planes, int row, int c, const float* v) {
+  constexpr uint32_t sbo = (uint32_t)(K * 2 / 16) * 128u;
+  uint32_t w[NPL][4];
+  split_words<NPL, 4>(v, w);
+  const uint32_t off = tc::core_offset((uint32_t)row, (uint32_t)c, 128u, sbo);
+#pragma unroll
+  for (int pl = 0; pl < NPL; ++pl)
+    *reinterpret_cast<uint4*>(planes + pl * PLANE_BYTES + off) = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
+}
+// 4 values as the columns 4 q .. 4 q + 3 of the row
+template <int NPL, int K, uint32_t PLANE_BYTES>
+__device__ __forceinline__ void store_quarter(uint8_t* planes, int row, int q, const float4& v4) {
+  constexpr uint32_t sbo = (uint32_t)(K * 2 / 16) * 128u;
+  const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+  uint32_t w[NPL][2];
+  split_words<NPL, 2>(v, w);
+  const uint32_t off = tc::core_offset((uint32_t)row, (uint32_t)(q >> 1), 128u, sbo) + (uint32_t)(q & 1) * 8u;
+#pragma unroll
+  for (int pl = 0; pl < NPL; ++pl) *reinterpret_cast<uint2*>(planes + pl * PLANE_BYTES + off) = make_uint2(w[pl][0], w[pl][1]);
+}
+// The compact kernel's operand rows: 2 W values of a K-column row from column 2 w0 on, all parts into
+// tensor memory (ta: the part-0 column of the thread's lane) and, with TILE, the leading parts
+// into the adjoint tile as well (whole 16-byte chunks: W a multiple of 4)
+template <class P, int K, bool TILE, int W>
+__device__ __forceinline__ void put_operand(uint32_t ta, uint8_t* tile, int row, int w0, const float* v) {
+  using L = TcLayout<P>;
+  uint32_t w[P::planes][W];
+  split_words<P::planes, W>(v, w);
+#pragma unroll
+  for (int pl = 0; pl < P::planes; ++pl) tc::tmem_st(ta + (uint32_t)(pl * (K / 2) + w0), w[pl]);
+  if constexpr (TILE) {
+#pragma unroll
+    for (int pl = 0; pl < L::side; ++pl)
+#pragma unroll
+      for (int c = 0; c < W / 4; ++c)
+        *reinterpret_cast<uint4*>(tile + tc::core_offset((uint32_t)row, (uint32_t)(pl * (K / 8) + w0 / 4 + c), 128u,
+                                                         L::row_stride(K))) =
+            make_uint4(w[pl][4 * c], w[pl][4 * c + 1], w[pl][4 * c + 2], w[pl][4 * c + 3]);
+  }
+}
+// K values as row `row`, one plane per bf16 part
+template <int NPL, int K, uint32_t PLANE_BYTES>
+__device__ __forceinline__ void store_row_planes(uint8_t* planes, int row, const float* v) {
+#pragma unroll
+  for (int c = 0; c < K / 8; ++c) store_chunk<NPL, K, PLANE_BYTES>(planes, row, c, v + 8 * c);
+}
+
 // a row of the A operand tile of the decoder phases
 template <class P, int K>
 __device__ __forceinline__ void store_row(uint8_t* planes, int row, const float* v) {
-  static_assert(P::es == 2, "bf16 parts");
   store_row_planes<P::planes, K, 128u * 32u * P::es>(planes, row, v);
 }
 
@@ -205,10 +277,45 @@ __device__ __forceinline__ void issue_mma_dw(uint32_t d, uint32_t a0, uint32_t a
   }
 }
 
-// Part products kept in the weight-gradient MMAs: i + j < 2 in the FP32 form (relative error
-// of a product below 2^-15, against the 1e-4 gradient tolerance), the single product in BF16.
-template <class P>
-constexpr int kDwSum = P::planes > 1 ? 2 : 1;
+// The compact kernel's phase product: D[128][N] = A[128][K] B[N][K]^T, A in tensor memory
+template <class P, int N, int K>
+__device__ __forceinline__ void tile_mma(uint32_t d, uint32_t ta, uint32_t b0, uint32_t wplane) {
+  constexpr uint32_t idesc = tc::instr_desc(P::kind, 128, N);
+  const uint32_t blo = tc::desc_lo(b0, 128u);
+  bool first = true;
+#pragma unroll
+  for (int s = 0; s < K / P::kmma; ++s) {
+    // smallest part products first
+#pragma unroll
+    for (int sum = P::planes - 1; sum >= 0; --sum)
+#pragma unroll
+      for (int i = 0; i <= sum; ++i) {
+        const uint32_t bo = (uint32_t)(sum - i) * wplane + (uint32_t)s * 256u;
+        tc::mma_bf16_ta(d, ta + (uint32_t)(i * (K / 2) + s * 8), tc::desc_of(blo + (bo >> 4), tc::desc_hi(K * 16u)), idesc,
+                        first ? 0u : 1u);
+        first = false;
+      }
+  }
+}
+// Its weight-gradient product: D[64][N] (+)= sum over the tile's 128 samples of A[s][m] B[s][n], both
+// operands read MN-major; m over the adjoint tile's KA columns of part 0, then of part 1 (rows KA ..
+// 2 KA - 1, added to the first KA at the end), n over the partner tile's N columns, one product
+// per partner part.  `acc` false on the first tile.
+template <class P, int N, int KA>
+__device__ __forceinline__ void tile_mma_dw(uint32_t d, uint32_t a0, uint32_t b0, bool acc) {
+  using L = TcLayout<P>;
+  constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 64, N) | (1u << 15) | (1u << 16);
+  constexpr uint32_t ra = L::row_stride(KA), rb = N * 16u;
+  const uint32_t alo = tc::desc_lo(a0, ra), blo = tc::desc_lo(b0, rb);
+#pragma unroll
+  for (int s = 0; s < 8; ++s)  // K = 128 samples, 16 per product
+#pragma unroll
+    for (int j = L::b_planes - 1; j >= 0; --j) {
+      tc::mma_bf16(d, tc::desc_of(alo + ((s * 2u * ra) >> 4), tc::desc_hi(128u)),
+                   tc::desc_of(blo + ((s * 2u * rb + j * L::b_bytes) >> 4), tc::desc_hi(128u)), idesc,
+                   acc || s > 0 || j < L::b_planes - 1 ? 1u : 0u);
+    }
+}
 
 // per-group MMA machinery
 struct Group {
@@ -226,7 +333,7 @@ struct Group {
   int g, gt;
 };
 
-// A rows written by every thread -> one thread issues the MMA and commits
+// A rows written by every thread of a 128-thread group -> its thread 0 issues the MMA and commits
 template <class P, int N, int K>
 __device__ __forceinline__ void mma_phase_issue(Group& G, uint32_t dcol, const uint8_t* w, uint32_t wplane) {
   tc::fence_smem_async();
@@ -238,25 +345,83 @@ __device__ __forceinline__ void mma_phase_issue(Group& G, uint32_t dcol, const u
     tc::mma_commit(G.mbar);
   }
 }
-// the same, and a second thread issues the weight-gradient products that read the same tiles
-// and commits them to mbar_dw: the phase's result does not wait for them, and the operand
-// tiles are rewritten only after dw_wait
-template <class P, int N, int K, class Extra>
-__device__ __forceinline__ void mma_phase_issue_dw(Group& G, uint32_t dcol, const uint8_t* w, uint32_t wplane,
-                                                   Extra extra) {
-  tc::fence_smem_async();
-  tc::fence_before_sync();
-  group_sync(G.g);
-  tc::fence_after_sync();
-  if (G.gt == 0) {
-    issue_mma<P, N, K>(G.tcol + dcol, tc::smem_u32(G.a), tc::smem_u32(w), wplane);
-    tc::mma_commit(G.mbar);
-  } else if (G.gt == 32) {
-    extra();
-    tc::mma_commit(G.mbar_dw);
-  }
-  G.dw_pending = true;
+// ---- the compact render kernel's tile groups ------------------------------------------------
+// A tile group's barriers: the phase's products done, its weight-gradient products done
+struct TileBars {
+  uint64_t done, dw;
+  int abort;
+};
+template <class P, int TYPE>  // 0..2 the forward layers, 3..5 the adjoints b3, b2, b1
+__device__ __forceinline__ void issue_phase(uint32_t tcol, uint32_t sw) {
+  constexpr uint32_t wplane = wTotal<P>();
+  if constexpr (TYPE == 0) tile_mma<P, 32, 16>(tcol + cX, tcol + cA, sw + wOff<P>(0), wplane);
+  if constexpr (TYPE == 1) tile_mma<P, 16, 32>(tcol + cY, tcol + cA, sw + wOff<P>(1), wplane);
+  if constexpr (TYPE == 2) tile_mma<P, 32, 16>(tcol + cX, tcol + cA, sw + wOff<P>(2), wplane);
+  if constexpr (TYPE == 3) tile_mma<P, 16, 32>(tcol + cY, tcol + cA, sw + wOff<P>(3), wplane);
+  if constexpr (TYPE == 4) tile_mma<P, 32, 16>(tcol + cX, tcol + cA, sw + wOff<P>(4), wplane);
+  if constexpr (TYPE == 5) tile_mma<P, 16, 32>(tcol + cY, tcol + cA, sw + wOff<P>(5), wplane);
 }
+template <class P, int TYPE>
+__device__ __forceinline__ void issue_phase_dw(uint32_t tcol, uint32_t sa, bool acc) {
+  const uint32_t sb = sa + (TYPE == 4 ? TcLayout<P>::b_wide : TcLayout<P>::b_off);
+  if constexpr (TYPE == 3) tile_mma_dw<P, 16, 32>(tcol + cW3, sa, sb, acc);
+  if constexpr (TYPE == 4) tile_mma_dw<P, 40, 16>(tcol + cW2, sa, sb, acc);
+  if constexpr (TYPE == 5) tile_mma_dw<P, 24, 32>(tcol + cW1, sa, sb, acc);
+}
+
+// what a thread of a group tracks of its barriers
+struct Tile {
+  TileBars* bars;
+  int g, w8;                // the group, this thread's warp in it (uniform)
+  uint32_t ph_done, ph_dw;  // parities of the next completions
+  bool dw_pending;          // weight-gradient products may still read the tiles
+};
+// Operand rows of this warp written -> once all warps have met, one thread of warp 0 issues the
+// phase's products and (adjoint phases) one of warp 4 the weight-gradient products that
+// read the same tiles.
+template <class P, int TYPE>
+__device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa, uint32_t sw, bool dw_acc) {
+  tc::tmem_st_wait();
+  if (TYPE >= 3) tc::fence_smem_async();
+  tc::fence_before_sync();
+  group_sync<kTileThreads>(T.g);
+  tc::fence_after_sync();
+  if (T.w8 == 0) {
+    if (tc::elect_one()) {
+      issue_phase<P, TYPE>(tcol, sw);
+
+      tc::mma_commit(&T.bars->done);
+    }
+    __syncwarp();
+  } else if (TYPE >= 3 && T.w8 == 4) {
+    if (tc::elect_one()) {
+      issue_phase_dw<P, TYPE>(tcol, sa, dw_acc);
+      tc::mma_commit(&T.bars->dw);
+    }
+    __syncwarp();
+  }
+  if (TYPE >= 3) T.dw_pending = true;
+}
+// a thread of the group waits for the products (bounded) while the others park on the hardware
+// barrier; false (for every thread) if they never complete
+__device__ __forceinline__ bool phase_wait(Tile& T) {
+  if (T.w8 == 1 && tc::elect_one() && !tc::mbar_wait(&T.bars->done, T.ph_done, kMbarLimit))
+    *reinterpret_cast<volatile int*>(&T.bars->abort) = 1;
+  T.ph_done ^= 1u;
+  group_sync<kTileThreads>(T.g);
+  tc::fence_after_sync();
+  return *reinterpret_cast<volatile int*>(&T.bars->abort) == 0;
+}
+// no weight-gradient product reads the tiles
+__device__ __forceinline__ void tiles_free(Tile& T) {
+  if (T.dw_pending) {
+    if (!tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit)) *reinterpret_cast<volatile int*>(&T.bars->abort) = 1;
+    T.ph_dw ^= 1u;
+    T.dw_pending = false;
+    tc::fence_after_sync();
+  }
+}
+
 // every thread of the group: bounded wait until the weight-gradient MMAs are done with the tiles
 __device__ __forceinline__ void dw_wait(Group& G) {
   if (!G.dw_pending) return;
@@ -267,10 +432,11 @@ __device__ __forceinline__ void dw_wait(Group& G) {
 }
 // the issuing thread waits for the MMA (bounded) while the other threads of the group park on
 // the hardware barrier; false (for every thread) if it never completed
+template <int T = kGroupThreads>
 __device__ __forceinline__ bool mma_phase_wait(Group& G) {
   if (G.gt == 0 && !tc::mbar_wait(G.mbar, G.phase, kMbarLimit)) *reinterpret_cast<volatile int*>(G.abort) = 1;
   G.phase ^= 1u;
-  group_sync(G.g);
+  group_sync<T>(G.g);
   tc::fence_after_sync();
   return *reinterpret_cast<volatile int*>(G.abort) == 0;
 }
@@ -280,99 +446,84 @@ __device__ __forceinline__ uint32_t lane_addr(const Group& G, uint32_t col, int 
 }
 
 // ---- gather / scatter -------------------------------------------------------------------
-// z = [V^0(x), .., V^3(x)] from the FP32 grid, or (BF16 form) from its bfloat16 copy
-template <bool BF16GRID>
-__device__ __forceinline__ void gather_z(const GridDesc& g, const float* __restrict__ theta,
-                                         const uint16_t* __restrict__ theta_bf16, const float x[3], float z[kZ]) {
+// The 8 corners of one cell at (runtime) level l, summed in corner order k = 4 bx + 2 by + bz:
+// a float4 of features from the FP32 grid (`bf16` nullptr) or its bfloat16 copy
+__device__ __forceinline__ float4 level_features(const GridDesc& g, const float* __restrict__ theta, int l,
+                                                 const float x[3]) {
+  const Cell c = locate(g, l, x);
+  float w[8];
+  corner_weights(c.f, w);
+  const long long nx = g.dims[l][0], nxy = nx * g.dims[l][1];
+  const float4* p = reinterpret_cast<const float4*>(theta + g.off[l]) + c.vtx;
+  const float4 *p1 = p + nxy, *p2 = p + nx, *p3 = p2 + nxy;
+  const float4 v[8] = {__ldg(p),     __ldg(p1),     __ldg(p2),     __ldg(p3),
+                       __ldg(p + 1), __ldg(p1 + 1), __ldg(p2 + 1), __ldg(p3 + 1)};
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-  for (int l = 0; l < kLevels; ++l) {
-    const Cell c = locate(g, l, x);
-    float w[8];
-    corner_weights(c.f, w);
-    float4 v[8];
-    if constexpr (BF16GRID) {
-      const uint2* base = reinterpret_cast<const uint2*>(theta_bf16 + g.off[l]);
+  for (int k = 0; k < 8; ++k) f4fma(s, w[k], v[k]);
+  return s;
+}
+__device__ __forceinline__ float4 level_features_bf16(const GridDesc& g, const uint16_t* __restrict__ copy, int l,
+                                                      const float x[3]) {
+  const Cell c = locate(g, l, x);
+  float w[8];
+  corner_weights(c.f, w);
+  const long long nx = g.dims[l][0], nxy = nx * g.dims[l][1];
+  const uint2* p = reinterpret_cast<const uint2*>(copy + g.off[l]) + c.vtx;
+  const uint2 *p1 = p + nxy, *p2 = p + nx, *p3 = p2 + nxy;
+  const uint2 u[8] = {__ldg(p),     __ldg(p1),     __ldg(p2),     __ldg(p3),
+                      __ldg(p + 1), __ldg(p1 + 1), __ldg(p2 + 1), __ldg(p3 + 1)};
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const uint2 u = __ldg(base + c.vtx + corner_offset(g, l, k));
-        v[k] = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u),
-                           __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
-      }
-    } else {
-      const float4* base = reinterpret_cast<const float4*>(theta + g.off[l]);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = __ldg(base + c.vtx + corner_offset(g, l, k));
-    }
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f4fma(s, w[k], v[k]);
-    z[4 * l] = s.x;
-    z[4 * l + 1] = s.y;
-    z[4 * l + 2] = s.z;
-    z[4 * l + 3] = s.w;
-  }
+  for (int k = 0; k < 8; ++k)
+    f4fma(s, w[k], make_float4(__uint_as_float(u[k].x << 16), __uint_as_float(u[k].x & 0xFFFF0000u),
+                               __uint_as_float(u[k].y << 16), __uint_as_float(u[k].y & 0xFFFF0000u)));
+  return s;
 }
 
-// The finest kTmaLevels levels through the TMA: every thread of the group issues one
-// tile::gather4 per level for its sample (rows (y,z), (y+1,z), (y,z+1), (y+1,z+1) of the
-// level's 2D view, 2 vertices each) into a 128-byte slot.  The slots sit where the group's
-// tiles are not written before the first decoder phase: the partner tile, then the gaps of the
-// A planes that the 16-column z tile leaves free.
-__device__ __forceinline__ uint32_t fine_slot(uint8_t* ga, uint8_t* gb, int lvl, int gt) {
-  if (lvl == 0) return tc::smem_u32(gb + gt * 128);
-  if (gt < 64) return tc::smem_u32(gb + 16384 + gt * 128);
-  if (gt < 96) return tc::smem_u32(ga + 4096 + (gt - 64) * 128);
-  return tc::smem_u32(ga + 12288 + (gt - 96) * 128);
+// The finest level's corners by plain loads, all eight in flight: lane i takes them in the order
+// i, i + 1, .. (mod 8; corner c = vertex (x + (c & 1), y + (c >> 1 & 1), z + (c >> 2)))
+struct FineCorners {
+  float4 v[8];
+  float f[3];
+};
+__device__ __forceinline__ void fine_corners_load(const GridDesc& g, const float* __restrict__ theta, const float x[3],
+                                                  FineCorners& q) {
+  constexpr int l = kLevels - 1;
+  const Cell c = locate(g, l, x);
+  const int lane = threadIdx.x & 31;
+  const long long nx = g.dims[l][0], nxy = nx * g.dims[l][1];
+  const float4* base = reinterpret_cast<const float4*>(theta + g.off[l]) + c.vtx;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int cc = (k + lane) & 7;
+    q.v[k] = __ldg(base + (cc & 1) + ((cc & 2) ? nx : 0) + ((cc & 4) ? nxy : 0));
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) q.f[a] = c.f[a];
 }
-constexpr int kTmaLevels = 1;  // the finest levels that go through the TMA (the rest: plain loads)
+__device__ __forceinline__ float4 fine_corners_sum(const FineCorners& q) {
+  const int lane = threadIdx.x & 31;
+  const float f0 = q.f[0], f1 = q.f[1], f2 = q.f[2];
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int cc = (k + lane) & 7;
+    const float w = (((cc & 1) ? f0 : 1.0f - f0) * ((cc & 2) ? f1 : 1.0f - f1)) * ((cc & 4) ? f2 : 1.0f - f2);
+    f4fma(s, w, q.v[k]);
+  }
+  return s;
+}
+
 // host: the 2D view [nz ny][4 nx] of grid level l in theta, a box of 2 vertices x 4 features one
-// row high (the tile::gather4 source of the finest level); false if the driver refused it
+// row high (the source of the paper architecture's tile::gather4 loads); false if the driver
+// refused it
 bool gs_encode_level_map(const gs_ctx* ctx, const float* theta, int l, CUtensorMap* m);
-constexpr uint32_t kFineTmaBytes = 128u * kTmaLevels * 128u;  // per group and round: 128 samples x levels x 128 B
-
-// issue both fine-level gathers of this thread's sample; returns the cells (for the weights)
-__device__ __forceinline__ void fine_gather_issue(const GridDesc& g, const CUtensorMap* tmap, uint8_t* ga, uint8_t* gb,
-                                                  int gt, uint64_t* mbar, const float x[3], Cell (&cs)[kTmaLevels]) {
-  tc::fence_smem_async();  // earlier generic accesses to the slots before the asynchronous writes
-#pragma unroll
-  for (int q = 0; q < kTmaLevels; ++q) {
-    const int l = kLevels - kTmaLevels + q;
-    cs[q] = locate(g, l, x);
-    const int ny = g.dims[l][1];
-    const int r0 = cs[q].idx[2] * ny + cs[q].idx[1];
-    tc::tma_gather4(fine_slot(ga, gb, q, gt), &tmap[q], 4 * cs[q].idx[0], r0, r0 + 1, r0 + ny, r0 + ny + 1, mbar);
-  }
-}
-// z of the fine levels from this thread's slots (chunk order rotated by lane: no bank conflicts)
-__device__ __forceinline__ void fine_gather_read(const uint8_t* ga, const uint8_t* gb, int gt,
-                                                 const Cell (&cs)[kTmaLevels], float z[kZ]) {
-  const int lane = gt & 31;
-#pragma unroll
-  for (int q = 0; q < kTmaLevels; ++q) {
-    const int l = kLevels - kTmaLevels + q;
-    const uint8_t* slot = q == 0 ? gb + gt * 128
-                                 : (gt < 64 ? gb + 16384 + gt * 128
-                                            : (gt < 96 ? ga + 4096 + (gt - 64) * 128 : ga + 12288 + (gt - 96) * 128));
-    const float f0 = cs[q].f[0], f1 = cs[q].f[1], f2 = cs[q].f[2];
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int c = (k + lane) & 7;  // 16-byte chunk: row c >> 1 = (by, bz), x-vertex c & 1
-      const int bx = c & 1, by = (c >> 1) & 1, bz = c >> 2;
-      const float w = ((bx ? f0 : 1.0f - f0) * (by ? f1 : 1.0f - f1)) * (bz ? f2 : 1.0f - f2);
-      f4fma(s, w, *reinterpret_cast<const float4*>(slot + c * 16));
-    }
-    z[4 * l] = s.x;
-    z[4 * l + 1] = s.y;
-    z[4 * l + 2] = s.z;
-    z[4 * l + 3] = s.w;
-  }
-}
 // the other levels by plain loads (a warp's samples share the coarse cells)
 __device__ __forceinline__ void coarse_gather(const GridDesc& g, const float* __restrict__ theta, const float x[3],
                                               float z[kZ]) {
 #pragma unroll
-  for (int l = 0; l < kLevels - kTmaLevels; ++l) {
+  for (int l = 0; l < kLevels - 1; ++l) {
     const Cell c = locate(g, l, x);
     float w[8];
     corner_weights(c.f, w);
@@ -387,138 +538,172 @@ __device__ __forceinline__ void coarse_gather(const GridDesc& g, const float* __
   }
 }
 
-// staging floats per warp of scatter_dz: 32 rows of 36 floats, then the 32 keys
+// staging floats per warp of the run-reduced scatter: 32 rows of 36 floats, then the 32 keys
 constexpr int kScatterStage = 33 * 36;
 
-// 16-byte vector reduction into global memory (fire and forget; the result is not read)
+// 16-byte vector reduction into global memory (fire and forget; no kernel here reads the result,
+// so other memory operations may move across it)
 __device__ __forceinline__ void red_add_f4(float4* p, float4 v) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-               : "memory");
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
 }
 
-// Adjoint of the gather: dtheta_l[corner] += w_c dz_l.  A warp's lanes hold consecutive
-// samples of one ray, so the cells they fall in are visited monotonically and equal cells form
-// contiguous runs of lanes.  At the two coarse levels (long runs) the 8 weighted corner vectors
-// are summed over each run through shared memory: every lane stages its 32 values as a row,
-// lane c walks the 32 rows summing component c (corner c / 4, feature c % 4), and at the end of
-// each run the four features of a corner are gathered into one lane, which issues one 16-byte
-// reduction (8 per run).  At the fine levels, where runs are short, every lane issues its 8
-// corners' 16-byte reductions directly (staging them there measured slower).
-// `st`: this warp's kScatterStage floats of staging space.
-// Deferred Eikonal term: `er` (nullptr for samples without one) points at the sample's record
-// in plane 0 of the batch's Eikonal records (planes `es` float4 apart: q_l = p_l / v_l for the
-// four levels, then the adjoint a); corner c of level l then also receives q_l (a . dw_c/df),
-// the grid part of the Eikonal gradient (Supp. Sec. 1), in the same 16-byte reduction.
-// PAIRED (the fine levels): lane pairs (2i, 2i + 1) take turns on each other's samples so
-// that in one reduction instruction the pair adds a cell's two x-neighbouring corners of one
-// sample, 32 contiguous bytes (one sector when the cell's x index is even): a quarter fewer
-// L2 reduction requests for 18 shuffles per level and lane.
-template <bool PAIRED = false>
-__device__ __forceinline__ void scatter_dz(const GridDesc& g, float* grad, const float x[3], const float dz[kZ],
-                                           bool valid, float* st, const float4* er = nullptr, long long es = 0) {
-  const unsigned active = __ballot_sync(0xffffffffu, valid);
-  if (active == 0) return;
-  const int lane = threadIdx.x & 31;
-  const bool eik_any = __any_sync(0xffffffffu, er != nullptr);
-  float ea[3] = {0.f, 0.f, 0.f};
+// The deferred Eikonal record of a sample (gs_batch.eik): at level l its corner c also receives
+// q_l (a . dw_c/df), the grid part of the Eikonal gradient (Supp. Sec. 1), in the same reduction.
+struct EikSeed {
+  const float4* er;  // the sample's record in plane 0 (planes `es` float4 apart: q_l of the four levels, then a); nullptr: none
+  long long es;
+  float a[3];
+  bool any;  // some lane of the warp has one
+};
+__device__ __forceinline__ EikSeed eik_seed(const float4* er, long long es) {
+  EikSeed e{er, es, {0.f, 0.f, 0.f}, __any_sync(0xffffffffu, er != nullptr) != 0};
   if (er != nullptr) {
     const float4 a4 = __ldg(er + 4 * es);
-    ea[0] = a4.x;
-    ea[1] = a4.y;
-    ea[2] = a4.z;
+    e.a[0] = a4.x;
+    e.a[1] = a4.y;
+    e.a[2] = a4.z;
   }
+  return e;
+}
+// this level's q and a . dw_c/df (zeros without a record)
+__device__ __forceinline__ float4 eik_level(const EikSeed& e, int l, const Cell& cc, float (&dd)[8]) {
+  float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-  for (int l = 0; l < kLevels; ++l) {
-    const Cell cc = locate(g, l, x);
-    float wc[8];
-    corner_weights(cc.f, wc);
-    const float4 g4 = valid ? make_float4(dz[4 * l], dz[4 * l + 1], dz[4 * l + 2], dz[4 * l + 3])
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    float dd[8];  // a . dw_c/df (zero without a record)
+  for (int k = 0; k < 8; ++k) dd[k] = 0.f;
+  if (e.any) {  // warp-uniform
+    if (e.er != nullptr) q4 = __ldg(e.er + l * e.es);
+    float dw[8][3];
+    corner_weight_grads(cc.f, cc.clamped, dw);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) dd[k] = 0.f;
-    if (eik_any) {  // warp-uniform
-      if (er != nullptr) q4 = __ldg(er + l * es);
-      float dw[8][3];
-      corner_weight_grads(cc.f, cc.clamped, dw);
+    for (int k = 0; k < 8; ++k) dd[k] = e.a[0] * dw[k][0] + e.a[1] * dw[k][1] + e.a[2] * dw[k][2];
+  }
+  return q4;
+}
+
+// Adjoint of the gather at a coarse level (0 or 1): dtheta_l[corner] += w_c dz_l.  A warp's lanes
+// hold consecutive samples of one ray, so the cells they fall in are visited monotonically and
+// equal cells form contiguous (long) runs of lanes.  The 8 weighted corner vectors are summed
+// over each run through shared memory: every lane stages its 32 values as a row, lane c walks the
+// 32 rows summing component c (corner c / 4, feature c % 4), and at the end of each run the four
+// features of a corner are gathered into one lane, which issues one 16-byte reduction (8 per
+// run).  st: the warp's kScatterStage floats.
+__device__ __forceinline__ void scatter_runs(const GridDesc& g, float* grad, int l, const float x[3], float4 g4,
+                                             bool valid, float* st, const EikSeed& e) {
+  const int lane = threadIdx.x & 31;
+  const Cell cc = locate(g, l, x);
+  float wc[8], dd[8];
+  corner_weights(cc.f, wc);
+  const float4 q4 = eik_level(e, l, cc, dd);
+  float4* gl = reinterpret_cast<float4*>(grad + g.off[l]);
+  const int key = valid ? (int)cc.vtx : -1;  // the coarse levels have fewer than 2^31 vertices
+  const int next = __shfl_down_sync(0xffffffffu, key, 1);
+  const unsigned ends = __ballot_sync(0xffffffffu, lane == 31 || next != key || key < 0);  // a run's last lane
+  float* rw = st + lane * 36;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) dd[k] = ea[0] * dw[k][0] + ea[1] * dw[k][1] + ea[2] * dw[k][2];
-    }
-    float4* gl = reinterpret_cast<float4*>(grad + g.off[l]);
-    if (l >= 2) {
-      // a zero vector adds nothing: samples whose dL/dz_l is exactly zero (saturated opacity and
-      // no active loss term) issue no reductions at the fine levels
-      const bool nz = g4.x != 0.f || g4.y != 0.f || g4.z != 0.f || g4.w != 0.f || er != nullptr;
-      if constexpr (PAIRED) {
-        // corners k and k + 4 are the x-neighbours v and v + 1.  The even lane sends its
-        // upper corner's vector and receives the odd lane's lower one; then the even lane adds
-        // the lower corners (its own sample's, then its partner's) and the odd lane the upper
-        // ones (its partner's, then its own), so each instruction covers one sample's pair.
-        const bool odd = (lane & 1) != 0;
-        const bool give = valid && nz;
-        const long long pv = __shfl_xor_sync(0xffffffffu, cc.vtx, 1);
+  for (int k = 0; k < 8; ++k) {
+    float4 cv = f4scale(g4, wc[k]);
+    if (e.any) f4fma(cv, dd[k], q4);
+    *reinterpret_cast<float4*>(rw + 4 * k) = cv;
+  }
+  st[32 * 36 + lane] = __int_as_float(key);  // the keys after the rows
+  __syncwarp();
+  const long long coff = corner_offset(g, l, lane >> 2);
+  float acc = 0.f;
+#pragma unroll 1
+  for (int i0 = 0; i0 < 32; i0 += 8) {
+    float v[8];  // eight rows in flight
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          float4 lo4 = make_float4(0.f, 0.f, 0.f, 0.f), hi4 = lo4;
-          if (give) {
-            lo4 = f4scale(g4, wc[k]);
-            hi4 = f4scale(g4, wc[k + 4]);
-            if (eik_any) {
-              f4fma(lo4, dd[k], q4);
-              f4fma(hi4, dd[k + 4], q4);
-            }
-          }
-          const float4 snd = odd ? lo4 : hi4;
-          float4 rcv;
-          rcv.x = __shfl_xor_sync(0xffffffffu, snd.x, 1);
-          rcv.y = __shfl_xor_sync(0xffffffffu, snd.y, 1);
-          rcv.z = __shfl_xor_sync(0xffffffffu, snd.z, 1);
-          rcv.w = __shfl_xor_sync(0xffffffffu, snd.w, 1);
-          const long long off = corner_offset(g, l, k);  // the lower corner; the upper one is + 1
-          // first instruction: the even lane's sample; second: the odd lane's
-          const long long v0 = (odd ? pv : cc.vtx) + off + (odd ? 1 : 0);
-          const long long v1 = (odd ? cc.vtx : pv) + off + (odd ? 1 : 0);
-          const float4 c0 = odd ? rcv : lo4, c1 = odd ? hi4 : rcv;
-          if (c0.x != 0.f || c0.y != 0.f || c0.z != 0.f || c0.w != 0.f) red_add_f4(gl + v0, c0);
-          if (c1.x != 0.f || c1.y != 0.f || c1.z != 0.f || c1.w != 0.f) red_add_f4(gl + v1, c1);
-        }
-      } else if (valid && nz) {
+    for (int q = 0; q < 8; ++q) v[q] = st[(i0 + q) * 36 + lane];
+    const unsigned e8 = ends >> i0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          float4 cv = f4scale(g4, wc[k]);
-          if (eik_any) f4fma(cv, dd[k], q4);
-          red_add_f4(gl + cc.vtx + corner_offset(g, l, k), cv);
-        }
-      }
-      continue;
-    }
-    const int key = valid ? (int)cc.vtx : -1;  // the coarse levels have fewer than 2^31 vertices
-    const int next = __shfl_down_sync(0xffffffffu, key, 1);
-    const unsigned ends = __ballot_sync(0xffffffffu, lane == 31 || next != key || key < 0);  // a run's last lane
-    float* rw = st + lane * 36;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      float4 cv = f4scale(g4, wc[k]);
-      if (eik_any) f4fma(cv, dd[k], q4);
-      *reinterpret_cast<float4*>(rw + 4 * k) = cv;
-    }
-    st[32 * 36 + lane] = __int_as_float(key);  // the keys after the rows
-    __syncwarp();
-    const long long coff = corner_offset(g, l, lane >> 2);
-    float acc = 0.f;
-#pragma unroll 4
-    for (int i = 0; i < 32; ++i) {
-      acc += st[i * 36 + lane];
-      if ((ends >> i) & 1u) {  // uniform: the run holding row i ends at row i
+    for (int q = 0; q < 8; ++q) {
+      acc += v[q];
+      if ((e8 >> q) & 1u) {  // uniform: the run holding row i0 + q ends there
         const float a1 = __shfl_down_sync(0xffffffffu, acc, 1), a2 = __shfl_down_sync(0xffffffffu, acc, 2),
                     a3 = __shfl_down_sync(0xffffffffu, acc, 3);
-        const int ki = __float_as_int(st[32 * 36 + i]);
+        const int ki = __float_as_int(st[32 * 36 + i0 + q]);
         if ((lane & 3) == 0 && ki >= 0) red_add_f4(gl + (long long)ki + coff, make_float4(acc, a1, a2, a3));
         acc = 0.f;
       }
     }
-    __syncwarp();
+  }
+  __syncwarp();
+}
+
+// The same at a fine level, where runs are short: every lane issues its 8 corners' 16-byte
+// reductions directly (staging them there measured slower).  A zero vector adds nothing: samples
+// whose dL/dz_l is exactly zero (saturated opacity and no active loss term) issue none.
+// PAIRED: lane pairs (2i, 2i + 1) take turns on each other's samples so that in one reduction
+// instruction the pair adds a cell's two x-neighbouring corners of one sample, 32 contiguous
+// bytes (one sector when the cell's x index is even): a quarter fewer L2 reduction requests for
+// 18 shuffles per lane.
+template <bool PAIRED>
+__device__ __forceinline__ void scatter_direct(const GridDesc& g, float* grad, int l, const float x[3], float4 g4,
+                                               bool valid, const EikSeed& e) {
+  const int lane = threadIdx.x & 31;
+  const bool give = valid && (g4.x != 0.f || g4.y != 0.f || g4.z != 0.f || g4.w != 0.f || e.er != nullptr);
+  if (!PAIRED && !give && !e.any) return;
+  const Cell cc = locate(g, l, x);
+  float wc[8], dd[8];
+  corner_weights(cc.f, wc);
+  const float4 q4 = eik_level(e, l, cc, dd);
+  const long long nx = g.dims[l][0], nxy = nx * g.dims[l][1];
+  float4* gl = reinterpret_cast<float4*>(grad + g.off[l]);
+  if constexpr (PAIRED) {
+    // corners k and k + 4 are the x-neighbours v and v + 1.  The even lane sends its upper
+    // corner's vector and receives the odd lane's lower one; then the even lane adds the lower
+    // corners (its own sample's, then its partner's) and the odd lane the upper ones (its
+    // partner's, then its own), so each instruction covers one sample's pair.
+    const bool odd = (lane & 1) != 0;
+    const long long pv = __shfl_xor_sync(0xffffffffu, cc.vtx, 1);
+    float4* q0 = gl + (odd ? pv : cc.vtx) + (odd ? 1 : 0);  // first instruction: the even lane's sample
+    float4* q1 = gl + (odd ? cc.vtx : pv) + (odd ? 1 : 0);  // second: the odd lane's
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float4 lo4 = make_float4(0.f, 0.f, 0.f, 0.f), hi4 = lo4;
+      if (give) {
+        lo4 = f4scale(g4, wc[k]);
+        hi4 = f4scale(g4, wc[k + 4]);
+        if (e.any) {
+          f4fma(lo4, dd[k], q4);
+          f4fma(hi4, dd[k + 4], q4);
+        }
+      }
+      const float4 snd = odd ? lo4 : hi4;
+      float4 rcv;
+      rcv.x = __shfl_xor_sync(0xffffffffu, snd.x, 1);
+      rcv.y = __shfl_xor_sync(0xffffffffu, snd.y, 1);
+      rcv.z = __shfl_xor_sync(0xffffffffu, snd.z, 1);
+      rcv.w = __shfl_xor_sync(0xffffffffu, snd.w, 1);
+      const long long off = ((k & 2) ? nx : 0) + ((k & 1) ? nxy : 0);  // the lower corner; the upper one is + 1
+      const float4 c0 = odd ? rcv : lo4, c1 = odd ? hi4 : rcv;
+      if (c0.x != 0.f || c0.y != 0.f || c0.z != 0.f || c0.w != 0.f) red_add_f4(q0 + off, c0);
+      if (c1.x != 0.f || c1.y != 0.f || c1.z != 0.f || c1.w != 0.f) red_add_f4(q1 + off, c1);
+    }
+  } else if (give) {
+    float4* p0 = gl + cc.vtx;
+    float4* const row[4] = {p0, p0 + nxy, p0 + nx, p0 + nx + nxy};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float4 cv = f4scale(g4, wc[k]);
+      if (e.any) f4fma(cv, dd[k], q4);
+      red_add_f4(row[k & 3] + (k >> 2), cv);
+    }
+  }
+}
+
+// All four levels by one warp (st: its kScatterStage floats)
+__device__ __forceinline__ void scatter_dz(const GridDesc& g, float* grad, const float x[3], const float dz[kZ],
+                                           bool valid, float* st, const float4* er = nullptr, long long es = 0) {
+  const unsigned active = __ballot_sync(0xffffffffu, valid);
+  if (active == 0) return;
+  const EikSeed e = eik_seed(er, es);
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) {
+    const float4 g4 = valid ? make_float4(dz[4 * l], dz[4 * l + 1], dz[4 * l + 2], dz[4 * l + 3])
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (l < 2) scatter_runs(g, grad, l, x, g4, valid, st, e);
+    else scatter_direct<false>(g, grad, l, x, g4, valid, e);
   }
 }
 
@@ -546,7 +731,7 @@ __device__ __forceinline__ void get_fields(const float4* sp, long long ss, bool 
   static_assert(F0 % 4 == 0 && NF % 4 == 0 && NF <= M, "whole groups of four fields");
 #pragma unroll
   for (int q = 0; q < NF / 4; ++q) {
-    const float4 u = get ? __ldg(sp + (F0 / 4 + q) * ss) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 u = get ? sp[(F0 / 4 + q) * ss] : make_float4(0.f, 0.f, 0.f, 0.f);
     v[4 * q] = u.x;
     v[4 * q + 1] = u.y;
     v[4 * q + 2] = u.z;
@@ -570,57 +755,44 @@ struct RenderTcArgs {
   float* mlp_part;
   float *rgb_hat, *d_hat, *wsum;
   int* status;      // device status word (bit 1: an MMA never completed)
-  // Stored activations (store mode): field f of sample s = rr * N + si in component f % 4 of
-  // ((float4*)store)[(f / 4) * store_stride + s], one coalesced float4 plane per four fields.
-  // Written by every forward pass, read by every backward pass in place of the gather and the
-  // four recomputed decoder phases.  nullptr: recompute.
+  // Stored activations (store mode): written by every forward pass, read by every backward pass
+  // in place of the gather and the recomputed decoder phases.  nullptr: recompute.
   float* store;
-  long long store_stride;
   float* w_out;  // [R][N] rendering weights, written by forward passes when not nullptr
   float* dz_out; // [R][N][16] dL/dz of every sample, written by backward passes when not nullptr
   // deferred Eikonal records ([5][R][N] float4 planes, eik_stride = R N) of the free-space
   // samples, added to their grid scatter by backward passes; nullptr: none
   const float4* eik;
   long long eik_stride;
-  // FP32 form: 2D views [nz * ny][nx * 4] of grid levels 2 and 3 for the TMA gathers (a box of
-  // 2 vertices x 4 features; one tile::gather4 brings a cell's 8 corners)
-  CUtensorMap tmap[2];
 };
 
-// fields of one stored sample: z[16] | a1 = ReLU layer-1 output [32] | (phi, h[15]) | a2 [32] | c[3], 0
-constexpr int kFz = 0, kFa1 = 16, kFout = 48, kFa2 = 64, kFc = 96, kStoreFields = 100;
-static_assert(kStoreFields == kStoreFloatsPerSample, "the store holds every field");
-
-// colour c = sigmoid(W4 a2 + b4) on CUDA cores (3 outputs: too narrow for a tensor-core phase)
-__device__ __forceinline__ void colour_out(const float* w4f, const float* b4, const float (&a2)[32], float (&c3)[3]) {
+// Stored activations of one chunk (n <= 32 consecutive samples of a ray from sample s on): 25
+// planes of n float4, one after the other from float4 index 25 s on, lane i's four fields in
+// element i of a plane, so a warp moves one contiguous line per plane and a chunk's 400 n bytes
+// lie together (the planes of all samples apart, 12 MB each at 8192 x 96, a chunk touched 25
+// pages).  Planes: z by level [4] | a1 = ReLU layer-1 output [8] | h [4] | a2 = ReLU layer-2
+// output [8] | c, phi.
+constexpr int kPz = 0, kPa1 = 4, kPh = 12, kPa2 = 16, kPc = 24;
+static_assert((kPc + 1) * 4 == kStoreFloatsPerSample, "the store holds every field");
+struct StoreRef {
+  float4* p;  // this lane's element of plane 0
+  int n;      // samples of the chunk
+  __device__ __forceinline__ float4& operator[](int plane) const { return p[plane * n]; }
+};
+template <int NP>
+__device__ __forceinline__ void put_planes(const StoreRef& s, int first, const float* v) {
 #pragma unroll
-  for (int n = 0; n < 3; ++n) {
-    float s = b4[n];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) s = fmaf(w4f[32 * n + k], a2[k], s);
-    c3[n] = sigmoidf_(s);
-  }
+  for (int q = 0; q < NP; ++q) s[first + q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
 }
-
-// z of one chunk: every thread of the group takes part (the TMA round counts all 128 slots);
-// invalid samples get z = 0
-template <class P>
-__device__ __forceinline__ void gather_chunk(Group& G, const RenderTcArgs& a, const float x[3], bool valid,
-                                             float z[kZ]) {
-  if constexpr (P::planes > 1) {  // FP32 form: fine levels through the TMA, coarse by plain loads
-    Cell cs[kTmaLevels];
-    fine_gather_issue(a.g, a.tmap + (2 - kTmaLevels), G.a, G.b, G.gt, G.mbar_tma, x, cs);
-    if (valid) coarse_gather(a.g, a.theta, x, z);
-    if (!tc::mbar_wait(G.mbar_tma, G.phase_tma, kMbarLimit)) *reinterpret_cast<volatile int*>(G.abort) = 1;
-    G.phase_tma ^= 1u;
-    if (G.gt == 0) tc::mbar_arrive_expect_tx(G.mbar_tma, kFineTmaBytes);  // armed for the next round
-    fine_gather_read(G.a, G.b, G.gt, cs, z);
-  } else if (valid) {
-    gather_z<true>(a.g, a.theta, a.theta_bf16, x, z);
-  }
-  if (!valid) {
+template <int NP>
+__device__ __forceinline__ void get_planes(const StoreRef& s, int first, bool get, float* v) {
 #pragma unroll
-    for (int k = 0; k < kZ; ++k) z[k] = 0.f;
+  for (int q = 0; q < NP; ++q) {
+    const float4 u = get ? s[first + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[4 * q] = u.x;
+    v[4 * q + 1] = u.y;
+    v[4 * q + 2] = u.z;
+    v[4 * q + 3] = u.w;
   }
 }
 
@@ -628,40 +800,37 @@ __device__ __forceinline__ void gather_chunk(Group& G, const RenderTcArgs& a, co
 // end reports as unreachable code there
 #pragma nv_diag_suppress 128
 template <class P, int NCH, int GR, bool FWD, bool BWD>
-__global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const __grid_constant__ RenderTcArgs a) {
+__global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const __grid_constant__ RenderTcArgs a) {
   using L = TcLayout<P>;
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr uint32_t wplane = wTotal<P>();  // one bf16 part of all weight tiles
-  uint8_t* wt0 = smem;
-  float* acc = reinterpret_cast<float*>(smem + wplane * P::planes);  // [kMlpPad] + loss [kLossPad]
-  float* lacc = acc + kMlpPad;
-  float* bias = lacc + kLossPad;  // b1[32] b2[16] b3[32] b4[4] kappa
+  // tile groups | weight tiles | exchange rows [GR][NCH][128] float4 | rays | accumulators, biases
+  uint8_t* gbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem) + 127) & ~uintptr_t(127));
+  uint8_t* wt0 = gbase + (size_t)GR * L::group_bytes;
+  float4* xch0 = reinterpret_cast<float4*>(wt0 + wplane * P::planes);
+  float4* rays0 = xch0 + (size_t)GR * NCH * 128;
+  float* sums0 = reinterpret_cast<float*>(rays0 + GR * 20);  // [GR][4][kSums]: a compositing warp's running sums
+  float* bias = sums0 + GR * 4 * kSums;  // b1[32] b2[16] b3[32] b4[4] kappa
   float* w4f = bias + 88;         // W4 [3][32] in FP32: the colour output layer runs on CUDA cores
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(w4f + 96);
-  float* gacc = reinterpret_cast<float*>(tslot + 4);  // per-group decoder-gradient accumulators [GR][kMlpPad]
-  uint8_t* gbase = reinterpret_cast<uint8_t*>(gacc + GR * kMlpPad);
-  gbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(gbase) + 1023) & ~uintptr_t(1023));
+  float* kc = w4f + 96;           // loss scales of rgb, depth, sdf, fs; sharpness
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(kc + 8);
 
-  const int tid = threadIdx.x, gi = tid / kGroupThreads, gt = tid % kGroupThreads, warp_g = gt >> 5,
-            lane = tid & 31;
-  uint8_t* gmem = gbase + (size_t)gi * L::group_bytes;
-  Group G;
-  G.a = gmem;
-  G.b = gmem + L::a_bytes * P::planes;
-  G.mbar = reinterpret_cast<uint64_t*>(gmem + L::a_bytes * P::planes + L::b_bytes * L::b_planes);
-  G.mbar_dw = G.mbar + 1;
-  G.mbar_tma = G.mbar + 2;
-  G.abort = reinterpret_cast<int*>(G.mbar + 3);
-  G.phase_dw = 0;
-  G.phase_tma = 0;
-  G.dw_pending = false;
-  G.g = gi;
-  G.gt = gt;
-  G.phase = 0;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
+  const int gi = warp >> 3, w8 = warp & 7, half = w8 >> 2, wq = w8 & 3;
+  const int row = 32 * wq + lane;  // tile row of this thread's sample
+  uint8_t* const tileA = gbase + (size_t)gi * L::group_bytes;
+  uint8_t* const tileB = tileA + L::b_off;
+  Tile T;
+  T.bars = reinterpret_cast<TileBars*>(tileA + L::bar_off);
+  T.ph_done = T.ph_dw = 0;
+  T.w8 = w8;
+  T.g = gi;
+  T.dw_pending = false;
 
   // ---- CTA set-up: weight tiles, biases, accumulators, barriers, tensor memory ----
   const float* mlp = a.theta + a.g.n_grid;
-  for (int m = 0; m < 8; ++m) {
+  for (int m = 0; m < kTiles; ++m) {
     const int Nn = wN(m), K = wK(m);
     for (int e = tid; e < Nn * K; e += blockDim.x) {
       const int n = e / K, k = e % K;
@@ -670,10 +839,8 @@ __global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const 
         case 0: v = mlp[oW1 + n * kZ + k]; break;
         case 1: v = mlp[oW2 + n * kH1 + k]; break;
         case 2: v = k < kHF ? mlp[oW3 + n * kHF + k] : 0.f; break;
-        case 3: v = n < kRGB ? mlp[oW4 + n * kH2 + k] : 0.f; break;
-        case 4: v = k < kRGB ? mlp[oW4 + k * kH2 + n] : 0.f; break;
-        case 5: v = n < kHF ? mlp[oW3 + k * kHF + n] : 0.f; break;
-        case 6: v = mlp[oW2 + k * kH1 + n]; break;
+        case 3: v = n < kHF ? mlp[oW3 + k * kHF + n] : 0.f; break;
+        case 4: v = mlp[oW2 + k * kH1 + n]; break;
         default: v = mlp[oW1 + k * kZ + n]; break;
       }
       store_w<P>(wt0 + wOff<P>(m), wplane, K, n, k, v);
@@ -689,151 +856,220 @@ __global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const 
     else if (i == 84) v = mlp[oKappa];
     bias[i] = v;
   }
-  for (int i = tid; i < kMlpPad + kLossPad; i += blockDim.x) acc[i] = 0.f;
-  for (int i = tid; i < GR * kMlpPad; i += blockDim.x) gacc[i] = 0.f;
-  if (gt == 0) {
-    tc::mbar_init(G.mbar, 1);
-    tc::mbar_init(G.mbar_dw, 1);
-    tc::mbar_init(G.mbar_tma, 1);
+  if (tid < GR * 4 * kSums) sums0[tid] = 0.f;
+  if (w8 == 0 && lane == 0) {
+    tc::mbar_init(&T.bars->done, 1);
+    tc::mbar_init(&T.bars->dw, 1);
     tc::fence_mbar_init();
-    if (P::planes > 1) tc::mbar_arrive_expect_tx(G.mbar_tma, kFineTmaBytes);  // armed for the first round
-    *G.abort = 0;
+    T.bars->abort = 0;
+  }
+  if (tid == 0) {
+    float wt[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) wt[k] = a.dloss[k] + a.lam[k] * a.dloss[5];
+    const int n_d = a.counts[0], n_tr = a.counts[1], n_fs = a.counts[2];
+    kc[0] = a.R > 0 ? wt[0] * 2.0f / (float)a.R : 0.f;
+    kc[1] = n_d > 0 ? wt[1] / (float)n_d : 0.0f;
+    kc[2] = n_tr > 0 ? wt[2] / (float)n_tr : 0.0f;
+    kc[3] = n_fs > 0 ? wt[3] / (float)n_fs : 0.0f;
+    kc[4] = expf(mlp[oKappa]);
   }
   static_assert(tmem_cols(GR) <= 512, "tensor memory holds 512 columns");
-  if (tid < 32) tc::tmem_alloc(tslot, tmem_cols(GR));
+  if (warp == 0) tc::tmem_alloc(tslot, tmem_cols(GR));
   tc::fence_smem_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  G.tcol = *tslot + (uint32_t)(gi * kGroupCols);
-  const float* b1 = bias;
-  const float* b2 = bias + 32;
-  const float* b3 = bias + 48;
-  const float* b4 = bias + 80;
-  const float s_sharp = expf(bias[84]);
-  float* macc = gacc + gi * kMlpPad;  // this group's decoder-gradient accumulator
-
-  const int N = a.N;
-  float wt[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) wt[k] = a.dloss[k] + a.lam[k] * a.dloss[5];
-  const int n_d = a.counts[0], n_tr = a.counts[1], n_fs = a.counts[2];
-  const float k_rgb = a.R > 0 ? wt[0] * 2.0f / (float)a.R : 0.f;
-  const float k_d = n_d > 0 ? wt[1] / (float)n_d : 0.0f;
-  const float k_sdf = n_tr > 0 ? wt[2] / (float)n_tr : 0.0f;
-  const float k_fs = n_fs > 0 ? wt[3] / (float)n_fs : 0.0f;
-  float l_rgb = 0.f, l_d = 0.f, l_sdf = 0.f, l_fs = 0.f, g_kappa = 0.f;
-  const int row = gt;  // tile row of this thread's sample
+  const uint32_t tmem0 = __shfl_sync(0xffffffffu, *tslot, 0);
+  const int N = a.N, quads = (a.R + 3) / 4;
+  const bool stored = a.store != nullptr;
+  const bool fphases = FWD || !stored;  // the forward layers run before the compositing
   bool alive = true;
   bool dw_acc = false;  // the weight-gradient accumulators hold a first tile (accumulate from then on)
-  float w4acc[3] = {0.f, 0.f, 0.f}, b4acc = 0.f;  // this warp's dW4[.][lane] and (lanes < 3) db4[lane]
+  // dW4[.][16 half + lane % 16] over this warp's samples of parity lane / 16
+  float w4acc[3] = {0.f, 0.f, 0.f};
 
-  // ray-quads are dealt CTA-major (quad = round * G + CTA * GR + gi): when the quads do not
-  // divide evenly, whole SMs finish a round early, and the smoothness kernel, launched beside
-  // this one on another stream, runs there
-  for (int quad = blockIdx.x * GR + gi; quad * 4 < a.R && alive; quad += gridDim.x * GR) {
-    const int ray = quad * 4 + warp_g;
+  const uint32_t sw = tc::smem_u32(wt0), sa = tc::smem_u32(gbase) + (uint32_t)gi * L::group_bytes;
+  const uint32_t tcol = tmem0 + (uint32_t)(gi * kGroupCols);
+  const uint32_t tq = tcol + ((uint32_t)(32 * wq) << 16), ta = tq + cA;  // this warp's lanes
+  const float* b1 = bias + 16 * half;  // this half's units
+  const float* b2 = bias + 32;
+  const float* b3 = bias + 48 + 16 * half;
+  const float* b4 = bias + 80;
+  const float* w4h = w4f + 16 * half;
+  float4* xch = xch0 + (size_t)gi * NCH * 128;
+  float4* rays = rays0 + (gi * 8 + w8) * 2;                     // this warp's ray: o, r
+  float4* tint = rays0 + GR * 8 * 2 + gi * 4 + wq;              // its colour and depth (written by the upper half)
+  const int l_lo = half ? 1 : 0, l_hi = half ? 2 : 3;  // this half's grid levels (coarse, fine)
+
+  // this half's features of the sample at x into the A operand (levels' columns 4 l .. 4 l + 3)
+  auto gather_store = [&](const float x[3], bool valid, float4& zl, float4& zh) {
+    zl = zh = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (valid) {
+      if constexpr (P::planes > 1) {
+        if (half == 0) {
+          FineCorners fc;
+          fine_corners_load(a.g, a.theta, x, fc);
+          zl = level_features(a.g, a.theta, 0, x);
+          zh = fine_corners_sum(fc);
+        } else {
+          zh = level_features(a.g, a.theta, 2, x);
+          zl = level_features(a.g, a.theta, 1, x);
+        }
+      } else {
+        zh = level_features_bf16(a.g, a.theta_bf16, l_hi, x);
+        zl = level_features_bf16(a.g, a.theta_bf16, l_lo, x);
+      }
+    }
+    __syncwarp();
+    const float lo4[4] = {zl.x, zl.y, zl.z, zl.w}, hi4[4] = {zh.x, zh.y, zh.z, zh.w};
+    put_operand<P, 16, false, 2>(ta, nullptr, row, 2 * l_lo, lo4);
+    put_operand<P, 16, false, 2>(ta, nullptr, row, 2 * l_hi, hi4);
+  };
+  auto position = [&](float t, float x[3]) {
+    const float4 o4 = rays[0], r4 = rays[1];
+    const float o[3] = {o4.x, o4.y, o4.z}, r[3] = {r4.x, r4.y, r4.z};
+    sample_pos(o, r, t, x);
+  };
+  // this half's 8 columns of [h | 0] from the 16 outputs [phi, h] of the second layer
+  auto hidden_row = [&](const float (&u)[16], float (&h)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float lo = u[k + 1] + b2[k + 1], hi = k < 7 ? u[k < 7 ? k + 9 : 0] + b2[k < 7 ? k + 9 : 0] : 0.f;
+      h[k] = half == 0 ? lo : hi;
+    }
+  };
+
+  // ray-quads are dealt group-major (quad = round * G + group * CTAs + CTA): a batch with fewer
+  // quads than tile groups spreads over all SMs, and so does the last, partial round
+  for (int quad = gi * (int)gridDim.x + (int)blockIdx.x; quad < quads && alive; quad += (int)gridDim.x * GR) {
+    const int ray = quad * 4 + wq;
     const bool has_ray = ray < a.R;
     const int rr = has_ray ? ray : 0;
-    const float o[3] = {a.o[3 * rr], a.o[3 * rr + 1], a.o[3 * rr + 2]};
-    const float r[3] = {a.r[3 * rr], a.r[3 * rr + 1], a.r[3 * rr + 2]};
-    const float D = has_ray ? a.D[rr] : 0.f;
-    const float I[3] = {a.rgb[3 * rr], a.rgb[3 * rr + 1], a.rgb[3 * rr + 2]};
-    float tt[NCH], ph[NCH], col[NCH][3];
-    int clv[NCH];  // sample classes
-    // every per-sample input of the ray up front: one memory round trip instead of one per chunk
+    // every sample depth of the ray up front: one memory round trip instead of one per chunk
+    float tt[NCH];
 #pragma unroll
     for (int q = 0; q < NCH; ++q) {
       const int si = 32 * q + lane;
-      const bool in = has_ray && si < N;
-      tt[q] = in ? a.t[(size_t)rr * N + si] : 0.f;
-      clv[q] = in ? (int)a.cls[(size_t)rr * N + si] : 0;
+      tt[q] = has_ray && si < N ? a.t[(size_t)rr * N + si] : 0.f;
     }
+    __syncwarp();
+    if (lane < 6) reinterpret_cast<float*>(rays)[lane < 3 ? lane : lane + 1] = lane < 3 ? a.o[3 * rr + lane] : a.r[3 * rr + lane - 3];
+    __syncwarp();
+    float ph[NCH], col[NCH][3];
 
-    // ================= forward: gather, then 4 decoder phases per chunk =================
+    // ================= forward: gather, then 3 decoder phases per chunk =================
 #pragma unroll 1
     for (int j = 0; j < NCH && alive; ++j) {
       const int si = 32 * j + lane;
       const bool valid = has_ray && si < N;
-      const float t = pick_tc(tt, j);
-      float4* sp = a.store != nullptr ? reinterpret_cast<float4*>(a.store) + (size_t)rr * N + si : nullptr;
-      const long long ss = a.store_stride;
-      if (!FWD && sp != nullptr) {  // stored by the forward pass: no decoder phases here
-        const float4 o4 = valid ? sp[(kFout / 4) * ss] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 c4 = valid ? sp[(kFc / 4) * ss] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const StoreRef sp{reinterpret_cast<float4*>(a.store) + ((size_t)rr * N + 32 * j) * 25 + lane, min(32, N - 32 * j)};
+      if (!fphases) {  // stored by the forward pass: no decoder phases here
+        if (half != 0) {
+          xch[j * 128 + row].w = __int_as_float(valid ? (int)a.cls[(size_t)rr * N + si] : 0);
+          if (j == 0 && lane == 0) *tint = make_float4(a.rgb[3 * rr], a.rgb[3 * rr + 1], a.rgb[3 * rr + 2], has_ray ? a.D[rr] : 0.f);
+          continue;
+        }
+        const float4 c4 = valid ? sp[kPc] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int q = 0; q < NCH; ++q)
           if (q == j) {
-            tt[q] = t;
-            ph[q] = o4.x;
+            ph[q] = c4.w;
             col[q][0] = c4.x;
             col[q][1] = c4.y;
             col[q][2] = c4.z;
           }
         continue;
       }
-      const bool put = FWD && sp != nullptr && valid;
-      float z[kZ];
+      const bool put = FWD && stored && valid;
+      int cl = 0;
+      float4 i4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (half != 0) {  // the compositing's other inputs, fetched by the half that does not composite
+        if (valid) cl = (int)a.cls[(size_t)rr * N + si];
+        if (j == 0 && lane == 0) i4 = make_float4(a.rgb[3 * rr], a.rgb[3 * rr + 1], a.rgb[3 * rr + 2], has_ray ? a.D[rr] : 0.f);
+      }
+      float4 zl, zh;
       {
         float x[3];
-        sample_pos(o, r, t, x);
-        dw_wait(G);  // the TMA slots overlap the partner tile and the A planes
-        gather_chunk<P>(G, a, x, valid, z);
+        position(pick_tc(tt, j), x);
+        gather_store(x, valid, zl, zh);
       }
-      store_row<P, 16>(G.a, row, z);
-      mma_phase_issue<P, 32, 16>(G, cD1, wt0 + wOff<P>(0), wplane);
-      if (put) put_fields<kFz, 16>(sp, ss, z);
-      if (!(alive = mma_phase_wait(G))) break;
-      float v[32];
-      tc::tmem_ld32(lane_addr(G, cD1, warp_g), v);
+      phase_issue<P, 0>(T, tcol, sa, sw, dw_acc);
+      if (put) {
+        sp[kPz + l_lo] = zl;
+        sp[kPz + l_hi] = zh;
+      }
+      if (!(alive = phase_wait(T))) break;
+      float v[16];
+      tc::tmem_ld16(tq + cX + 16 * half, v);
       tc::tmem_ld_wait();
 #pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = fmaxf(v[k] + b1[k], 0.f);
-      store_row<P, 32>(G.a, row, v);
-      mma_phase_issue<P, 16, 32>(G, cD2, wt0 + wOff<P>(1), wplane);
-      if (put) put_fields<kFa1, 32>(sp, ss, v);
-      if (!(alive = mma_phase_wait(G))) break;
+      for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k] + b1[k], 0.f);
+      put_operand<P, 32, false, 8>(ta, nullptr, row, 8 * half, v);
+      phase_issue<P, 1>(T, tcol, sa, sw, dw_acc);
+      if (put) put_planes<4>(sp, kPa1 + 4 * half, v);
+      if (!(alive = phase_wait(T))) break;
       float u[16];
-      tc::tmem_ld16(lane_addr(G, cD2, warp_g), u);
+      tc::tmem_ld16(tq + cY, u);
       tc::tmem_ld_wait();
       const float phi = u[0] + b2[0];
-      float h[16];
-#pragma unroll
-      for (int k = 0; k < 15; ++k) h[k] = u[k + 1] + b2[k + 1];
-      h[15] = 0.f;
-      store_row<P, 16>(G.a, row, h);
-      mma_phase_issue<P, 32, 16>(G, cD3, wt0 + wOff<P>(2), wplane);
-      if (put) {
-        float oh[16];
-        oh[0] = phi;
-#pragma unroll
-        for (int k = 0; k < 15; ++k) oh[k + 1] = h[k];
-        put_fields<kFout, 16>(sp, ss, oh);
-      }
-      if (!(alive = mma_phase_wait(G))) break;
-      tc::tmem_ld32(lane_addr(G, cD3, warp_g), v);
+      float h[8];
+      hidden_row(u, h);
+      put_operand<P, 16, false, 4>(ta, nullptr, row, 4 * half, h);
+      phase_issue<P, 2>(T, tcol, sa, sw, dw_acc);
+      if (put) put_planes<2>(sp, kPh + 2 * half, h);
+      if (!(alive = phase_wait(T))) break;
+      tc::tmem_ld16(tq + cX + 16 * half, v);
       tc::tmem_ld_wait();
 #pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = fmaxf(v[k] + b3[k], 0.f);
-      if (put) put_fields<kFa2, 32>(sp, ss, v);
+      for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k] + b3[k], 0.f);
+      if (put) put_planes<4>(sp, kPa2 + 4 * half, v);
+      // this half's part of the colour pre-activations W4 a2 + b4
       float c3[3];
-      colour_out(w4f, b4, v, c3);
-      if (put) {
-        const float c4[4] = {c3[0], c3[1], c3[2], 0.f};
-        put_fields<kFc, 4>(sp, ss, c4);
+#pragma unroll
+      for (int n = 0; n < 3; ++n) {
+        float s = half == 0 ? b4[n] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s = fmaf(w4h[32 * n + k], v[k], s);
+        c3[n] = s;
+      }
+      if (half != 0) {
+        xch[j * 128 + row] = make_float4(c3[0], c3[1], c3[2], __int_as_float(cl));
+        if (j == 0 && lane == 0) *tint = i4;
       }
       // keep per-chunk values in registers (compile-time index via a selector loop)
 #pragma unroll
       for (int q = 0; q < NCH; ++q)
         if (q == j) {
-          tt[q] = t;
           ph[q] = valid ? phi : 0.f;
-          col[q][0] = valid ? c3[0] : 0.f;
-          col[q][1] = valid ? c3[1] : 0.f;
-          col[q][2] = valid ? c3[2] : 0.f;
+          col[q][0] = c3[0];
+          col[q][1] = c3[1];
+          col[q][2] = c3[2];
         }
     }
     if (!alive) break;
+    // the upper half's parts of the colours, the classes, the observed colour and depth
+    group_sync<kTileThreads>(gi);
+
+    if (half == 0) {  // ---- compositing and its adjoint: the lower half, a warp per ray ----
+    int clv[NCH];  // sample classes
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+      const bool valid = has_ray && 32 * j + lane < N;
+      const float4 p4 = xch[j * 128 + row];
+      clv[j] = __float_as_int(p4.w);
+      if (fphases) {
+        col[j][0] = valid ? sigmoidf_(col[j][0] + p4.x) : 0.f;
+        col[j][1] = valid ? sigmoidf_(col[j][1] + p4.y) : 0.f;
+        col[j][2] = valid ? sigmoidf_(col[j][2] + p4.z) : 0.f;
+        if (FWD && stored && valid)
+          reinterpret_cast<float4*>(a.store)[((size_t)rr * N + 32 * j) * 25 + kPc * min(32, N - 32 * j) + lane] =
+              make_float4(col[j][0], col[j][1], col[j][2], ph[j]);
+      }
+    }
+    const float4 in4 = *tint;
+    const float D = in4.w, I[3] = {in4.x, in4.y, in4.z}, s_sharp = kc[4];
+    float l_rgb = 0.f, l_d = 0.f, l_sdf = 0.f, l_fs = 0.f, g_kappa = 0.f, db4[3] = {0.f, 0.f, 0.f};
 
     // ================= NeuS opacity, transmittance, weights (Sec. 3.2) =================
     float Ph[NCH], PhN[NCH], al[NCH], T[NCH], w[NCH];
@@ -906,13 +1142,13 @@ __global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const 
         else if (cl == CLS_FS) l_fs += fmaxf(fmaxf(0.f, expf(-a.kappa_fs * ph[j]) - 1.0f), ph[j] - b);
       }
     }
-    if constexpr (!BWD) continue;
+    if constexpr (BWD) {
 
     // ================= adjoint of compositing: dL/dalpha_k = T_k (e_k - U_k) =================
     float gc[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) gc[k] = has_ray ? k_rgb * (ch[k] - I[k]) : 0.f;
-    const float gd = (has_ray && D > 0.f) ? k_d * ((dh > D) ? 1.f : (dh < D ? -1.f : 0.f)) : 0.f;
+    for (int k = 0; k < 3; ++k) gc[k] = has_ray ? kc[0] * (ch[k] - I[k]) : 0.f;
+    const float gd = (has_ray && D > 0.f) ? kc[1] * ((dh > D) ? 1.f : (dh < D ? -1.f : 0.f)) : 0.f;
     float e[NCH], U[NCH];
 #pragma unroll
     for (int j = 0; j < NCH; ++j) e[j] = gc[0] * col[j][0] + gc[1] * col[j][1] + gc[2] * col[j][2] + gd * tt[j];
@@ -938,7 +1174,6 @@ __global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const 
       cA = fmaf(B0, cA, A0);
     }
     float dnext_prev = 0.f;
-    float dphi[NCH];
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
       const int si = 32 * j + lane;
@@ -965,7 +1200,7 @@ __global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const 
         const float b = __fsub_rn(D, tt[j]);
         if (cl == CLS_TR) {
           const float df = ph[j] - b;
-          d += k_sdf * (df > 0.f ? 1.f : (df < 0.f ? -1.f : 0.f));
+          d += kc[2] * (df > 0.f ? 1.f : (df < 0.f ? -1.f : 0.f));
         } else if (cl == CLS_FS) {
           const float ex = expf(-a.kappa_fs * ph[j]) - 1.0f, lin = ph[j] - b;
           int arg = 0;
@@ -975,278 +1210,281 @@ __global__ void __launch_bounds__(GR * kGroupThreads, 1) render_tc_kernel(const 
             arg = 1;
           }
           if (lin > top) arg = 2;
-          d += k_fs * (arg == 1 ? -a.kappa_fs * (ex + 1.0f) : (arg == 2 ? 1.0f : 0.0f));
+          d += kc[3] * (arg == 1 ? -a.kappa_fs * (ex + 1.0f) : (arg == 2 ? 1.0f : 0.0f));
         }
       } else {
         d = 0.f;
       }
-      dphi[j] = d;
+      // the reverse pass's seeds of the sample: the colour pre-activations' (w gc c (1 - c)) and phi's
+      float dp[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) dp[k] = valid ? w[j] * gc[k] * col[j][k] * (1.0f - col[j][k]) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) db4[k] += dp[k];
+      xch[j * 128 + row] = make_float4(dp[0], dp[1], dp[2], d);
     }
+    }  // BWD
+    {
+      float q[kSums] = {l_rgb, l_d, l_sdf, l_fs, g_kappa, db4[0], db4[1], db4[2]};
+#pragma unroll
+      for (int k = 0; k < kSums; ++k) q[k] = warp_sum(q[k]);
+      if (lane == 0) {
+        float* sm = sums0 + (gi * 4 + wq) * kSums;
+#pragma unroll
+        for (int k = 0; k < kSums; ++k) sm[k] += q[k];
+      }
+    }
+    }  // lower half
+    if constexpr (!BWD) continue;
+    group_sync<kTileThreads>(gi);  // the reverse pass's seeds
 
-    // ================= reverse, chunk by chunk: recompute, 4 adjoint phases =================
+    // ================= reverse, chunk by chunk: (recompute,) 3 adjoint phases =================
 #pragma unroll 1
     for (int j = 0; j < NCH && alive; ++j) {
       const int si = 32 * j + lane;
       const bool valid = has_ray && si < N;
-      const float t = pick_tc(tt, j);
-      float x[3];
-      sample_pos(o, r, t, x);
-      const float4* sp = a.store != nullptr ? reinterpret_cast<const float4*>(a.store) + (size_t)rr * N + si : nullptr;
-      const long long ss = a.store_stride;
-      const bool get = sp != nullptr && valid;
-      float z[kZ], v[32], h[16], u[16], c3[3];
-      uint32_t mask2 = 0;
-      if (sp != nullptr) {  // stored activations: z, a2, h and c now, a1 where it is used
-        get_fields<kFz, 16>(sp, ss, get, z);
-        get_fields<kFa2, 32>(sp, ss, get, v);
-        float oh[16];
-        get_fields<kFout, 16>(sp, ss, get, oh);
-#pragma unroll
-        for (int k = 0; k < 15; ++k) h[k] = oh[k + 1];
-        h[15] = 0.f;
-        float c4[4];
-        get_fields<kFc, 4>(sp, ss, get, c4);
-        c3[0] = c4[0];
-        c3[1] = c4[1];
-        c3[2] = c4[2];
+      const StoreRef sp{reinterpret_cast<float4*>(a.store) + ((size_t)rr * N + 32 * j) * 25 + lane, min(32, N - 32 * j)};
+      const bool get = stored && valid;
+      float v[16], h[8], a1[16];
+      float4 zl, zh;
+      if (stored) {  // stored activations: a2 and h now, a1 and z where they are used
+        get_planes<4>(sp, kPa2 + 4 * half, get, v);
+        get_planes<2>(sp, kPh + 2 * half, get, h);
       } else {
-        dw_wait(G);
-        gather_chunk<P>(G, a, x, valid, z);
-        // recompute the decoders (the same four phases as the forward)
-        store_row<P, 16>(G.a, row, z);
-        mma_phase_issue<P, 32, 16>(G, cD1, wt0 + wOff<P>(0), wplane);
-        if (!(alive = mma_phase_wait(G))) break;
-        tc::tmem_ld32(lane_addr(G, cD1, warp_g), v);
+        // recompute the decoders (the same phases as the forward)
+        {
+          float x[3];
+          position(pick_tc(tt, j), x);
+          gather_store(x, valid, zl, zh);
+        }
+        phase_issue<P, 0>(T, tcol, sa, sw, dw_acc);
+        if (!(alive = phase_wait(T))) break;
+        tc::tmem_ld16(tq + cX + 16 * half, a1);
         tc::tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = fmaxf(v[k] + b1[k], 0.f);
-        store_row<P, 32>(G.a, row, v);
-        mma_phase_issue<P, 16, 32>(G, cD2, wt0 + wOff<P>(1), wplane);
-        if (!(alive = mma_phase_wait(G))) break;
-        tc::tmem_ld16(lane_addr(G, cD2, warp_g), u);
+        for (int k = 0; k < 16; ++k) a1[k] = fmaxf(a1[k] + b1[k], 0.f);
+        put_operand<P, 32, false, 8>(ta, nullptr, row, 8 * half, a1);
+        phase_issue<P, 1>(T, tcol, sa, sw, dw_acc);
+        if (!(alive = phase_wait(T))) break;
+        float u[16];
+        tc::tmem_ld16(tq + cY, u);
+        tc::tmem_ld_wait();
+        hidden_row(u, h);
+        put_operand<P, 16, false, 4>(ta, nullptr, row, 4 * half, h);
+        phase_issue<P, 2>(T, tcol, sa, sw, dw_acc);
+        if (!(alive = phase_wait(T))) break;
+        tc::tmem_ld16(tq + cX + 16 * half, v);
         tc::tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < 15; ++k) h[k] = u[k + 1] + b2[k + 1];
-        h[15] = 0.f;
-        store_row<P, 16>(G.a, row, h);
-        mma_phase_issue<P, 32, 16>(G, cD3, wt0 + wOff<P>(2), wplane);
-        if (!(alive = mma_phase_wait(G))) break;
-        tc::tmem_ld32(lane_addr(G, cD3, warp_g), v);
-        tc::tmem_ld_wait();
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = fmaxf(v[k] + b3[k], 0.f);
-        colour_out(w4f, b4, v, c3);
+        for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k] + b3[k], 0.f);
       }
-#pragma unroll
-      for (int k = 0; k < 32; ++k) mask2 |= (v[k] > 0.f ? 1u : 0u) << k;
-      // colour output adjoint: dpre = w gc c (1 - c)
-      const float wj = pick_tc(w, j);
-      float dp[kKD];
-#pragma unroll
-      for (int k = 0; k < kKD; ++k) dp[k] = 0.f;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) dp[k] = valid ? wj * gc[k] * c3[k] * (1.0f - c3[k]) : 0.f;
-      dw_wait(G);  // no tensor-core product reads the tiles now: stage the colour layer's rows there
-      // --- b4 on CUDA cores: da2 = dpre W4 (3 x 32); dW4, db4 (+)= sum over the warp's samples ---
+      const float4 seed = xch[j * 128 + row];  // dL/d(colour pre-activations), dL/dphi
+      tiles_free(T);  // stage the colour layer's rows there
+      // --- b4 on CUDA cores: da2 = dpre W4 (3 x 32); dW4 (+)= sum over the warp's samples ---
       {
-        // 4 warps x 32 rows x 36 floats = 18 KB from the A planes on (the A and partner planes
-        // are contiguous and hold at least 20 KB in both forms)
-        static_assert(L::a_bytes * P::planes + L::b_bytes * L::b_planes >= 4u * 32u * 36u * 4u, "staging space");
-        float* st = reinterpret_cast<float*>(G.a) + warp_g * (32 * 36);  // row: dpre[3] | 0 | a2[32]
-        float* rw = st + lane * 36;
-        *reinterpret_cast<float4*>(rw) = make_float4(dp[0], dp[1], dp[2], 0.f);
+        // This warp's 16 a2 columns, 64 bytes a row (the 16-byte pieces rotated against bank
+        // conflicts), in the part of the adjoint tile that only this warp writes: of each 8-row group
+        // of a K = 32 tile, its half's 256 bytes of a part hold 4 staged rows.  The BF16 form's
+        // one part is too small: its rows have their own space.
+        constexpr uint32_t kBlk = P::planes > 1 ? L::row_stride(32) : 256u, kPl = P::planes > 1 ? 512u : 1024u;
+        uint8_t* st = P::planes > 1 ? tileA + wq * 4 * L::row_stride(32) + half * 256 : tileA + L::stage_off + w8 * 2048;
+        float* rw = reinterpret_cast<float*>(st + (lane >> 4) * kPl + ((lane >> 2) & 3) * kBlk + (lane & 3) * 64);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4*>(rw + 4 + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<float4*>(rw + 4 * ((q + (lane >> 1)) & 3)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         __syncwarp();
-#pragma unroll 4
-        for (int s2 = 0; s2 < 32; ++s2) {
-          const float* r2 = st + s2 * 36;
-          const float a2v = r2[4 + lane];
-          w4acc[0] = fmaf(r2[0], a2v, w4acc[0]);
-          w4acc[1] = fmaf(r2[1], a2v, w4acc[1]);
-          w4acc[2] = fmaf(r2[2], a2v, w4acc[2]);
-          b4acc += r2[lane & 3];
+        const int hi = lane >> 4, un = lane & 15;  // rows 2 i + hi, unit un of the half
+        const float4* sd = xch + j * 128 + 32 * wq + hi;
+        uint32_t rot[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) rot[i] = (uint32_t)((((un >> 2) + i) & 3) * 16 + (un & 3) * 4 + hi * 64);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const uint32_t off = (uint32_t)(i >> 3) * kPl + (uint32_t)((i >> 1) & 3) * kBlk + (uint32_t)(i & 1) * 128u;
+          const float a2v = *reinterpret_cast<const float*>(st + off + rot[i & 3]);
+          const float4 d4 = sd[2 * i];
+          w4acc[0] = fmaf(d4.x, a2v, w4acc[0]);
+          w4acc[1] = fmaf(d4.y, a2v, w4acc[1]);
+          w4acc[2] = fmaf(d4.z, a2v, w4acc[2]);
         }
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {  // dy2 = mask2 (.) (dpre W4)
-          const float d = fmaf(dp[0], w4f[k], fmaf(dp[1], w4f[32 + k], dp[2] * w4f[64 + k]));
-          v[k] = ((mask2 >> k) & 1u) ? d : 0.f;
+        for (int k = 0; k < 16; ++k) {  // dy2 = mask2 (.) (dpre W4)
+          const float d = fmaf(seed.x, w4h[k], fmaf(seed.y, w4h[32 + k], seed.z * w4h[64 + k]));
+          v[k] = v[k] > 0.f ? d : 0.f;
         }
-        group_sync(G.g);  // every warp has read its staged rows before the tiles are rewritten
       }
-      store_row<P, 32>(G.a, row, v);
-      h[15] = 1.f;  // ones column: the bias gradient db3 lands in column 15 of dW3
-      store_row_planes<L::b_planes, 16, L::b_bytes>(G.b, row, h);
+      put_operand<P, 32, true, 8>(ta, tileA, row, 8 * half, v);
+      if (half != 0) h[7] = 1.f;  // ones column: the bias gradient db3 lands in column 15 of dW3
+      store_chunk<L::b_planes, 16, L::b_bytes>(tileB, row, half, h);
       // --- b3: dh = dy2 W3;  dW3, db3 (+)= dy2^T [h | 1] ---
-      mma_phase_issue_dw<P, 16, 32>(G, cYb, wt0 + wOff<P>(5), wplane, [&] {
-        issue_mma_dw<P::planes, L::b_planes, kDwSum<P>, 16>(G.tcol + cW3, tc::smem_u32(G.a), L::a_bytes, 4u * 128u,
-                                                            tc::smem_u32(G.b), L::b_bytes, 2u * 128u, dw_acc);
-      });
-      if (!(alive = mma_phase_wait(G))) break;
-      tc::tmem_ld16(lane_addr(G, cYb, warp_g), u);
-      tc::tmem_ld_wait();
-      float dout[16];
-      dout[0] = valid ? pick_tc(dphi, j) : 0.f;
-#pragma unroll
-      for (int k = 1; k < 16; ++k) dout[k] = u[k - 1];
-      dw_wait(G);
-      store_row<P, 16>(G.a, row, dout);
-      uint32_t mask1 = 0;
+      phase_issue<P, 3>(T, tcol, sa, sw, dw_acc);
+      if (stored) get_planes<4>(sp, kPa1 + 4 * half, get, a1);
+      if (!(alive = phase_wait(T))) break;
       {
-        float ab[40];
-        if (sp != nullptr) {
-          get_fields<kFa1, 32>(sp, ss, get, ab);
-        } else {
-          float a1[32];
-          tc::tmem_ld32(lane_addr(G, cD1, warp_g), a1);
-          tc::tmem_ld_wait();
+        float u[16], dout[8];
+        tc::tmem_ld16(tq + cY, u);
+        tc::tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 32; ++k) ab[k] = fmaxf(a1[k] + b1[k], 0.f);
-        }
-#pragma unroll
-        for (int k = 0; k < 32; ++k) mask1 |= (ab[k] > 0.f ? 1u : 0u) << k;
-        ab[32] = 1.f;
-#pragma unroll
-        for (int k = 33; k < 40; ++k) ab[k] = 0.f;
-        store_row_planes<L::b_planes, 40, L::b_bytes>(G.b, row, ab);
+        for (int k = 0; k < 8; ++k) dout[k] = half == 0 ? (k == 0 ? (valid ? seed.w : 0.f) : u[k > 0 ? k - 1 : 0]) : u[k + 7];
+        tiles_free(T);
+        put_operand<P, 16, true, 4>(ta, tileA, row, 4 * half, dout);
       }
+#pragma unroll
+      for (int c = 0; c < 2; ++c) store_chunk<L::b_planes, 40, L::b_bytes>(tileA + L::b_wide, row, 2 * half + c, a1 + 8 * c);
+      const float one8[8] = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (half != 0) store_chunk<L::b_planes, 40, L::b_bytes>(tileA + L::b_wide, row, 4, one8);
       // --- b2: da1 = dout W2;  dW2^T, db2 (+)= [a1 | 1]^T dout ---
-      mma_phase_issue_dw<P, 32, 16>(G, cXb, wt0 + wOff<P>(6), wplane, [&] {
-        issue_mma_dw<L::b_planes, P::planes, kDwSum<P>, 16>(G.tcol + cW2, tc::smem_u32(G.b), L::b_bytes, 5u * 128u,
-                                                            tc::smem_u32(G.a), L::a_bytes, 2u * 128u, dw_acc);
-      });
-      if (!(alive = mma_phase_wait(G))) break;
-      tc::tmem_ld32(lane_addr(G, cXb, warp_g), v);
-      tc::tmem_ld_wait();
-#pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = ((mask1 >> k) & 1u) ? v[k] : 0.f;  // dy1
-      dw_wait(G);
-      store_row<P, 32>(G.a, row, v);
-      {
-        float zb[24];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) zb[k] = z[k];
-        zb[16] = 1.f;
-#pragma unroll
-        for (int k = 17; k < 24; ++k) zb[k] = 0.f;
-        store_row_planes<L::b_planes, 24, L::b_bytes>(G.b, row, zb);
+      phase_issue<P, 4>(T, tcol, sa, sw, dw_acc);
+      if (stored) {
+        zl = get ? sp[kPz + l_lo] : make_float4(0.f, 0.f, 0.f, 0.f);
+        zh = get ? sp[kPz + l_hi] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      // --- b1: dz = dy1 W1;  dW1, db1 (+)= dy1^T [z | 1] ---
-      mma_phase_issue_dw<P, 16, 32>(G, cYb, wt0 + wOff<P>(7), wplane, [&] {
-        issue_mma_dw<P::planes, L::b_planes, kDwSum<P>, 24>(G.tcol + cW1, tc::smem_u32(G.a), L::a_bytes, 4u * 128u,
-                                                            tc::smem_u32(G.b), L::b_bytes, 3u * 128u, dw_acc);
-      });
-      if (!(alive = mma_phase_wait(G))) break;
-      dw_acc = true;
-      tc::tmem_ld16(lane_addr(G, cYb, warp_g), u);
+      if (!(alive = phase_wait(T))) break;
+      tc::tmem_ld16(tq + cX + 16 * half, v);
       tc::tmem_ld_wait();
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = a1[k] > 0.f ? v[k] : 0.f;  // dy1
+      tiles_free(T);
+      put_operand<P, 32, true, 8>(ta, tileA, row, 8 * half, v);
+      store_quarter<L::b_planes, 24, L::b_bytes>(tileB, row, l_lo, zl);
+      store_quarter<L::b_planes, 24, L::b_bytes>(tileB, row, l_hi, zh);
+      if (half != 0) store_chunk<L::b_planes, 24, L::b_bytes>(tileB, row, 2, one8);
+      // --- b1: dz = dy1 W1;  dW1, db1 (+)= dy1^T [z | 1] ---
+      phase_issue<P, 5>(T, tcol, sa, sw, dw_acc);
+      if (!(alive = phase_wait(T))) break;
+      dw_acc = true;
+      float4 gl4, gh4;  // dL/dz at this half's levels
+      {
+        float u[16];
+        tc::tmem_ld16(tq + cY, u);
+        tc::tmem_ld_wait();
+        gl4 = half == 0 ? make_float4(u[0], u[1], u[2], u[3]) : make_float4(u[4], u[5], u[6], u[7]);
+        gh4 = half == 0 ? make_float4(u[12], u[13], u[14], u[15]) : make_float4(u[8], u[9], u[10], u[11]);
+      }
+      if (!valid) gl4 = gh4 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (a.dz_out != nullptr && valid) {  // dL/dz of this sample (camera-pose gradients)
         float4* dzo = reinterpret_cast<float4*>(a.dz_out + ((size_t)rr * N + si) * kZ);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) dzo[q] = make_float4(u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+        dzo[l_lo] = gl4;
+        dzo[l_hi] = gh4;
       }
-      dw_wait(G);  // the tiles' space holds the scatter's staging rows
-      static_assert(L::a_bytes * P::planes + L::b_bytes * L::b_planes >= 4u * kScatterStage * 4u, "staging space");
-      int clj = clv[0];
-#pragma unroll
-      for (int q = 1; q < NCH; ++q)
-        if (q == j) clj = clv[q];
-      const float4* er = a.eik != nullptr && valid && clj == CLS_FS ? a.eik + (size_t)rr * N + si : nullptr;
-      scatter_dz<(P::planes == 1)>(a.g, a.grad, x, u, valid, reinterpret_cast<float*>(G.a) + warp_g * kScatterStage, er,
-                                   a.eik_stride);
-      group_sync(G.g);  // every warp is done with its rows before the tiles are rewritten
+      float x[3];
+      position(pick_tc(tt, j), x);
+      const float4* er = nullptr;
+      if (a.eik != nullptr && valid && a.cls[(size_t)rr * N + si] == CLS_FS) er = a.eik + (size_t)rr * N + si;
+      const EikSeed es = eik_seed(er, a.eik_stride);
+      scatter_direct<(P::planes == 1)>(a.g, a.grad, l_hi, x, gh4, valid, es);
+      tiles_free(T);  // their space holds the run reduction's staging rows
+      {
+        static_assert(L::runs == 8u * kScatterStage * 4u, "staging space");
+        float* st = reinterpret_cast<float*>(tileA) + w8 * kScatterStage;
+        scatter_runs(a.g, a.grad, l_lo, x, gl4, valid, st, es);
+      }
+      group_sync<kTileThreads>(gi);  // every warp is done with its rows before the tiles are rewritten
     }
   }
 
-  // ---- epilogue: loss and decoder-gradient partials, coarsest level, tensor memory ----
-  if (FWD) {
-    l_rgb = warp_sum(l_rgb);
-    l_d = warp_sum(l_d);
-    l_sdf = warp_sum(l_sdf);
-    l_fs = warp_sum(l_fs);
-    if (lane == 0) {
-      atomicAdd(lacc + 0, l_rgb);
-      atomicAdd(lacc + 1, l_d);
-      atomicAdd(lacc + 2, l_sdf);
-      atomicAdd(lacc + 3, l_fs);
-    }
-  }
+  // ---- epilogue: loss and decoder-gradient partials, tensor memory ----
+  tiles_free(T);
+  if (!alive && w8 == 0 && lane == 0) atomicOr(a.status, 2);
+
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
   if (BWD) {
-    g_kappa = warp_sum(g_kappa);
-    if (lane == 0) atomicAdd(acc + oKappa, g_kappa);
-    dw_wait(G);
-    if (alive && dw_acc && *reinterpret_cast<volatile int*>(G.abort) == 0) {
-      // the group's weight-gradient accumulators: warp w holds rows 16 w .. 16 w + 15 of every
-      // M = 64 product in its lanes 0..15 (rows 32.. are the bias rows or unused)
-      float d1[32], d2[32];
-      tc::tmem_ld32(lane_addr(G, cW1, warp_g), d1);  // cW1 .. cW1 + 31: dW1 (24) | dW2^T (first 8)
-      tc::tmem_ld32(lane_addr(G, cW1 + 32, warp_g), d2);  // dW2^T (last 8) | dW3 (16) | dW4^T (8)
+    // each group's decoder gradients as a row over its tiles
+    for (int i = tid; i < GR * kMlpPad; i += blockDim.x)
+      reinterpret_cast<float*>(gbase + (size_t)(i / kMlpPad) * L::group_bytes)[i % kMlpPad] = 0.f;
+    __syncthreads();
+    float* macc = reinterpret_cast<float*>(tileA);
+    if (half == 0 && dw_acc && *reinterpret_cast<volatile int*>(&T.bars->abort) == 0) {
+      // The weight-gradient accumulators: warp w holds rows 16 w .. 16 w + 15 of every M = 64
+      // product in its lanes 0..15.  Rows 32 .. 63 of dW1 and dW3 (16 .. 31 of dW2) are the
+      // adjoints' second parts; without one they mean nothing.
+      const bool mine = lane < 16 && (wq < 2 || P::planes > 1);
+      const int m = (16 * wq + lane) & 31;
+      float d[16];
+      tc::tmem_ld16(tq + cW1, d);
       tc::tmem_ld_wait();
-      const int m = 16 * warp_g + lane;  // D row held by this lane
-      if (lane < 16 && m < 32) {
+      if (mine) {
 #pragma unroll
-        for (int n = 0; n < 16; ++n) macc[oW1 + m * kZ + n] += d1[n];  // dW1[m][n]
-        macc[ob1 + m] += d1[16];                                       // db1[m]
-#pragma unroll
-        for (int n = 0; n < 16; ++n) macc[oW2 + n * kH1 + m] += (n < 8 ? d1[24 + n] : d2[n - 8]);  // dW2[n][m]
-#pragma unroll
-        for (int n = 0; n < 15; ++n) macc[oW3 + m * kHF + n] += d2[8 + n];  // dW3[m][n]
-        macc[ob3 + m] += d2[8 + 15];                                      // db3[m]
-      } else if (lane == 0 && m == 32) {  // bias row of the transposed product
-#pragma unroll
-        for (int n = 0; n < 16; ++n) macc[ob2 + n] += (n < 8 ? d1[24 + n] : d2[n - 8]);
+        for (int n = 0; n < 16; ++n) atomicAdd(macc + oW1 + m * kZ + n, d[n]);
       }
+      tc::tmem_ld16(tq + cW1 + 16, d);
+      tc::tmem_ld_wait();
+      if (mine) atomicAdd(macc + ob1 + m, d[0]);
+      tc::tmem_ld16(tq + cW3, d);
+      tc::tmem_ld_wait();
+      if (mine) {
+#pragma unroll
+        for (int n = 0; n < 15; ++n) atomicAdd(macc + oW3 + m * kHF + n, d[n]);
+        atomicAdd(macc + ob3 + m, d[15]);
+      }
+      const bool mine2 = lane < 16 && (wq == 0 || (wq == 1 && P::planes > 1));  // row lane: output unit
+      tc::tmem_ld16(tq + cW2, d);
+      tc::tmem_ld_wait();
+      if (mine2) {
+#pragma unroll
+        for (int n = 0; n < 16; ++n) atomicAdd(macc + oW2 + lane * kH1 + n, d[n]);
+      }
+      tc::tmem_ld16(tq + cW2 + 16, d);
+      tc::tmem_ld_wait();
+      if (mine2) {
+#pragma unroll
+        for (int n = 0; n < 16; ++n) atomicAdd(macc + oW2 + lane * kH1 + 16 + n, d[n]);
+      }
+      tc::tmem_ld16(tq + cW2 + 32, d);
+      tc::tmem_ld_wait();
+      if (mine2) atomicAdd(macc + ob2 + lane, d[0]);
     }
     // the colour layer's gradient, accumulated per warp on CUDA cores
 #pragma unroll
-    for (int n = 0; n < 3; ++n) atomicAdd(macc + oW4 + n * kH2 + lane, w4acc[n]);
-    if (lane < 3) atomicAdd(macc + ob4 + lane, b4acc);
+    for (int n = 0; n < 3; ++n) atomicAdd(macc + oW4 + n * kH2 + 16 * half + (lane & 15), w4acc[n]);
+    __syncthreads();
+  } else {
+    __syncthreads();
   }
-  if (!alive && gt == 0) {
-    atomicOr(a.status, 2);
-    tc::mbar_wait(G.mbar, G.phase ^ 1u, kMbarLimit);  // let an MMA in flight finish
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (tid < kLossPad) a.loss_part[(size_t)blockIdx.x * kLossPad + tid] = lacc[tid];
-  for (int i = tid; i < kMlpPad; i += blockDim.x) {
-    float v = acc[i];
+  auto total = [&](int k) {  // running sum k over the compositing warps
+    float v = 0.f;
 #pragma unroll
-    for (int q = 0; q < GR; ++q) v += gacc[q * kMlpPad + i];
+    for (int q = 0; q < GR * 4; ++q) v += sums0[q * kSums + k];
+    return v;
+  };
+  if (tid < kLossPad) a.loss_part[(size_t)blockIdx.x * kLossPad + tid] = tid < 4 ? total(tid) : 0.f;
+  for (int i = tid; i < kMlpPad; i += blockDim.x) {
+    float v = i == oKappa ? total(4) : (i >= ob4 && i < ob4 + kRGB ? total(5 + i - ob4) : 0.f);
+    if (BWD) {
+#pragma unroll
+      for (int q = 0; q < GR; ++q) v += reinterpret_cast<const float*>(gbase + (size_t)q * L::group_bytes)[i];
+    }
     a.mlp_part[(size_t)blockIdx.x * kMlpPad + i] = v;
   }
-  if (tid < 32) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(*tslot, tmem_cols(GR));
-  }
+  if (warp == 0) tc::tmem_dealloc(*tslot, tmem_cols(GR));
 }
 #pragma nv_diag_default 128
 
-template <class P, int GR>
-size_t render_tc_smem() {
+template <class P, int NCH, int GR>
+constexpr size_t render_tc_smem() {
   using L = TcLayout<P>;
-  size_t b = wTotal<P>() * P::planes + (kMlpPad + kLossPad + 88 + 96 + 4 + GR * kMlpPad) * 4;
-  b = (b + 1023) & ~size_t(1023);
-  return b + (size_t)GR * L::group_bytes + 1024;  // + alignment slack of the dynamic window
+  static_assert(kMlpPad * 4 <= L::bar_off, "a group's decoder-gradient row fits over its tiles");
+  return 128 + (size_t)GR * L::group_bytes + wTotal<P>() * P::planes + (size_t)GR * NCH * 128 * 16 +
+         GR * 20 * 16 + (GR * 4 * kSums + 88 + 96 + 8 + 4) * 4;
 }
 
 template <class P, int NCH, int GR, bool FWD, bool BWD>
 gs_status launch_tc_t(const gs_ctx* ctx, RenderTcArgs& a, cudaStream_t st) {
-  const size_t smem = render_tc_smem<P, GR>();
+  constexpr size_t smem = render_tc_smem<P, NCH, GR>();
+  static_assert(smem <= 227u * 1024u, "shared memory per CTA");
   auto k = render_tc_kernel<P, NCH, GR, FWD, BWD>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return GS_ERR_CUDA;
-  k<<<ctx->render_ctas, GR * kGroupThreads, smem, st>>>(a);
+  k<<<ctx->render_ctas, GR * kTileThreads, smem, st>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 template <class P, int NCH>
 gs_status launch_tc_n(const gs_ctx* ctx, RenderTcArgs& a, int mode, cudaStream_t st) {
-  // tile groups in one CTA per SM; rays of 5 chunks keep more per-ray state in registers,
-  // which only fits with 2 groups (255 registers per thread)
-  constexpr int GR = NCH > 4 ? 2 : kRenderGroups;
+  constexpr int GR = kRenderGroups;  // tile groups in one CTA per SM
   if (mode == 1) return launch_tc_t<P, NCH, GR, true, false>(ctx, a, st);
   if (mode == 2) return launch_tc_t<P, NCH, GR, false, true>(ctx, a, st);
   return launch_tc_t<P, NCH, GR, true, true>(ctx, a, st);
