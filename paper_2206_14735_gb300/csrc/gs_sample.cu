@@ -88,14 +88,19 @@ __global__ void __launch_bounds__(128) sample_smooth_kernel(SmoothArgs a) {
 }
 
 // One warp per ray, its samples over the lanes, and behind the rays' blocks one thread per
-// smoothness point.  A thread per ray drew and merged its 96 samples one after the other: 19 us at
-// 1024 rays and 26 us at 8192 x 96, 8 blocks or 64 on 152 SMs, whatever the batch; now 6 us at 8192 x 96.
+// smoothness point.  A thread per ray drew and merged its 96 samples one after the other on 8 blocks
+// or 64: 28.7 us a call at 1024 x 64 and 33.2 us at 8192 x 96 with 4096 points; now 12.3 and 16.5.  The
+// counts are summed over a block first: one atomic per warp and count was 24 us of atomics on four
+// words at 8192 rays.
 // The two sorted lists merge by rank: a stratified sample follows the guided ones below it, a
 // guided one the stratified ones up to it (ties stratified first), so a sample's place is its own
 // index plus one binary search in the other list.
-constexpr int kSampleWarps = 4;
+constexpr int kSampleWarps = 16;
 __global__ void __launch_bounds__(kSampleWarps * 32) sample_rays_kernel(SampleArgs a, SmoothArgs sm, int ray_blocks) {
   __shared__ float list[kSampleWarps][GS_MAX_SAMPLES];
+  __shared__ int found[3];
+  if (threadIdx.x < 3) found[threadIdx.x] = 0;
+  __syncthreads();
   if ((int)blockIdx.x >= ray_blocks) {
     sample_smooth_point(sm, ((int)blockIdx.x - ray_blocks) * blockDim.x + threadIdx.x);
     return;
@@ -161,7 +166,9 @@ __global__ void __launch_bounds__(kSampleWarps * 32) sample_rays_kernel(SampleAr
       }
     }
   }
-  block_add_counts(a.counts, nd, ntr, nfs);
+  block_add_counts(found, nd, ntr, nfs);
+  __syncthreads();
+  if (threadIdx.x < 3 && found[threadIdx.x]) atomicAdd(a.counts + threadIdx.x, found[threadIdx.x]);
 }
 
 }  // namespace gs
@@ -186,7 +193,7 @@ gs_status gs_launch_sample(const gs_ctx* ctx, const gs_frames* f, uint64_t seed,
   SampleArgs a{fr,     seed,   step,   b->R,   ctx->cfg.n_strat, ctx->cfg.n_guided, ctx->cfg.near_m,
                ctx->cfg.far_m, ctx->cfg.guide_half, ctx->cfg.trunc, (long long*)b->pix, b->origin, b->dir,
                b->rgb, b->depth, b->t, b->cls, b->counts};
-  const int ray_blocks = (b->R + kSampleWarps - 1) / kSampleWarps, blocks = ray_blocks + (b->P + 127) / 128;
+  const int ray_blocks = (b->R + kSampleWarps - 1) / kSampleWarps, blocks = ray_blocks + (b->P + kSampleWarps * 32 - 1) / (kSampleWarps * 32);
   if (blocks > 0) sample_rays_kernel<<<blocks, kSampleWarps * 32, 0, st>>>(a, smooth_args(ctx, f, seed, step, b), ray_blocks);
   return cudaPeekAtLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
