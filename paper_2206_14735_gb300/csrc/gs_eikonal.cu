@@ -70,7 +70,6 @@ struct EtMisc {
   float lsum[kEtGroups * 4];
   uint64_t mbar[kEtGroups];
   uint64_t mbar_dw[kEtGroups];
-  uint64_t mbar_unused;
   int abort[kEtGroups];
   uint32_t tslot;
   int last;
@@ -269,10 +268,9 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
   G.b = gb + oJ;
   G.mbar = &ms.mbar[gi];
   G.mbar_dw = &ms.mbar_dw[gi];
-  G.mbar_tma = &ms.mbar_unused;
   G.abort = &ms.abort[gi];
   G.tcol = ms.tslot + gi * kEtCols;
-  G.phase = G.phase_dw = G.phase_tma = 0;
+  G.phase = G.phase_dw = 0;
   G.dw_pending = false;
   G.g = gi;
   G.gt = threadIdx.x & (kGroupThreads - 1);
@@ -520,7 +518,6 @@ struct EpMisc {
   float lsum[kEpGroups * 4];
   uint64_t mbar[kEpGroups];
   uint64_t mbar_dw[kEpGroups];
-  uint64_t mbar_unused;
   int abort[kEpGroups];
   uint32_t tslot;
   int last;
@@ -574,10 +571,9 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
   G.b = gb + qPM;
   G.mbar = &ms.mbar[gi];
   G.mbar_dw = &ms.mbar_dw[gi];
-  G.mbar_tma = &ms.mbar_unused;
   G.abort = &ms.abort[gi];
   G.tcol = ms.tslot + gi * kEpCols;
-  G.phase = G.phase_dw = G.phase_tma = 0;
+  G.phase = G.phase_dw = 0;
   G.dw_pending = false;
   G.g = gi;
   G.gt = threadIdx.x & (kGroupThreads - 1);

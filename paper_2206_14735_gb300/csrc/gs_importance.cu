@@ -89,9 +89,8 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
   G.b = nullptr;
   G.mbar = &mbar[gi];
   G.mbar_dw = &mbar[gi];
-  G.mbar_tma = &mbar[gi];
   G.abort = &abort_flag[gi];
-  G.phase = G.phase_dw = G.phase_tma = 0;
+  G.phase = G.phase_dw = 0;
   G.dw_pending = false;
   G.g = gi;
   G.gt = threadIdx.x & (kGroupThreads - 1);

@@ -151,36 +151,6 @@ __global__ void voxel_index_kernel(GridDesc g, const float* __restrict__ xq, int
 
 using namespace gs;
 
-// cuTensorMapEncodeTiled from the driver (the library links only the runtime)
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// 2D view [nz * ny][nx * 4] of grid level l with a box of 2 vertices x 4 features, one row high
-bool gs::gs_encode_level_map(const gs_ctx* ctx, const float* theta, int l, CUtensorMap* m) {
-  EncodeTiledFn fn = encode_tiled();
-  if (!fn) return false;
-  const GridDesc& g = ctx->grid;
-  const cuuint64_t dims[2] = {(cuuint64_t)g.dims[l][0] * 4, (cuuint64_t)g.dims[l][1] * g.dims[l][2]};
-  const cuuint64_t strides[1] = {(cuuint64_t)g.dims[l][0] * 16};
-  const cuuint32_t box[2] = {8, 1};
-  const cuuint32_t es[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(theta + g.off[l]), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 static_assert(kStatusRender == 2, "render_tc_kernel reports a bounded wait that ran out as bit 1 (value 2)");
 
 gs_status gs_launch_render(const gs_ctx* ctx, const float* theta, const uint16_t* theta_bf16, const gs_batch* b,

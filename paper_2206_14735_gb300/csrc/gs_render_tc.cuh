@@ -30,7 +30,6 @@
 // 8192 x 132: 251, 223, 198 us.
 #pragma once
 #include "gs_internal.h"
-#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include "gs_tc.cuh"
@@ -86,7 +85,7 @@ __host__ __device__ constexpr uint32_t tmem_cols(int groups) {
 
 constexpr int kGroupThreads = 128;  // a tile group of one thread per tile row
 constexpr int kTileThreads = 256;   // the compact render kernel's tile group: two threads per tile row
-constexpr int kSums = 8;            // running sums of a compositing thread: 4 losses, kappa, db4
+constexpr int kSums = 9;            // running sums of a compositing warp: 4 losses, kappa, the colour and SDF seeds
 constexpr uint32_t kMbarLimit = 1u << 20;  // bounded MMA-completion wait (tries of up to 2 us: ~2 s)
 
 // Shared memory per tile group: adjoint tile | partner planes of the weight-gradient products (an
@@ -323,12 +322,10 @@ struct Group {
   uint8_t* b;  // partner planes of the weight-gradient products
   uint64_t* mbar;     // completion of the phase MMAs (issued by thread 0 of the group)
   uint64_t* mbar_dw;  // completion of the weight-gradient MMAs (issued by thread 32)
-  uint64_t* mbar_tma; // completion of the fine-level TMA gathers (armed by thread 0)
   int* abort;
   uint32_t tcol;      // tensor-memory address of this group's column 0
   uint32_t phase;     // parity of the next completion on mbar
   uint32_t phase_dw;  // ... on mbar_dw
-  uint32_t phase_tma; // ... on mbar_tma
   bool dw_pending;    // weight-gradient MMAs may still read the operand tiles
   int g, gt;
 };
@@ -515,29 +512,6 @@ __device__ __forceinline__ float4 fine_corners_sum(const FineCorners& q) {
   return s;
 }
 
-// host: the 2D view [nz ny][4 nx] of grid level l in theta, a box of 2 vertices x 4 features one
-// row high (the source of the paper architecture's tile::gather4 loads); false if the driver
-// refused it
-bool gs_encode_level_map(const gs_ctx* ctx, const float* theta, int l, CUtensorMap* m);
-// the other levels by plain loads (a warp's samples share the coarse cells)
-__device__ __forceinline__ void coarse_gather(const GridDesc& g, const float* __restrict__ theta, const float x[3],
-                                              float z[kZ]) {
-#pragma unroll
-  for (int l = 0; l < kLevels - 1; ++l) {
-    const Cell c = locate(g, l, x);
-    float w[8];
-    corner_weights(c.f, w);
-    const float4* base = reinterpret_cast<const float4*>(theta + g.off[l]);
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f4fma(s, w[k], __ldg(base + c.vtx + corner_offset(g, l, k)));
-    z[4 * l] = s.x;
-    z[4 * l + 1] = s.y;
-    z[4 * l + 2] = s.z;
-    z[4 * l + 3] = s.w;
-  }
-}
-
 // staging floats per warp of the run-reduced scatter: 32 rows of 36 floats, then the 32 keys
 constexpr int kScatterStage = 33 * 36;
 
@@ -716,29 +690,6 @@ __device__ __forceinline__ float pick_tc(const float (&arr)[N], int j) {
   return v;
 }
 
-// Stored activations come in groups of four fields, one float4 plane per group: field f of
-// sample s sits in component f % 4 of ((float4*)store)[(f / 4) * ss + s], so a warp's 32
-// consecutive samples read or write one 512-byte line per group.  sp points at sample s's
-// element of plane 0.
-template <int F0, int NF, int M>
-__device__ __forceinline__ void put_fields(float4* sp, long long ss, const float (&v)[M]) {
-  static_assert(F0 % 4 == 0 && NF % 4 == 0 && NF <= M, "whole groups of four fields");
-#pragma unroll
-  for (int q = 0; q < NF / 4; ++q) sp[(F0 / 4 + q) * ss] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-}
-template <int F0, int NF, int M>
-__device__ __forceinline__ void get_fields(const float4* sp, long long ss, bool get, float (&v)[M]) {
-  static_assert(F0 % 4 == 0 && NF % 4 == 0 && NF <= M, "whole groups of four fields");
-#pragma unroll
-  for (int q = 0; q < NF / 4; ++q) {
-    const float4 u = get ? sp[(F0 / 4 + q) * ss] : make_float4(0.f, 0.f, 0.f, 0.f);
-    v[4 * q] = u.x;
-    v[4 * q + 1] = u.y;
-    v[4 * q + 2] = u.z;
-    v[4 * q + 3] = u.w;
-  }
-}
-
 struct RenderTcArgs {
   GridDesc g;
   const float* theta;
@@ -793,6 +744,183 @@ __device__ __forceinline__ void get_planes(const StoreRef& s, int first, bool ge
     v[4 * q + 1] = u.y;
     v[4 * q + 2] = u.z;
     v[4 * q + 3] = u.w;
+  }
+}
+
+// NeuS compositing of one ray by one warp (lane = sample within the chunk), the losses of Sec.
+// 3.2-3.4 and, with BWD, the adjoint down to each sample's seeds: dL/d(colour pre-activations)
+// and dL/dphi into xch[128 j] of chunk j.  kc: the loss terms' scales (rgb, depth, sdf, fs) and
+// the sharpness; sums: the warp's running sums (kSums: the four losses, dL/dkappa, the seeds').
+template <int NCH, bool FWD, bool BWD, class Args>
+__device__ __forceinline__ void composite_ray(const Args& a, int ray, bool has_ray, const float (&tt)[NCH],
+                                              const float (&ph)[NCH], const float (&col)[NCH][3],
+                                              const int (&clv)[NCH], const float4& seen, const float* kc, float4* xch,
+                                              float* sums) {
+  const int lane = threadIdx.x & 31, N = a.N;
+  const float D = seen.w, I[3] = {seen.x, seen.y, seen.z}, s_sharp = kc[4];
+  float l_rgb = 0.f, l_d = 0.f, l_sdf = 0.f, l_fs = 0.f, g_kappa = 0.f, db4[3] = {0.f, 0.f, 0.f}, sum_d = 0.f;
+  // ================= NeuS opacity, transmittance, weights (Sec. 3.2) =================
+  float Ph[NCH], PhN[NCH], al[NCH], T[NCH], w[NCH];
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) Ph[j] = (has_ray && 32 * j + lane < N) ? sigmoidf_(s_sharp * ph[j]) : 0.f;
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+    float nx = __shfl_down_sync(0xffffffffu, Ph[j], 1);
+    const float nx0 = (j + 1 < NCH) ? __shfl_sync(0xffffffffu, Ph[j + 1 < NCH ? j + 1 : j], 0) : 0.f;
+    if (lane == 31) nx = nx0;
+    PhN[j] = nx;
+    float q = 0.f;
+    if (has_ray && 32 * j + lane < N - 1) q = (Ph[j] - nx) / fmaxf(Ph[j], 1e-6f);
+    al[j] = q > 0.f ? q : 0.f;
+  }
+  float carry = 1.0f;
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+    float inc = 1.0f - al[j];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float y = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc *= y;
+    }
+    float exc = __shfl_up_sync(0xffffffffu, inc, 1);
+    if (lane == 0) exc = 1.0f;
+    T[j] = carry * exc;
+    carry *= __shfl_sync(0xffffffffu, inc, 31);
+    w[j] = T[j] * al[j];
+  }
+  if (FWD && a.w_out != nullptr && has_ray) {
+#pragma unroll
+    for (int j = 0; j < NCH; ++j)
+      if (32 * j + lane < N) a.w_out[(size_t)ray * N + 32 * j + lane] = w[j];
+  }
+  float ch[3] = {0.f, 0.f, 0.f}, dh = 0.f, ws = 0.f;
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ch[k] = fmaf(w[j], col[j][k], ch[k]);
+    dh = fmaf(w[j], tt[j], dh);
+    ws += w[j];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) ch[k] = warp_sum(ch[k]);
+  dh = warp_sum(dh);
+  ws = warp_sum(ws);
+  if (FWD && has_ray) {
+    if (lane == 0) {
+      float e2 = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) e2 = fmaf(I[k] - ch[k], I[k] - ch[k], e2);
+      l_rgb += e2;
+      if (D > 0.f) l_d += fabsf(D - dh);
+      if (a.rgb_hat) {
+        a.rgb_hat[3 * ray] = ch[0];
+        a.rgb_hat[3 * ray + 1] = ch[1];
+        a.rgb_hat[3 * ray + 2] = ch[2];
+      }
+      if (a.d_hat) a.d_hat[ray] = dh;
+      if (a.wsum) a.wsum[ray] = ws;
+    }
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+      const int si = 32 * j + lane;
+      if (si >= N) continue;
+      const int cl = clv[j];
+      const float b = __fsub_rn(D, tt[j]);
+      if (cl == CLS_TR) l_sdf += fabsf(ph[j] - b);
+      else if (cl == CLS_FS) l_fs += fmaxf(fmaxf(0.f, expf(-a.kappa_fs * ph[j]) - 1.0f), ph[j] - b);
+    }
+  }
+  if constexpr (BWD) {
+
+  // ================= adjoint of compositing: dL/dalpha_k = T_k (e_k - U_k) =================
+  float gc[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) gc[k] = has_ray ? kc[0] * (ch[k] - I[k]) : 0.f;
+  const float gd = (has_ray && D > 0.f) ? kc[1] * ((dh > D) ? 1.f : (dh < D ? -1.f : 0.f)) : 0.f;
+  float e[NCH], U[NCH];
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) e[j] = gc[0] * col[j][0] + gc[1] * col[j][1] + gc[2] * col[j][2] + gd * tt[j];
+  float cA = 0.f;
+#pragma unroll
+  for (int j = NCH - 1; j >= 0; --j) {
+    float A = al[j] * e[j], B = 1.0f - al[j];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float A2 = __shfl_down_sync(0xffffffffu, A, off), B2 = __shfl_down_sync(0xffffffffu, B, off);
+      if (lane + off < 32) {
+        A = fmaf(B, A2, A);
+        B *= B2;
+      }
+    }
+    float eA = __shfl_down_sync(0xffffffffu, A, 1), eB = __shfl_down_sync(0xffffffffu, B, 1);
+    if (lane == 31) {
+      eA = 0.f;
+      eB = 1.f;
+    }
+    U[j] = fmaf(eB, cA, eA);
+    const float A0 = __shfl_sync(0xffffffffu, A, 0), B0 = __shfl_sync(0xffffffffu, B, 0);
+    cA = fmaf(B0, cA, A0);
+  }
+  float dnext_prev = 0.f;
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+    const int si = 32 * j + lane;
+    const bool valid = has_ray && si < N;
+    const float dal = T[j] * (e[j] - U[j]);
+    float dself = 0.f, dnext = 0.f;
+    if (valid && si < N - 1) {
+      const float den = fmaxf(Ph[j], 1e-6f);
+      if (Ph[j] - PhN[j] > 0.f) {
+        dnext = -dal / den;
+        dself = (Ph[j] > 1e-6f) ? dal * PhN[j] / (Ph[j] * Ph[j]) : dal * 1e6f;
+      }
+    }
+    float recv = __shfl_up_sync(0xffffffffu, dnext, 1);
+    const float last = __shfl_sync(0xffffffffu, dnext, 31);
+    if (lane == 0) recv = dnext_prev;
+    dnext_prev = last;
+    const float dPh = dself + recv;
+    const float dsig = Ph[j] * (1.0f - Ph[j]);
+    float d = dPh * s_sharp * dsig;
+    if (valid) {
+      g_kappa = fmaf(dPh * dsig * s_sharp, ph[j], g_kappa);
+      const int cl = clv[j];
+      const float b = __fsub_rn(D, tt[j]);
+      if (cl == CLS_TR) {
+        const float df = ph[j] - b;
+        d += kc[2] * (df > 0.f ? 1.f : (df < 0.f ? -1.f : 0.f));
+      } else if (cl == CLS_FS) {
+        const float ex = expf(-a.kappa_fs * ph[j]) - 1.0f, lin = ph[j] - b;
+        int arg = 0;
+        float top = 0.f;
+        if (ex > top) {
+          top = ex;
+          arg = 1;
+        }
+        if (lin > top) arg = 2;
+        d += kc[3] * (arg == 1 ? -a.kappa_fs * (ex + 1.0f) : (arg == 2 ? 1.0f : 0.0f));
+      }
+    } else {
+      d = 0.f;
+    }
+    // the reverse pass's seeds of the sample: the colour pre-activations' (w gc c (1 - c)) and phi's
+    float dp[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dp[k] = valid ? w[j] * gc[k] * col[j][k] * (1.0f - col[j][k]) : 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) db4[k] += dp[k];
+    xch[j * 128] = make_float4(dp[0], dp[1], dp[2], d);
+    sum_d += d;
+  }
+  }  // BWD
+  {
+    float q[kSums] = {l_rgb, l_d, l_sdf, l_fs, g_kappa, db4[0], db4[1], db4[2], sum_d};
+#pragma unroll
+    for (int k = 0; k < kSums; ++k) q[k] = warp_sum(q[k]);
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < kSums; ++k) sums[k] += q[k];
+    }
   }
 }
 
@@ -1068,172 +1196,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       }
     }
     const float4 in4 = *tint;
-    const float D = in4.w, I[3] = {in4.x, in4.y, in4.z}, s_sharp = kc[4];
-    float l_rgb = 0.f, l_d = 0.f, l_sdf = 0.f, l_fs = 0.f, g_kappa = 0.f, db4[3] = {0.f, 0.f, 0.f};
-
-    // ================= NeuS opacity, transmittance, weights (Sec. 3.2) =================
-    float Ph[NCH], PhN[NCH], al[NCH], T[NCH], w[NCH];
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) Ph[j] = (has_ray && 32 * j + lane < N) ? sigmoidf_(s_sharp * ph[j]) : 0.f;
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      float nx = __shfl_down_sync(0xffffffffu, Ph[j], 1);
-      const float nx0 = (j + 1 < NCH) ? __shfl_sync(0xffffffffu, Ph[j + 1 < NCH ? j + 1 : j], 0) : 0.f;
-      if (lane == 31) nx = nx0;
-      PhN[j] = nx;
-      float q = 0.f;
-      if (has_ray && 32 * j + lane < N - 1) q = (Ph[j] - nx) / fmaxf(Ph[j], 1e-6f);
-      al[j] = q > 0.f ? q : 0.f;
-    }
-    float carry = 1.0f;
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      float inc = 1.0f - al[j];
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, inc, off);
-        if (lane >= off) inc *= y;
-      }
-      float exc = __shfl_up_sync(0xffffffffu, inc, 1);
-      if (lane == 0) exc = 1.0f;
-      T[j] = carry * exc;
-      carry *= __shfl_sync(0xffffffffu, inc, 31);
-      w[j] = T[j] * al[j];
-    }
-    if (FWD && a.w_out != nullptr && has_ray) {
-#pragma unroll
-      for (int j = 0; j < NCH; ++j)
-        if (32 * j + lane < N) a.w_out[(size_t)ray * N + 32 * j + lane] = w[j];
-    }
-    float ch[3] = {0.f, 0.f, 0.f}, dh = 0.f, ws = 0.f;
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) ch[k] = fmaf(w[j], col[j][k], ch[k]);
-      dh = fmaf(w[j], tt[j], dh);
-      ws += w[j];
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) ch[k] = warp_sum(ch[k]);
-    dh = warp_sum(dh);
-    ws = warp_sum(ws);
-    if (FWD && has_ray) {
-      if (lane == 0) {
-        float e2 = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) e2 = fmaf(I[k] - ch[k], I[k] - ch[k], e2);
-        l_rgb += e2;
-        if (D > 0.f) l_d += fabsf(D - dh);
-        if (a.rgb_hat) {
-          a.rgb_hat[3 * ray] = ch[0];
-          a.rgb_hat[3 * ray + 1] = ch[1];
-          a.rgb_hat[3 * ray + 2] = ch[2];
-        }
-        if (a.d_hat) a.d_hat[ray] = dh;
-        if (a.wsum) a.wsum[ray] = ws;
-      }
-#pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const int si = 32 * j + lane;
-        if (si >= N) continue;
-        const int cl = clv[j];
-        const float b = __fsub_rn(D, tt[j]);
-        if (cl == CLS_TR) l_sdf += fabsf(ph[j] - b);
-        else if (cl == CLS_FS) l_fs += fmaxf(fmaxf(0.f, expf(-a.kappa_fs * ph[j]) - 1.0f), ph[j] - b);
-      }
-    }
-    if constexpr (BWD) {
-
-    // ================= adjoint of compositing: dL/dalpha_k = T_k (e_k - U_k) =================
-    float gc[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) gc[k] = has_ray ? kc[0] * (ch[k] - I[k]) : 0.f;
-    const float gd = (has_ray && D > 0.f) ? kc[1] * ((dh > D) ? 1.f : (dh < D ? -1.f : 0.f)) : 0.f;
-    float e[NCH], U[NCH];
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) e[j] = gc[0] * col[j][0] + gc[1] * col[j][1] + gc[2] * col[j][2] + gd * tt[j];
-    float cA = 0.f;
-#pragma unroll
-    for (int j = NCH - 1; j >= 0; --j) {
-      float A = al[j] * e[j], B = 1.0f - al[j];
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const float A2 = __shfl_down_sync(0xffffffffu, A, off), B2 = __shfl_down_sync(0xffffffffu, B, off);
-        if (lane + off < 32) {
-          A = fmaf(B, A2, A);
-          B *= B2;
-        }
-      }
-      float eA = __shfl_down_sync(0xffffffffu, A, 1), eB = __shfl_down_sync(0xffffffffu, B, 1);
-      if (lane == 31) {
-        eA = 0.f;
-        eB = 1.f;
-      }
-      U[j] = fmaf(eB, cA, eA);
-      const float A0 = __shfl_sync(0xffffffffu, A, 0), B0 = __shfl_sync(0xffffffffu, B, 0);
-      cA = fmaf(B0, cA, A0);
-    }
-    float dnext_prev = 0.f;
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      const int si = 32 * j + lane;
-      const bool valid = has_ray && si < N;
-      const float dal = T[j] * (e[j] - U[j]);
-      float dself = 0.f, dnext = 0.f;
-      if (valid && si < N - 1) {
-        const float den = fmaxf(Ph[j], 1e-6f);
-        if (Ph[j] - PhN[j] > 0.f) {
-          dnext = -dal / den;
-          dself = (Ph[j] > 1e-6f) ? dal * PhN[j] / (Ph[j] * Ph[j]) : dal * 1e6f;
-        }
-      }
-      float recv = __shfl_up_sync(0xffffffffu, dnext, 1);
-      const float last = __shfl_sync(0xffffffffu, dnext, 31);
-      if (lane == 0) recv = dnext_prev;
-      dnext_prev = last;
-      const float dPh = dself + recv;
-      const float dsig = Ph[j] * (1.0f - Ph[j]);
-      float d = dPh * s_sharp * dsig;
-      if (valid) {
-        g_kappa = fmaf(dPh * dsig * s_sharp, ph[j], g_kappa);
-        const int cl = clv[j];
-        const float b = __fsub_rn(D, tt[j]);
-        if (cl == CLS_TR) {
-          const float df = ph[j] - b;
-          d += kc[2] * (df > 0.f ? 1.f : (df < 0.f ? -1.f : 0.f));
-        } else if (cl == CLS_FS) {
-          const float ex = expf(-a.kappa_fs * ph[j]) - 1.0f, lin = ph[j] - b;
-          int arg = 0;
-          float top = 0.f;
-          if (ex > top) {
-            top = ex;
-            arg = 1;
-          }
-          if (lin > top) arg = 2;
-          d += kc[3] * (arg == 1 ? -a.kappa_fs * (ex + 1.0f) : (arg == 2 ? 1.0f : 0.0f));
-        }
-      } else {
-        d = 0.f;
-      }
-      // the reverse pass's seeds of the sample: the colour pre-activations' (w gc c (1 - c)) and phi's
-      float dp[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) dp[k] = valid ? w[j] * gc[k] * col[j][k] * (1.0f - col[j][k]) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) db4[k] += dp[k];
-      xch[j * 128 + row] = make_float4(dp[0], dp[1], dp[2], d);
-    }
-    }  // BWD
-    {
-      float q[kSums] = {l_rgb, l_d, l_sdf, l_fs, g_kappa, db4[0], db4[1], db4[2]};
-#pragma unroll
-      for (int k = 0; k < kSums; ++k) q[k] = warp_sum(q[k]);
-      if (lane == 0) {
-        float* sm = sums0 + (gi * 4 + wq) * kSums;
-#pragma unroll
-        for (int k = 0; k < kSums; ++k) sm[k] += q[k];
-      }
-    }
+    composite_ray<NCH, FWD, BWD>(a, ray, has_ray, tt, ph, col, clv, in4, kc, xch + row, sums0 + (gi * 4 + wq) * kSums);
     }  // lower half
     if constexpr (!BWD) continue;
     group_sync<kTileThreads>(gi);  // the reverse pass's seeds

@@ -70,14 +70,6 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ---- MMA issue (single thread) --------------------------------------------------------
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
@@ -122,19 +114,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* mbar, uint32_t parity, u
       : "memory");
   return ok != 0;
 }
-// one look at the barrier, without suspending
-__device__ __forceinline__ bool mbar_test(uint64_t* mbar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(mbar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
-}
 // bounded wait: false after `limit` tries of up to 2 us each (the caller records an error and leaves)
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint32_t limit) {
   for (uint32_t i = 0; i < limit; ++i)
@@ -142,24 +121,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint3
   return false;
 }
 
-// arrival of the calling thread that also announces `bytes` of asynchronous copies on this phase
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* mbar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes) : "memory");
-}
-// mbarrier initialisation visible to the asynchronous (TMA) proxy
+// mbarrier initialisation visible to the asynchronous proxy
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-// ---- TMA ----------------------------------------------------------------------------------
-// 4 rows (row0..row3) x the tensor map's box width, starting at column `col` (a multiple of
-// 16 bytes), from a 2D tensor map into 4 consecutive box rows at `dst`; completes `bytes` on mbar
-__device__ __forceinline__ void tma_gather4(uint32_t dst, const void* tmap, int col, int row0, int row1, int row2,
-                                            int row3, uint64_t* mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
-      "%4, %5, %6}], [%7];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(col), "r"(row0), "r"(row1), "r"(row2), "r"(row3), "r"(smem_u32(mbar))
-      : "memory");
-}
 
 // ---- tensor memory -> registers: warp reads its 32 lanes, 16 / 32 consecutive columns ----
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
@@ -201,13 +164,6 @@ __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&r)[8]) 
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// binary32 -> tf32 (round to nearest, ties away), kept in a 32-bit container
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
 
 }  // namespace tc
 }  // namespace gs
