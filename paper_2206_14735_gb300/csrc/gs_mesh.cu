@@ -4,7 +4,7 @@
 // closed surface wherever the lattice values do).
 //
 // lattice_sdf_pair_kernel / lattice_sdf_paper_kernel: phi at lo + (i, j, k) * step (binary32
-// positions, FP32 SDF) with the workload's decoder (two points per thread, packed FMAs) or the
+// positions, FP32 SDF) with the workload's decoder (two points per thread) or the
 // paper's.
 // mesh_kernel: one thread per cell; a tetrahedron with 1 or 3 corners below iso gives one
 // triangle, with 2 below two; each vertex is interpolated along its tetrahedron edge from the
@@ -68,71 +68,63 @@ __global__ void __launch_bounds__(128) lattice_sdf_paper_kernel(LatticeArgs a) {
   }
 }
 
-// packed pair of FP32 values: element 0 in the low half
-__device__ __forceinline__ unsigned long long pk2(float lo, float hi) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(unsigned long long r, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
-}
-// both halves: d = a * b + c, each an IEEE fma rounded to nearest, as fmaf
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-
-// The workload's decoder: two neighbouring lattice points per thread, their features side by
-// side in packed pairs; every weight is kept twice in shared memory so that one 128-bit
-// broadcast read gives two packed weight pairs and one packed FMA advances both points.  Per
-// point the operations and their order are sdf_at's, so phi is the same to the bit.
-struct LatticePairDecoder {
-  unsigned long long W1[kH1][kZ];  // (W1[j][k], W1[j][k])
-  unsigned long long bw[kH1][2];   // (b1[j], b1[j]), (W2[0][j], W2[0][j])
-  unsigned long long b2;           // (b2[0], b2[0])
+// The workload's decoder: two neighbouring lattice points per thread.  The pass is bound by the L1 /
+// shared-memory data path, most of it the decoder's weights (a 128-bit read takes four cycles of
+// it, broadcast or not): the weights lie transposed, so that one read gives four units' weights of
+// one input, for both points.  Stored twice, as packed pairs for one packed FMA per weight and
+// pair of points, they took twice the reads: 1227 us for the 18 M points and the triangles of the
+// room at 2 cm, now 1068.  Taking the second point's corners from the first one's where their cells
+// meet saved a third of the corner loads and measured slower (1135 us: registers, and the selects).
+// Per point the operations and their order are sdf_at's, so phi is the same to the bit.
+struct LatticeDecoder {
+  float W1t[kZ][kH1];  // W1t[k][j] = W1[j][k]
+  float b1[kH1], w2[kH1], b2;
 };
 
-__global__ void __launch_bounds__(128) lattice_sdf_pair_kernel(LatticeArgs a) {
-  __shared__ __align__(16) LatticePairDecoder d;
+__global__ void __launch_bounds__(128, 4) lattice_sdf_pair_kernel(LatticeArgs a) {
+  __shared__ __align__(16) LatticeDecoder d;
   const float* mlp = a.theta + a.g.n_grid;
-  for (int i = threadIdx.x; i < kH1 * kZ; i += blockDim.x) {
-    const float v = mlp[oW1 + i];
-    d.W1[i / kZ][i % kZ] = pk2(v, v);
-  }
+  for (int i = threadIdx.x; i < kH1 * kZ; i += blockDim.x) d.W1t[i % kZ][i / kZ] = mlp[oW1 + i];
   for (int j = threadIdx.x; j < kH1; j += blockDim.x) {
-    d.bw[j][0] = pk2(mlp[ob1 + j], mlp[ob1 + j]);
-    d.bw[j][1] = pk2(mlp[oW2 + j], mlp[oW2 + j]);
+    d.b1[j] = mlp[ob1 + j];
+    d.w2[j] = mlp[oW2 + j];
   }
-  if (threadIdx.x == 0) d.b2 = pk2(mlp[ob2], mlp[ob2]);
+  if (threadIdx.x == 0) d.b2 = mlp[ob2];
   __syncthreads();
   const long long np = (long long)a.nx * a.ny * a.nz, npair = (np + 1) / 2;
   const bool narrow = np <= 0xffffffffLL;
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npair; p += (long long)gridDim.x * blockDim.x) {
     const long long id0 = 2 * p, id1 = id0 + 1 < np ? id0 + 1 : id0;  // an odd count repeats the last point
-    unsigned long long zz[kZ];
+    float z0[kZ], z1[kZ];
     {
-      float x[3], z0[kZ], z1[kZ];
-      lattice_x(a, id0, narrow, x);
-      grid_z(a.g, a.theta, x, z0);
-      lattice_x(a, id1, narrow, x);
-      grid_z(a.g, a.theta, x, z1);
-#pragma unroll
-      for (int k = 0; k < kZ; ++k) zz[k] = pk2(z0[k], z1[k]);
+      float x0[3], x1[3];
+      lattice_x(a, id0, narrow, x0);
+      lattice_x(a, id1, narrow, x1);
+      grid_z(a.g, a.theta, x0, z0);
+      grid_z(a.g, a.theta, x1, z1);
     }
-    unsigned long long phi = d.b2;
-#pragma unroll 4
-    for (int j = 0; j < kH1; ++j) {
-      unsigned long long s = d.bw[j][0];
+    float phi0 = d.b2, phi1 = phi0;
+#pragma unroll 1
+    for (int j = 0; j < kH1; j += 8) {  // eight units at a time
+      float s0[8], s1[8];
 #pragma unroll
-      for (int k = 0; k < kZ; ++k) s = ffma2(d.W1[j][k], zz[k], s);
-      float s0, s1;
-      upk2(s, s0, s1);
-      phi = ffma2(d.bw[j][1], pk2(fmaxf(s0, 0.f), fmaxf(s1, 0.f)), phi);
+      for (int q = 0; q < 8; ++q) s0[q] = s1[q] = d.b1[j + q];
+#pragma unroll
+      for (int k = 0; k < kZ; ++k) {
+        const float4 wa = *reinterpret_cast<const float4*>(&d.W1t[k][j]), wb = *reinterpret_cast<const float4*>(&d.W1t[k][j + 4]);
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          s0[q] = fmaf(w[q], z0[k], s0[q]);
+          s1[q] = fmaf(w[q], z1[k], s1[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        phi0 = fmaf(d.w2[j + q], fmaxf(s0[q], 0.f), phi0);
+        phi1 = fmaf(d.w2[j + q], fmaxf(s1[q], 0.f), phi1);
+      }
     }
-    float phi0, phi1;
-    upk2(phi, phi0, phi1);
     a.phi[id0] = phi0;
     if (id1 != id0) a.phi[id1] = phi1;
   }
@@ -220,6 +212,7 @@ __global__ void __launch_bounds__(128) mesh_kernel(MeshArgs a) {
         cnt += (ni == 0 || ni == 4) ? 0 : (ni == 2 ? 2 : 1);
       }
     }
+    if (!__any_sync(0xffffffffu, cnt > 0)) continue;  // no surface in the warp's cells: most warps
     int incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
