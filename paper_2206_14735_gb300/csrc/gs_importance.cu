@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
     atomicOr(status, kStatusImportance);
     tc::mbar_wait(G.mbar, G.phase ^ 1u, kItMbarLimit);  // let an MMA in flight finish
   }
-  block_add_counts(a.counts, nd, ntr, nfs);
+  add_counts_per_block(a.counts, nd, ntr, nfs);
   tc::fence_before_sync();
   __syncthreads();
   if (threadIdx.x < 32) {

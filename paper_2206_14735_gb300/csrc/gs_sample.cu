@@ -98,9 +98,6 @@ __global__ void __launch_bounds__(128) sample_smooth_kernel(SmoothArgs a) {
 constexpr int kSampleWarps = 16;
 __global__ void __launch_bounds__(kSampleWarps * 32) sample_rays_kernel(SampleArgs a, SmoothArgs sm, int ray_blocks) {
   __shared__ float list[kSampleWarps][GS_MAX_SAMPLES];
-  __shared__ int found[3];
-  if (threadIdx.x < 3) found[threadIdx.x] = 0;
-  __syncthreads();
   if ((int)blockIdx.x >= ray_blocks) {
     sample_smooth_point(sm, ((int)blockIdx.x - ray_blocks) * blockDim.x + threadIdx.x);
     return;
@@ -166,9 +163,7 @@ __global__ void __launch_bounds__(kSampleWarps * 32) sample_rays_kernel(SampleAr
       }
     }
   }
-  block_add_counts(found, nd, ntr, nfs);
-  __syncthreads();
-  if (threadIdx.x < 3 && found[threadIdx.x]) atomicAdd(a.counts + threadIdx.x, found[threadIdx.x]);
+  add_counts_per_block(a.counts, nd, ntr, nfs);
 }
 
 }  // namespace gs

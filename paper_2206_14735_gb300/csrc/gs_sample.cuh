@@ -51,4 +51,15 @@ __device__ __forceinline__ void block_add_counts(int* counts, int a, int b, int 
   }
 }
 
+// the same summed over the block first (every thread of the block calls it): the words take their
+// atomics one after the other
+__device__ __forceinline__ void add_counts_per_block(int* counts, int a, int b, int c) {
+  __shared__ int sum[3];
+  if (threadIdx.x < 3) sum[threadIdx.x] = 0;
+  __syncthreads();
+  block_add_counts(sum, a, b, c);
+  __syncthreads();
+  if (threadIdx.x < 3 && sum[threadIdx.x]) atomicAdd(counts + threadIdx.x, sum[threadIdx.x]);
+}
+
 }  // namespace gs
