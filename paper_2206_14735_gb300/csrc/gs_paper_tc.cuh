@@ -26,7 +26,8 @@
 // deferred Eikonal records of the free-space samples), the colour grid (6 floats per finest-level
 // vertex) with one 16-byte and one 8-byte reduction per corner; samples whose vectors are exactly
 // zero issue none.  With one thread per row for both decoders the SM held 8 warps at 255 registers;
-// 8192 x 96, stored: 974 us a call, now 854 (recomputed 1160 -> 1047).
+// 8192 x 96, stored: 974 us a call, then 854; with the operands in tensor memory 828 (recomputed
+// 1160, 1047, 976).
 #pragma once
 #include "gs_paper.cuh"
 #include "gs_render_tc.cuh"
@@ -60,12 +61,14 @@ constexpr uint32_t kAP = 128u * 32u * 2u;  // one part of an A tile
 constexpr uint32_t kBPg = 128u * 32u * 2u, kBP = 128u * 40u * 2u;  // one part of a partner tile
 constexpr uint32_t oAg = 0, oAc = 3 * kAP, oBg = 6 * kAP, oBc = oBg + 2 * kBPg, oBar = oBc + 2 * kBP;
 constexpr uint32_t kPGroupBytes = oBar + 128;
-constexpr int kPGroups = 2;  // tensor memory: 2 groups x 192 columns
+constexpr int kPGroups = 2;  // tensor memory: 2 groups x 256 columns
 constexpr int kPThreads = kPGroups * kTileThreads;
 
-// tensor-memory columns of a group: phase outputs (geometry, colour), then the weight-gradient
-// accumulators (M = 64 layout: row m in lane 32 (m / 16) + m % 16)
-constexpr uint32_t cG = 0, cC = 32, cWg2 = 64, cWc2 = 96, cWg1 = 128, cWc1 = 160, kPCols = 192;
+// tensor-memory columns of a group: phase outputs (geometry, colour), the weight-gradient
+// accumulators (M = 64 layout: row m in lane 32 (m / 16) + m % 16), then the two leading parts of the
+// phases' A operands (part p of a K-column row in columns p K / 2 ..; the third part, read by one
+// product of six, has no columns left and stays in the A tile)
+constexpr uint32_t cG = 0, cC = 32, cWg2 = 64, cWc2 = 96, cWg1 = 128, cWc1 = 160, cAg = 192, cAc = 224, kPCols = 256;
 constexpr uint32_t kPTmem = 512;
 static_assert(kPGroups * kPCols <= kPTmem, "tensor-memory columns");
 
@@ -163,6 +166,7 @@ __device__ __forceinline__ void scatter_colour(const PaperTcArgs& a, const float
 // tiles (two commits to the dw barrier; the tiles are rewritten only after them)
 template <bool DW, class F, class Fg, class Fc>
 __device__ __forceinline__ void phase2(Tile& T, F mma, Fg dwg, Fc dwc) {
+  tc::tmem_st_wait();
   tc::fence_smem_async();
   tc::fence_before_sync();
   group_sync<kTileThreads>(T.g);
@@ -184,11 +188,54 @@ __device__ __forceinline__ void phase2(Tile& T, F mma, Fg dwg, Fc dwc) {
   if (DW) T.dw_pending = true;
 }
 
-// D[128][N] = A[128][K] B[N][K]^T over the six leading part products (A parts kAP apart,
-// B parts kTW apart)
+// D[128][N] = A[128][K] B[N][K]^T over the six leading part products, smallest first: A's parts 0
+// and 1 from tensor memory (ta), part 2 from the A tile at a0, B's parts kTW apart
 template <int N, int K>
-__device__ __forceinline__ void mma3(uint32_t d, uint32_t a0, uint32_t b0) {
-  issue_mma<P3, N, K>(d, a0, b0, kTW);
+__device__ __forceinline__ void mma3(uint32_t d, uint32_t ta, uint32_t a0, uint32_t b0) {
+  constexpr uint32_t sbo = K * 16u, idesc = tc::instr_desc(tc::KIND_BF16, 128, N);
+  const uint32_t alo = tc::desc_lo(a0 + 2 * kAP, 128u), blo = tc::desc_lo(b0, 128u);
+  bool first = true;
+#pragma unroll
+  for (int s = 0; s < K / 16; ++s) {
+    const uint32_t off = (uint32_t)s * 256u;
+#pragma unroll
+    for (int sum = 2; sum >= 0; --sum)
+#pragma unroll
+      for (int i = 0; i <= sum; ++i) {
+        const uint64_t bd = tc::desc_of(blo + (((sum - i) * kTW + off) >> 4), tc::desc_hi(sbo));
+        if (i < 2) tc::mma_bf16_ta(d, ta + (uint32_t)(i * (K / 2) + s * 8), bd, idesc, first ? 0u : 1u);
+        else tc::mma_bf16(d, tc::desc_of(alo + (off >> 4), tc::desc_hi(sbo)), bd, idesc, first ? 0u : 1u);
+        first = false;
+      }
+  }
+}
+// 2 W values of a K-column operand row from column 2 w0 on: parts 0 and 1 into tensor memory and,
+// for the weight-gradient products (DW), the A tile; part 2 into the A tile
+template <int K, bool DW, int W>
+__device__ __forceinline__ void put_row(uint32_t ta, uint8_t* tile, int row, int w0, const float* v) {
+  uint32_t w[3][W];
+  split_words<3, W>(v, w);
+  tc::tmem_st(ta + (uint32_t)w0, w[0]);
+  tc::tmem_st(ta + (uint32_t)(K / 2 + w0), w[1]);
+#pragma unroll
+  for (int pl = DW ? 0 : 2; pl < 3; ++pl) {
+    uint8_t* t = tile + pl * kAP;
+    if constexpr (W >= 4) {
+#pragma unroll
+      for (int c = 0; c < W / 4; ++c)
+        *reinterpret_cast<uint4*>(t + tc::core_offset((uint32_t)row, (uint32_t)(w0 / 4 + c), 128u, K * 16u)) =
+            make_uint4(w[pl][4 * c], w[pl][4 * c + 1], w[pl][4 * c + 2], w[pl][4 * c + 3]);
+    } else {
+      *reinterpret_cast<uint2*>(t + tc::core_offset((uint32_t)row, (uint32_t)(w0 / 4), 128u, K * 16u) + (uint32_t)(w0 & 3) * 4u) =
+          make_uint2(w[pl][0], w[pl][1]);
+    }
+  }
+}
+// a whole row
+template <int K, bool DW>
+__device__ __forceinline__ void put_rows(uint32_t ta, uint8_t* tile, int row, const float* v) {
+#pragma unroll
+  for (int c = 0; c < K / 16; ++c) put_row<K, DW, 8>(ta, tile, row, 8 * c, v + 16 * c);
 }
 
 // the forward-only instantiation ends each ray-quad before its reverse pass, which the front
@@ -279,7 +326,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
   tc::fence_after_sync();
   const uint32_t tcol = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(gi * kPCols);
   const uint32_t tq = tcol + ((uint32_t)(32 * wq) << 16);      // this warp's lanes
-  const uint32_t tx = tq + (half ? cC : cG);                   // and its decoder's phase output
+  const uint32_t tx = tq + (half ? cC : cG), ta = tq + (half ? cAc : cAg);  // its decoder's phase output and operand
   const uint32_t sg = tc::smem_u32(base) + (uint32_t)gi * kPGroupBytes, sw = tc::smem_u32(wt);
   const float* hb1 = sc + (half ? sc_cb1 : sc_gb1);
   const float* hb2 = sc + (half ? sc_cb2 : sc_gb2);
@@ -330,23 +377,25 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
       }
     }
     tiles_free(T);
+    __syncwarp();
     if (half == 0) {
-      store_quarter<3, 16, kAP>(tileA, row, 0, make_float4(u[0], u[1], u[2], u[3]));
-      store_chunk<3, 16, kAP>(tileA, row, 1, u + 8);
+      put_row<16, false, 2>(ta, tileA, row, 0, u);
+      put_row<16, false, 4>(ta, tileA, row, 4, u + 8);
     } else {
       view_inputs(u);
-      store_row_planes<3, 16, kAP>(tileA, row, u);
-      store_quarter<3, 16, kAP>(gmem + oAg, row, 1, z1);
+      put_rows<16, false>(ta, tileA, row, u);
+      const float q1[4] = {z1.x, z1.y, z1.z, z1.w};
+      put_row<16, false, 2>(tq + cAg, gmem + oAg, row, 2, q1);
     }
   };
   auto nop = [] {};
   auto f1 = [&] {
-    mma3<32, 16>(tcol + cG, sg + oAg, sw + tOff(0));
-    mma3<32, 16>(tcol + cC, sg + oAc, sw + tOff(1));
+    mma3<32, 16>(tcol + cG, tcol + cAg, sg + oAg, sw + tOff(0));
+    mma3<32, 16>(tcol + cC, tcol + cAc, sg + oAc, sw + tOff(1));
   };
   auto f2 = [&] {
-    mma3<32, 32>(tcol + cG, sg + oAg, sw + tOff(2));
-    mma3<32, 32>(tcol + cC, sg + oAc, sw + tOff(3));
+    mma3<32, 32>(tcol + cG, tcol + cAg, sg + oAg, sw + tOff(2));
+    mma3<32, 32>(tcol + cC, tcol + cAc, sg + oAc, sw + tOff(3));
   };
 
   // ray-quads are dealt group-major, as in the compact kernel
@@ -403,7 +452,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
         tc::tmem_ld_wait();
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = fmaxf(v[k] + hb1[k], 0.f);
-        store_row_planes<3, 32, kAP>(tileA, row, v);
+        put_rows<32, false>(ta, tileA, row, v);
         phase2<false>(T, f2, nop, nop);
         if (put) put_planes<8>(sp, half ? kQr1 : kQa1, v);
         if (!(alive = phase_wait(T))) break;
@@ -493,7 +542,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
         tc::tmem_ld_wait();
 #pragma unroll
         for (int k = 0; k < 32; ++k) h1[k] = fmaxf(h1[k] + hb1[k], 0.f);
-        store_row_planes<3, 32, kAP>(tileA, row, h1);
+        put_rows<32, false>(ta, tileA, row, h1);
         phase2<false>(T, f2, nop, nop);
         if (!(alive = phase_wait(T))) break;
         tc::tmem_ld32(tx, v);
@@ -547,7 +596,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
           v[k] = v[k] > 0.f ? d : 0.f;
         }
       }
-      store_row_planes<3, 32, kAP>(tileA, row, v);
+      put_rows<32, true>(ta, tileA, row, v);
       const float one8[8] = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // ones column: the bias gradient lands in its row
       if (half == 0) {
         store_row_planes<2, 32, kBPg>(tileB, row, h1);
@@ -558,8 +607,8 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
       }
       // B1: dA1 = dY2 gW2, dR1 = dQ2 cW2; dW2^T (+)= a1^T dY2 and the colour's [r1 | 1]^T dQ2
       phase2<true>(T, [&] {
-        mma3<32, 32>(tcol + cG, sg + oAg, sw + tOff(4));
-        mma3<32, 32>(tcol + cC, sg + oAc, sw + tOff(5));
+        mma3<32, 32>(tcol + cG, tcol + cAg, sg + oAg, sw + tOff(4));
+        mma3<32, 32>(tcol + cC, tcol + cAc, sg + oAc, sw + tOff(5));
       }, [&] {
         issue_mma_dw<2, 3, 2, 32>(tcol + cWg2, sg + oBg, kBPg, 4u * 128u, sg + oAg, kAP, 4u * 128u, dw_acc);
       }, [&] {
@@ -583,7 +632,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
 #pragma unroll
       for (int k = 0; k < 32; ++k) v[k] = h1[k] > 0.f ? v[k] : 0.f;  // dy1, dq1
       tiles_free(T);
-      store_row_planes<3, 32, kAP>(tileA, row, v);
+      put_rows<32, true>(ta, tileA, row, v);
       if (half == 0) {
         store_quarter<2, 24, kBPg>(tileB, row, 0, make_float4(u[0], u[1], u[2], u[3]));
         store_chunk<2, 24, kBPg>(tileB, row, 1, u + 8);
@@ -595,8 +644,8 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
       }
       // B2: dZ = dY1 gW1, dU = dQ1 cW1; dW1, db1 (+)= [z | 1]^T dY1 and the colour's [u | 1]^T dQ1
       phase2<true>(T, [&] {
-        mma3<16, 32>(tcol + cG, sg + oAg, sw + tOff(6));
-        mma3<16, 32>(tcol + cC, sg + oAc, sw + tOff(7));
+        mma3<16, 32>(tcol + cG, tcol + cAg, sg + oAg, sw + tOff(6));
+        mma3<16, 32>(tcol + cC, tcol + cAc, sg + oAc, sw + tOff(7));
       }, [&] {
         issue_mma_dw<2, 3, 2, 32>(tcol + cWg1, sg + oBg, kBPg, 3u * 128u, sg + oAg, kAP, 4u * 128u, dw_acc);
       }, [&] {
