@@ -46,12 +46,17 @@ struct ImpArgs {
 // the tensor core (three bfloat16 parts per operand, six part products: FP32-grade); the
 // workload's decoder finishes phi = W2[0,:] relu(H1 + b1) + b2[0] on CUDA cores, the paper's
 // runs H2 = A1 gW2^T as a second phase and phi = gw3 . relu(H2 + gb2) + gb3.  Opacities,
-// scans, draws and the rank merge stay per warp on CUDA cores as above.
+// scans, draws and the rank merge stay per warp on CUDA cores as above.  The A operands are in
+// tensor memory (in shared memory every product read its 4 KB again, and the 98 KB of tiles were
+// taken from the L1 cache that the corner loads live on): 231 us for 8192 x 132 with the paper's
+// decoder, now 184.
 constexpr int kItGroups = 4;
 constexpr int kItThreads = kItGroups * kGroupThreads;
-constexpr uint32_t kItA = 128u * 32u * 2u * 3u;  // a group's A tile: 3 parts of 128 x 32 (z, then a1)
 constexpr uint32_t kItW1 = 32u * 16u * 2u, kItW2 = 32u * 32u * 2u;  // one part of W1 {32, 16}, gW2 {32, 32}
-constexpr uint32_t oItW = kItGroups * kItA, oItScal = oItW + 3u * (kItW1 + kItW2);
+constexpr uint32_t oItW = 0, oItScal = oItW + 3u * (kItW1 + kItW2);
+// tensor-memory columns: a group's result (32), then its A operand (3 parts of K / 2 columns)
+constexpr uint32_t kItCols = 80, kItTmem = 512;
+static_assert(kItGroups * kItCols <= kItTmem, "tensor-memory columns");
 constexpr uint32_t kItMbarLimit = 1u << 20;
 
 template <bool kPaper>
@@ -85,8 +90,7 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = warp >> 2, warp_g = warp & 3;
   Group G;
-  G.a = base + gi * kItA;
-  G.b = nullptr;
+  G.a = G.b = nullptr;
   G.mbar = &mbar[gi];
   G.mbar_dw = &mbar[gi];
   G.abort = &abort_flag[gi];
@@ -99,13 +103,28 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
     tc::fence_mbar_init();
     *G.abort = 0;
   }
-  if (threadIdx.x < 32) tc::tmem_alloc(&tslot, 128);
+  if (threadIdx.x < 32) tc::tmem_alloc(&tslot, kItTmem);
   tc::fence_smem_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  G.tcol = tslot + (uint32_t)(gi * 32);
-  const int row = G.gt;
+  const int gu = __shfl_sync(0xffffffffu, gi, 0), wu = __shfl_sync(0xffffffffu, warp_g, 0);  // uniform
+  G.tcol = __shfl_sync(0xffffffffu, tslot, 0) + (uint32_t)gu * kItCols;
+  const uint32_t ta = lane_addr(G, 32, wu), sW1 = tc::smem_u32(W1t), sW2 = tc::smem_u32(W2t);
+  // operand rows in tensor memory -> one thread of the group's first warp issues the products
+  auto issue = [&](auto products) {
+    tc::tmem_st_wait();
+    tc::fence_before_sync();
+    group_sync(gu);
+    tc::fence_after_sync();
+    if (wu == 0) {
+      if (tc::elect_one()) {
+        products();
+        tc::mma_commit(G.mbar);
+      }
+      __syncwarp();
+    }
+  };
   bool alive = true;
   const float s_sharp = expf(mlp[kPaper ? paper::A_kappa : oKappa]);
   // one phi round of the whole group: this lane's point x (valid) or an idle row
@@ -117,8 +136,9 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
 #pragma unroll
       for (int k = 0; k < kZ; ++k) z[k] = 0.f;
     }
-    store_row_planes<3, kZ, 128u * 32u * 2u>(G.a, row, z);
-    mma_phase_issue<PrecBF16x3, 32, kZ>(G, 0, W1t, kItW1);
+    __syncwarp();
+    put_operand<PrecBF16x3, kZ, false, 8>(ta, nullptr, 0, 0, z);
+    issue([&] { tile_mma<PrecBF16x3, 32, kZ>(G.tcol, G.tcol + 32, sW1, kItW1); });
     if (!(alive = alive && mma_phase_wait(G))) return 0.f;
     float v[32];
     tc::tmem_ld32(lane_addr(G, 0, warp_g), v);
@@ -130,8 +150,9 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
     } else {
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j] + sc[j], 0.f);
-      store_row_planes<3, 32, 128u * 32u * 2u>(G.a, row, v);
-      mma_phase_issue<PrecBF16x3, 32, 32>(G, 0, W2t, kItW2);
+      put_operand<PrecBF16x3, 32, false, 8>(ta, nullptr, 0, 0, v);
+      put_operand<PrecBF16x3, 32, false, 8>(ta, nullptr, 0, 8, v + 16);
+      issue([&] { tile_mma<PrecBF16x3, 32, 32>(G.tcol, G.tcol + 32, sW2, kItW2); });
       if (!(alive = alive && mma_phase_wait(G))) return 0.f;
       tc::tmem_ld32(lane_addr(G, 0, warp_g), v);
       tc::tmem_ld_wait();
@@ -307,7 +328,7 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
   __syncthreads();
   if (threadIdx.x < 32) {
     tc::fence_after_sync();
-    tc::tmem_dealloc(tslot, 128);
+    tc::tmem_dealloc(tslot, kItTmem);
   }
 }
 

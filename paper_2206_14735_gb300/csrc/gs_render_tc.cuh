@@ -330,18 +330,6 @@ struct Group {
   int g, gt;
 };
 
-// A rows written by every thread of a 128-thread group -> its thread 0 issues the MMA and commits
-template <class P, int N, int K>
-__device__ __forceinline__ void mma_phase_issue(Group& G, uint32_t dcol, const uint8_t* w, uint32_t wplane) {
-  tc::fence_smem_async();
-  tc::fence_before_sync();
-  group_sync(G.g);
-  tc::fence_after_sync();
-  if (G.gt == 0) {
-    issue_mma<P, N, K>(G.tcol + dcol, tc::smem_u32(G.a), tc::smem_u32(w), wplane);
-    tc::mma_commit(G.mbar);
-  }
-}
 // ---- the compact render kernel's tile groups ------------------------------------------------
 // A tile group's barriers: the phase's products done, its weight-gradient products done
 struct TileBars {
