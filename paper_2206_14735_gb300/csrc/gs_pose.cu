@@ -127,34 +127,39 @@ __global__ void __launch_bounds__(128) pose_backward_kernel(PoseBwdArgs a) {
       float gx[3] = {0.f, 0.f, 0.f};
 #pragma unroll
       for (int l = 0; l < kLevels; ++l) {
-        float4 dl[3];
+        // sum_c (theta_c . dL/dz_l) dw_c/dx: a corner's features meet the record first (one product
+        // sum per corner, then three axes) instead of three axes of four features each
+        const Cell c = locate(a.g, l, x);
         float dw[8][3];
-        const Cell c = level_jacobian(a.g, a.theta, l, x, dl, dw);
+        corner_weight_grads(c.f, c.clamped, dw);
         const float4 d4 = dzk[l];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) gx[q] += dl[q].x * d4.x + dl[q].y * d4.y + dl[q].z * d4.z + dl[q].w * d4.w;
-        if (kPaper && l == kLevels - 1) {  // colour grid on the finest level's cell
-          const float4 c0 = dzk[4], c1 = dzk[5];
-          const float dcf[6] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y};
+        const long long nx = a.g.dims[l][0], nxy = nx * a.g.dims[l][1];
+        const float4* p = reinterpret_cast<const float4*>(a.theta + a.g.off[l]) + c.vtx;
+        const bool colour = kPaper && l == kLevels - 1;  // the colour grid lies on the finest level's cells
+        float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+        if (colour) {
+          c0 = dzk[4];
+          c1 = dzk[5];
           gd[0] += c1.z;
           gd[1] += c1.w;
           gd[2] += dzk[6].x;
-          const float2* cg = reinterpret_cast<const float2*>(a.theta + a.colour_off);
-          const float iv = a.g.inv_voxel[l];
-#pragma unroll
-          for (int cc = 0; cc < 8; ++cc) {
-            const long long v2 = (c.vtx + corner_offset(a.g, l, cc)) * 3;
-            float sf = 0.f;
-#pragma unroll
-            for (int e = 0; e < 3; ++e) {
-              const float2 f2 = __ldg(cg + v2 + e);
-              sf = fmaf(f2.x, dcf[2 * e], sf);
-              sf = fmaf(f2.y, dcf[2 * e + 1], sf);
-            }
-#pragma unroll
-            for (int q = 0; q < 3; ++q) gx[q] = fmaf(sf * iv, dw[cc][q], gx[q]);
-          }
         }
+        float sg[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int cc = 0; cc < 8; ++cc) {
+          const long long at = (cc >> 2) + ((cc & 2) ? nx : 0) + ((cc & 1) ? nxy : 0);
+          const float4 v = __ldg(p + at);
+          float sf = v.x * d4.x + v.y * d4.y + v.z * d4.z + v.w * d4.w;
+          if (colour) {
+            const float2* cg = reinterpret_cast<const float2*>(a.theta + a.colour_off) + (c.vtx + at) * 3;
+            const float2 e0 = __ldg(cg), e1 = __ldg(cg + 1), e2 = __ldg(cg + 2);
+            sf += e0.x * c0.x + e0.y * c0.y + e1.x * c0.z + e1.y * c0.w + e2.x * c1.x + e2.y * c1.y;
+          }
+#pragma unroll
+          for (int q = 0; q < 3; ++q) sg[q] = fmaf(sf, dw[cc][q], sg[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) gx[q] = fmaf(a.g.inv_voxel[l], sg[q], gx[q]);
       }
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
@@ -267,14 +272,19 @@ struct EikPoseArgs {
 
 // one warp per ray, lanes over its samples (free-space ones only), then lane 0 adds the
 // ray's sums to its frame's six derivatives
-template <bool kPaper>
-__global__ void __launch_bounds__(128) eikonal_pose_kernel(EikPoseArgs a) {
-  __shared__ __align__(16) float sd[kSensFloats<kPaper>];
-  __shared__ __align__(16) float sp[128][kZ];           // this thread's p, read level by level
-  __shared__ float sh[kPaper ? 128 : 1][kPaper ? 65 : 1];  // the paper decoder's hidden layers
-  const float* mlp = a.theta + a.g.n_grid;
-  for (int i = threadIdx.x; i < kSensFloats<kPaper>; i += blockDim.x) sd[i] = mlp[i];
-  __syncthreads();
+// kRec: the batch's Eikonal records hold the sensitivity; without the decoder's evaluation the
+// kernel takes 64 registers for 168 (the paper's decoder), and its corner loads get more than twice
+// the warps: 146 us for 8192 x 132, now 74
+template <bool kPaper, bool kRec>
+__global__ void __launch_bounds__(128, kRec ? 8 : (kPaper ? 3 : 2)) eikonal_pose_kernel(EikPoseArgs a) {
+  __shared__ __align__(16) float sd[kRec ? 4 : kSensFloats<kPaper>];
+  __shared__ __align__(16) float sp[128][kZ];  // this thread's p, read level by level
+  __shared__ float sh[kPaper && !kRec ? 128 : 1][kPaper && !kRec ? 65 : 1];  // the paper decoder's hidden layers
+  if constexpr (!kRec) {
+    const float* mlp = a.theta + a.g.n_grid;
+    for (int i = threadIdx.x; i < kSensFloats<kPaper>; i += blockDim.x) sd[i] = mlp[i];
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31;
   const int n_fs = a.counts[2];
   const float kscale = n_fs > 0 ? (a.dloss != nullptr ? a.dloss[0] : 1.f) * -2.f / (float)n_fs : 0.f;
@@ -288,7 +298,7 @@ __global__ void __launch_bounds__(128) eikonal_pose_kernel(EikPoseArgs a) {
       const float tk = a.t[(size_t)i * a.N + k];
       float x[3];
       sample_pos(o, r, tk, x);
-      if (a.eik != nullptr) {  // q_l = p_l / v_l from the records
+      if constexpr (kRec) {  // q_l = p_l / v_l from the records
         const float4* rec = a.eik + (size_t)i * a.N + k;
 #pragma unroll
         for (int l = 0; l < kLevels; ++l) *reinterpret_cast<float4*>(myp + 4 * l) = __ldg(rec + l * a.eik_stride);
@@ -320,33 +330,33 @@ __global__ void __launch_bounds__(128) eikonal_pose_kernel(EikPoseArgs a) {
         const Cell c = locate(a.g, l, x);
         const float4* lv = reinterpret_cast<const float4*>(a.theta + a.g.off[l]);
         const float4 p4 = *reinterpret_cast<const float4*>(myp + 4 * l);
-        float4 d0 = make_float4(0.f, 0.f, 0.f, 0.f), d1 = d0, d2 = d0, e01 = d0, e02 = d0, e12 = d0;
+        const long long nx = a.g.dims[l][0], nxy = nx * a.g.dims[l][1];
+        float dot0 = 0.f, dot1 = 0.f, dot2 = 0.f, e01 = 0.f, e02 = 0.f, e12 = 0.f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int bx = (q >> 2) & 1, by = (q >> 1) & 1, bz = q & 1;
           const float wx = bx ? c.f[0] : 1.f - c.f[0], wy = by ? c.f[1] : 1.f - c.f[1], wz = bz ? c.f[2] : 1.f - c.f[2];
-          const float sx = bx ? 1.f : -1.f, sy = by ? 1.f : -1.f, sz = bz ? 1.f : -1.f;
-          const float4 v = __ldg(lv + c.vtx + corner_offset(a.g, l, q));
-          f4fma(d0, sx * wy * wz, v);
-          f4fma(d1, wx * sy * wz, v);
-          f4fma(d2, wx * wy * sz, v);
-          f4fma(e01, sx * sy * wz, v);
-          f4fma(e02, sx * wy * sz, v);
-          f4fma(e12, wx * sy * sz, v);
+          const float4 v = __ldg(lv + c.vtx + bx + (by ? nx : 0) + (bz ? nxy : 0));
+          // the corner's features meet the sensitivity once, then the six derivatives of its weight
+          const float sv = v.x * p4.x + v.y * p4.y + v.z * p4.z + v.w * p4.w;
+          const float sx = bx ? sv : -sv, sy = by ? sv : -sv, sz = bz ? sv : -sv;
+          dot0 = fmaf(wy * wz, sx, dot0);
+          dot1 = fmaf(wx * wz, sy, dot1);
+          dot2 = fmaf(wx * wy, sz, dot2);
+          e01 = fmaf(wz, by ? sx : -sx, e01);
+          e02 = fmaf(wy, bz ? sx : -sx, e02);
+          e12 = fmaf(wx, bz ? sy : -sy, e12);
         }
         // the records hold p_l already divided by v_l
-        const float iv = a.eik != nullptr ? 1.f : a.g.inv_voxel[l];
-        const float iv2 = a.eik != nullptr ? a.g.inv_voxel[l] : iv * iv;
+        const float iv = kRec ? 1.f : a.g.inv_voxel[l];
+        const float iv2 = kRec ? a.g.inv_voxel[l] : iv * iv;
         const bool cx = c.clamped & 1u, cy = c.clamped & 2u, cz = c.clamped & 4u;
-        const float dot0 = d0.x * p4.x + d0.y * p4.y + d0.z * p4.z + d0.w * p4.w;
-        const float dot1 = d1.x * p4.x + d1.y * p4.y + d1.z * p4.z + d1.w * p4.w;
-        const float dot2 = d2.x * p4.x + d2.y * p4.y + d2.z * p4.z + d2.w * p4.w;
         if (!cx) gx[0] = fmaf(dot0, iv, gx[0]);
         if (!cy) gx[1] = fmaf(dot1, iv, gx[1]);
         if (!cz) gx[2] = fmaf(dot2, iv, gx[2]);
-        if (!cx && !cy) h01 = fmaf(e01.x * p4.x + e01.y * p4.y + e01.z * p4.z + e01.w * p4.w, iv2, h01);
-        if (!cx && !cz) h02 = fmaf(e02.x * p4.x + e02.y * p4.y + e02.z * p4.z + e02.w * p4.w, iv2, h02);
-        if (!cy && !cz) h12 = fmaf(e12.x * p4.x + e12.y * p4.y + e12.z * p4.z + e12.w * p4.w, iv2, h12);
+        if (!cx && !cy) h01 = fmaf(e01, iv2, h01);
+        if (!cx && !cz) h02 = fmaf(e02, iv2, h02);
+        if (!cy && !cz) h12 = fmaf(e12, iv2, h12);
       }
       const float nrm = sqrtf(gx[0] * gx[0] + gx[1] * gx[1] + gx[2] * gx[2]);
       if (!(nrm > 0.f)) continue;
@@ -426,7 +436,9 @@ gs_status gs_launch_eikonal_pose_backward(const gs_ctx* ctx, const float* theta,
   a.eik = reinterpret_cast<const float4*>(b->eik);
   a.eik_stride = (long long)b->R * b->N;
   const int blocks = (int)std::min<long long>(((long long)b->R * 32 + 127) / 128, 16LL * ctx->num_sms);
-  if (ctx->cfg.arch == GS_ARCH_PAPER) eikonal_pose_kernel<true><<<blocks, 128, 0, st>>>(a);
-  else eikonal_pose_kernel<false><<<blocks, 128, 0, st>>>(a);
+  const bool paper = ctx->cfg.arch == GS_ARCH_PAPER, rec = a.eik != nullptr;
+  auto k = paper ? (rec ? eikonal_pose_kernel<true, true> : eikonal_pose_kernel<true, false>)
+                 : (rec ? eikonal_pose_kernel<false, true> : eikonal_pose_kernel<false, false>);
+  k<<<blocks, 128, 0, st>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
