@@ -276,7 +276,7 @@ struct EikPoseArgs {
 // kernel takes 64 registers for 168 (the paper's decoder), and its corner loads get more than twice
 // the warps: 146 us for 8192 x 132, now 74
 template <bool kPaper, bool kRec>
-__global__ void __launch_bounds__(128, kRec ? 8 : (kPaper ? 3 : 2)) eikonal_pose_kernel(EikPoseArgs a) {
+__global__ void __launch_bounds__(128, kRec ? 8 : (kPaper ? 3 : 0)) eikonal_pose_kernel(EikPoseArgs a) {
   __shared__ __align__(16) float sd[kRec ? 4 : kSensFloats<kPaper>];
   __shared__ __align__(16) float sp[128][kZ];  // this thread's p, read level by level
   __shared__ float sh[kPaper && !kRec ? 128 : 1][kPaper && !kRec ? 65 : 1];  // the paper decoder's hidden layers
