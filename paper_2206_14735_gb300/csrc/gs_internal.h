@@ -13,7 +13,10 @@ constexpr int kSmoothCtas = 128;  // CTAs of the smoothness kernel (fixed, so pa
 constexpr int kRenderCtasPerSm = 1;  // persistent render CTAs per SM
 constexpr int kStoreFloatsPerSample = 100;  // stored activations: z 16, a1 32, (phi, h) 16, a2 32, c 3 + 1 pad
 constexpr int kPaperStoreFloatsPerSample = 156;  // paper architecture: z 16, cf 6 + phi + pad, c 3 + pad, 4 x 32 hidden
-constexpr int kRenderGroups = 2;     // tile groups (8 warps, 176 tensor-memory columns each) per render CTA
+// Tile groups (8 warps) per CTA of the compact render kernel.  With a reverse pass two of 128
+// registers a thread; a forward-only call holds less per thread, and its third group at 80
+// registers fills the waits of the other two: 8192 rays x 132, 197 us with two, 187 us with three.
+constexpr int kRenderGroups = 2, kForwardGroups = 3;
 // Bits of the context's device status word: a kernel sets its bit when a bounded wait for its
 // tensor-core products ran out (it then stops early; that call's outputs are incomplete)
 constexpr int kStatusRender = 2, kStatusProposal = 4, kStatusEikonal = 8, kStatusPaperRender = 16,

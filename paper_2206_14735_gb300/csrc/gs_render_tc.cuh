@@ -23,11 +23,11 @@
 // before the operands moved to tensor memory, in bursts: the phases of a group load it in turn)
 // and each group's serial chain; DRAM and the tensor cores are below 20 %.  Hence two threads per
 // row (half the chain at the same shared and tensor memory), the phases' A operands in tensor
-// memory, two groups of 128 registers without spills (three at 80 registers measured slower:
-// 607 against 476 us, at the same data path), the weight gradients' part pairs in as few products
+// memory, two groups of 128 registers without spills (three at 80 registers measured slower
+// with a reverse pass: 607 against 476 us, at the same data path), the weight gradients' part pairs in as few products
 // as the tile layout allows.  Render call, 8192 x 96, stored: one thread per row and three groups
 // 523 us, two threads and two groups 476 us, A operands in tensor memory 451 us; forward only,
-// 8192 x 132: 251, 223, 198 us.
+// 8192 x 132: 251, 223, 197 us, and 187 us with three groups, which only that form has.
 #pragma once
 #include "gs_internal.h"
 #include <cuda_bf16.h>
@@ -75,11 +75,16 @@ __host__ __device__ constexpr uint32_t wTotal() { return wOff<P>(kTiles); }
 // read back before the next phase that writes its columns), then the decoder weight gradients,
 // accumulated over all of the group's tiles (M = 64 layout: row m in lane 32 (m / 16) + m % 16)
 // and the phases' A operand: part p of a K-column row in columns cA + p K / 2 ..
-constexpr uint32_t cX = 0, cY = 32, cW1 = 48, cW2 = 72, cW3 = 112, cA = 128, kGroupCols = 176;
+// (a forward-only call has no weight gradients: its operand follows the results)
+constexpr uint32_t cX = 0, cY = 32, cW1 = 48, cW2 = 72, cW3 = 112;
+template <bool BWD>
+constexpr uint32_t cA = BWD ? 128 : 48;
+template <bool BWD>
+constexpr uint32_t kGroupCols = cA<BWD> + 48;
 // tcgen05.alloc takes a power of two >= 32 columns
-__host__ __device__ constexpr uint32_t tmem_cols(int groups) {
+__host__ __device__ constexpr uint32_t tmem_cols(uint32_t columns) {
   uint32_t c = 32;
-  while (c < (uint32_t)groups * kGroupCols) c <<= 1;
+  while (c < columns) c <<= 1;
   return c;
 }
 
@@ -336,15 +341,15 @@ struct TileBars {
   uint64_t done, dw;
   int abort;
 };
-template <class P, int TYPE>  // 0..2 the forward layers, 3..5 the adjoints b3, b2, b1
+template <class P, int TYPE, bool BWD>  // 0..2 the forward layers, 3..5 the adjoints b3, b2, b1
 __device__ __forceinline__ void issue_phase(uint32_t tcol, uint32_t sw) {
   constexpr uint32_t wplane = wTotal<P>();
-  if constexpr (TYPE == 0) tile_mma<P, 32, 16>(tcol + cX, tcol + cA, sw + wOff<P>(0), wplane);
-  if constexpr (TYPE == 1) tile_mma<P, 16, 32>(tcol + cY, tcol + cA, sw + wOff<P>(1), wplane);
-  if constexpr (TYPE == 2) tile_mma<P, 32, 16>(tcol + cX, tcol + cA, sw + wOff<P>(2), wplane);
-  if constexpr (TYPE == 3) tile_mma<P, 16, 32>(tcol + cY, tcol + cA, sw + wOff<P>(3), wplane);
-  if constexpr (TYPE == 4) tile_mma<P, 32, 16>(tcol + cX, tcol + cA, sw + wOff<P>(4), wplane);
-  if constexpr (TYPE == 5) tile_mma<P, 16, 32>(tcol + cY, tcol + cA, sw + wOff<P>(5), wplane);
+  if constexpr (TYPE == 0) tile_mma<P, 32, 16>(tcol + cX, tcol + cA<BWD>, sw + wOff<P>(0), wplane);
+  if constexpr (TYPE == 1) tile_mma<P, 16, 32>(tcol + cY, tcol + cA<BWD>, sw + wOff<P>(1), wplane);
+  if constexpr (TYPE == 2) tile_mma<P, 32, 16>(tcol + cX, tcol + cA<BWD>, sw + wOff<P>(2), wplane);
+  if constexpr (TYPE == 3) tile_mma<P, 16, 32>(tcol + cY, tcol + cA<BWD>, sw + wOff<P>(3), wplane);
+  if constexpr (TYPE == 4) tile_mma<P, 32, 16>(tcol + cX, tcol + cA<BWD>, sw + wOff<P>(4), wplane);
+  if constexpr (TYPE == 5) tile_mma<P, 16, 32>(tcol + cY, tcol + cA<BWD>, sw + wOff<P>(5), wplane);
 }
 template <class P, int TYPE>
 __device__ __forceinline__ void issue_phase_dw(uint32_t tcol, uint32_t sa, bool acc) {
@@ -364,7 +369,7 @@ struct Tile {
 // Operand rows of this warp written -> once all warps have met, one thread of warp 0 issues the
 // phase's products and (adjoint phases) one of warp 4 the weight-gradient products that
 // read the same tiles.
-template <class P, int TYPE>
+template <class P, int TYPE, bool BWD>
 __device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa, uint32_t sw, bool dw_acc) {
   tc::tmem_st_wait();
   if (TYPE >= 3) tc::fence_smem_async();
@@ -373,8 +378,7 @@ __device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa,
   tc::fence_after_sync();
   if (T.w8 == 0) {
     if (tc::elect_one()) {
-      issue_phase<P, TYPE>(tcol, sw);
-
+      issue_phase<P, TYPE, BWD>(tcol, sw);
       tc::mma_commit(&T.bars->done);
     }
     __syncwarp();
@@ -918,11 +922,14 @@ __device__ __forceinline__ void composite_ray(const Args& a, int ray, bool has_r
 template <class P, int NCH, int GR, bool FWD, bool BWD>
 __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const __grid_constant__ RenderTcArgs a) {
   using L = TcLayout<P>;
+  // a forward-only call writes no tiles: its groups have only their barriers in shared memory
+  static_assert(sizeof(TileBars) <= 128, "a group's barriers");
+  constexpr uint32_t kGroupBytes = BWD ? L::group_bytes : 128u, kBarOff = BWD ? L::bar_off : 0u;
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr uint32_t wplane = wTotal<P>();  // one bf16 part of all weight tiles
   // tile groups | weight tiles | exchange rows [GR][NCH][128] float4 | rays | accumulators, biases
   uint8_t* gbase = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem) + 127) & ~uintptr_t(127));
-  uint8_t* wt0 = gbase + (size_t)GR * L::group_bytes;
+  uint8_t* wt0 = gbase + (size_t)GR * kGroupBytes;
   float4* xch0 = reinterpret_cast<float4*>(wt0 + wplane * P::planes);
   float4* rays0 = xch0 + (size_t)GR * NCH * 128;
   float* sums0 = reinterpret_cast<float*>(rays0 + GR * 20);  // [GR][4][kSums]: a compositing warp's running sums
@@ -935,10 +942,10 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
   const int gi = warp >> 3, w8 = warp & 7, half = w8 >> 2, wq = w8 & 3;
   const int row = 32 * wq + lane;  // tile row of this thread's sample
-  uint8_t* const tileA = gbase + (size_t)gi * L::group_bytes;
+  uint8_t* const tileA = gbase + (size_t)gi * kGroupBytes;
   uint8_t* const tileB = tileA + L::b_off;
   Tile T;
-  T.bars = reinterpret_cast<TileBars*>(tileA + L::bar_off);
+  T.bars = reinterpret_cast<TileBars*>(tileA + kBarOff);
   T.ph_done = T.ph_dw = 0;
   T.w8 = w8;
   T.g = gi;
@@ -990,8 +997,8 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
     kc[3] = n_fs > 0 ? wt[3] / (float)n_fs : 0.0f;
     kc[4] = expf(mlp[oKappa]);
   }
-  static_assert(tmem_cols(GR) <= 512, "tensor memory holds 512 columns");
-  if (warp == 0) tc::tmem_alloc(tslot, tmem_cols(GR));
+  static_assert(tmem_cols(GR * kGroupCols<BWD>) <= 512, "tensor memory holds 512 columns");
+  if (warp == 0) tc::tmem_alloc(tslot, tmem_cols(GR * kGroupCols<BWD>));
   tc::fence_smem_async();
   tc::fence_before_sync();
   __syncthreads();
@@ -1005,9 +1012,9 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
   // dW4[.][16 half + lane % 16] over this warp's samples of parity lane / 16
   float w4acc[3] = {0.f, 0.f, 0.f};
 
-  const uint32_t sw = tc::smem_u32(wt0), sa = tc::smem_u32(gbase) + (uint32_t)gi * L::group_bytes;
-  const uint32_t tcol = tmem0 + (uint32_t)(gi * kGroupCols);
-  const uint32_t tq = tcol + ((uint32_t)(32 * wq) << 16), ta = tq + cA;  // this warp's lanes
+  const uint32_t sw = tc::smem_u32(wt0), sa = tc::smem_u32(gbase) + (uint32_t)gi * kGroupBytes;
+  const uint32_t tcol = tmem0 + (uint32_t)gi * kGroupCols<BWD>;
+  const uint32_t tq = tcol + ((uint32_t)(32 * wq) << 16), ta = tq + cA<BWD>;  // this warp's lanes
   const float* b1 = bias + 16 * half;  // this half's units
   const float* b2 = bias + 32;
   const float* b3 = bias + 48 + 16 * half;
@@ -1110,7 +1117,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
         position(pick_tc(tt, j), x);
         gather_store(x, valid, zl, zh);
       }
-      phase_issue<P, 0>(T, tcol, sa, sw, dw_acc);
+      phase_issue<P, 0, BWD>(T, tcol, sa, sw, dw_acc);
       if (put) {
         sp[kPz + l_lo] = zl;
         sp[kPz + l_hi] = zh;
@@ -1122,7 +1129,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
 #pragma unroll
       for (int k = 0; k < 16; ++k) v[k] = fmaxf(v[k] + b1[k], 0.f);
       put_operand<P, 32, false, 8>(ta, nullptr, row, 8 * half, v);
-      phase_issue<P, 1>(T, tcol, sa, sw, dw_acc);
+      phase_issue<P, 1, BWD>(T, tcol, sa, sw, dw_acc);
       if (put) put_planes<4>(sp, kPa1 + 4 * half, v);
       if (!(alive = phase_wait(T))) break;
       float u[16];
@@ -1132,7 +1139,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       float h[8];
       hidden_row(u, h);
       put_operand<P, 16, false, 4>(ta, nullptr, row, 4 * half, h);
-      phase_issue<P, 2>(T, tcol, sa, sw, dw_acc);
+      phase_issue<P, 2, BWD>(T, tcol, sa, sw, dw_acc);
       if (put) put_planes<2>(sp, kPh + 2 * half, h);
       if (!(alive = phase_wait(T))) break;
       tc::tmem_ld16(tq + cX + 16 * half, v);
@@ -1208,21 +1215,21 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
           position(pick_tc(tt, j), x);
           gather_store(x, valid, zl, zh);
         }
-        phase_issue<P, 0>(T, tcol, sa, sw, dw_acc);
+        phase_issue<P, 0, BWD>(T, tcol, sa, sw, dw_acc);
         if (!(alive = phase_wait(T))) break;
         tc::tmem_ld16(tq + cX + 16 * half, a1);
         tc::tmem_ld_wait();
 #pragma unroll
         for (int k = 0; k < 16; ++k) a1[k] = fmaxf(a1[k] + b1[k], 0.f);
         put_operand<P, 32, false, 8>(ta, nullptr, row, 8 * half, a1);
-        phase_issue<P, 1>(T, tcol, sa, sw, dw_acc);
+        phase_issue<P, 1, BWD>(T, tcol, sa, sw, dw_acc);
         if (!(alive = phase_wait(T))) break;
         float u[16];
         tc::tmem_ld16(tq + cY, u);
         tc::tmem_ld_wait();
         hidden_row(u, h);
         put_operand<P, 16, false, 4>(ta, nullptr, row, 4 * half, h);
-        phase_issue<P, 2>(T, tcol, sa, sw, dw_acc);
+        phase_issue<P, 2, BWD>(T, tcol, sa, sw, dw_acc);
         if (!(alive = phase_wait(T))) break;
         tc::tmem_ld16(tq + cX + 16 * half, v);
         tc::tmem_ld_wait();
@@ -1269,7 +1276,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       if (half != 0) h[7] = 1.f;  // ones column: the bias gradient db3 lands in column 15 of dW3
       store_chunk<L::b_planes, 16, L::b_bytes>(tileB, row, half, h);
       // --- b3: dh = dy2 W3;  dW3, db3 (+)= dy2^T [h | 1] ---
-      phase_issue<P, 3>(T, tcol, sa, sw, dw_acc);
+      phase_issue<P, 3, BWD>(T, tcol, sa, sw, dw_acc);
       if (stored) get_planes<4>(sp, kPa1 + 4 * half, get, a1);
       if (!(alive = phase_wait(T))) break;
       {
@@ -1286,7 +1293,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       const float one8[8] = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       if (half != 0) store_chunk<L::b_planes, 40, L::b_bytes>(tileA + L::b_wide, row, 4, one8);
       // --- b2: da1 = dout W2;  dW2^T, db2 (+)= [a1 | 1]^T dout ---
-      phase_issue<P, 4>(T, tcol, sa, sw, dw_acc);
+      phase_issue<P, 4, BWD>(T, tcol, sa, sw, dw_acc);
       if (stored) {
         zl = get ? sp[kPz + l_lo] : make_float4(0.f, 0.f, 0.f, 0.f);
         zh = get ? sp[kPz + l_hi] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1302,7 +1309,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       store_quarter<L::b_planes, 24, L::b_bytes>(tileB, row, l_hi, zh);
       if (half != 0) store_chunk<L::b_planes, 24, L::b_bytes>(tileB, row, 2, one8);
       // --- b1: dz = dy1 W1;  dW1, db1 (+)= dy1^T [z | 1] ---
-      phase_issue<P, 5>(T, tcol, sa, sw, dw_acc);
+      phase_issue<P, 5, BWD>(T, tcol, sa, sw, dw_acc);
       if (!(alive = phase_wait(T))) break;
       dw_acc = true;
       float4 gl4, gh4;  // dL/dz at this half's levels
@@ -1410,21 +1417,21 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
     }
     a.mlp_part[(size_t)blockIdx.x * kMlpPad + i] = v;
   }
-  if (warp == 0) tc::tmem_dealloc(*tslot, tmem_cols(GR));
+  if (warp == 0) tc::tmem_dealloc(*tslot, tmem_cols(GR * kGroupCols<BWD>));
 }
 #pragma nv_diag_default 128
 
-template <class P, int NCH, int GR>
+template <class P, int NCH, int GR, bool BWD>
 constexpr size_t render_tc_smem() {
   using L = TcLayout<P>;
   static_assert(kMlpPad * 4 <= L::bar_off, "a group's decoder-gradient row fits over its tiles");
-  return 128 + (size_t)GR * L::group_bytes + wTotal<P>() * P::planes + (size_t)GR * NCH * 128 * 16 +
+  return 128 + (size_t)GR * (BWD ? L::group_bytes : 128u) + wTotal<P>() * P::planes + (size_t)GR * NCH * 128 * 16 +
          GR * 20 * 16 + (GR * 4 * kSums + 88 + 96 + 8 + 4) * 4;
 }
 
 template <class P, int NCH, int GR, bool FWD, bool BWD>
 gs_status launch_tc_t(const gs_ctx* ctx, RenderTcArgs& a, cudaStream_t st) {
-  constexpr size_t smem = render_tc_smem<P, NCH, GR>();
+  constexpr size_t smem = render_tc_smem<P, NCH, GR, BWD>();
   static_assert(smem <= 227u * 1024u, "shared memory per CTA");
   auto k = render_tc_kernel<P, NCH, GR, FWD, BWD>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
@@ -1436,7 +1443,7 @@ gs_status launch_tc_t(const gs_ctx* ctx, RenderTcArgs& a, cudaStream_t st) {
 template <class P, int NCH>
 gs_status launch_tc_n(const gs_ctx* ctx, RenderTcArgs& a, int mode, cudaStream_t st) {
   constexpr int GR = kRenderGroups;  // tile groups in one CTA per SM
-  if (mode == 1) return launch_tc_t<P, NCH, GR, true, false>(ctx, a, st);
+  if (mode == 1) return launch_tc_t<P, NCH, kForwardGroups, true, false>(ctx, a, st);
   if (mode == 2) return launch_tc_t<P, NCH, GR, false, true>(ctx, a, st);
   return launch_tc_t<P, NCH, GR, true, true>(ctx, a, st);
 }
