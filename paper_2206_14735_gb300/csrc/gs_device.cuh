@@ -124,9 +124,6 @@ __device__ __forceinline__ long long corner_offset(const GridDesc& g, int l, int
          (c & 1) * (long long)g.dims[l][0] * g.dims[l][1];
 }
 
-__device__ __forceinline__ float4 f4add(float4 a, float4 b) {
-  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
 __device__ __forceinline__ float4 f4scale(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
 __device__ __forceinline__ void f4fma(float4& acc, float s, float4 b) {
   acc.x = fmaf(s, b.x, acc.x);

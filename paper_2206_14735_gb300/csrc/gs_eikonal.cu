@@ -264,8 +264,6 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
   const int gi = warp >> 2, warp_g = warp & 3;
   uint8_t* gb = base + gi * kEtGroupBytes;
   Group G;
-  G.a = gb + oZ;
-  G.b = gb + oJ;
   G.mbar = &ms.mbar[gi];
   G.mbar_dw = &ms.mbar_dw[gi];
   G.abort = &ms.abort[gi];
@@ -567,8 +565,6 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
   const int gi = warp >> 2, warp_g = warp & 3;
   uint8_t* gb = base + gi * kEpGroupBytes;
   Group G;
-  G.a = gb + qR1;
-  G.b = gb + qPM;
   G.mbar = &ms.mbar[gi];
   G.mbar_dw = &ms.mbar_dw[gi];
   G.abort = &ms.abort[gi];

@@ -90,7 +90,6 @@ __global__ void __launch_bounds__(kItThreads, 1) importance_tc_kernel(ImpArgs a,
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = warp >> 2, warp_g = warp & 3;
   Group G;
-  G.a = G.b = nullptr;
   G.mbar = &mbar[gi];
   G.mbar_dw = &mbar[gi];
   G.abort = &abort_flag[gi];

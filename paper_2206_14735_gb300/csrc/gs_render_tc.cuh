@@ -211,12 +211,6 @@ __device__ __forceinline__ void store_row_planes(uint8_t* planes, int row, const
   for (int c = 0; c < K / 8; ++c) store_chunk<NPL, K, PLANE_BYTES>(planes, row, c, v + 8 * c);
 }
 
-// a row of the A operand tile of the decoder phases
-template <class P, int K>
-__device__ __forceinline__ void store_row(uint8_t* planes, int row, const float* v) {
-  store_row_planes<P::planes, K, 128u * 32u * P::es>(planes, row, v);
-}
-
 // one element of a weight tile (planes `wplane` bytes apart)
 template <class P>
 __device__ __forceinline__ void store_w(uint8_t* planes, uint32_t wplane, int K, int n, int k, float v) {
@@ -226,33 +220,6 @@ __device__ __forceinline__ void store_w(uint8_t* planes, uint32_t wplane, int K,
   split_bf16<P::planes>(v, e);
 #pragma unroll
   for (int pl = 0; pl < P::planes; ++pl) *reinterpret_cast<__nv_bfloat16*>(planes + pl * wplane + off) = e[pl];
-}
-
-// D[128][N] (+)= A[128][K] * B[N][K]^T over the part products i + j < planes, one thread.  The
-// operand descriptors of the series are the first one's plus constants: built from their
-// addresses each, the issuing thread spent about 15 instructions per MMA, which the whole
-// group waits for.
-template <class P, int N, int K>
-__device__ __forceinline__ void issue_mma(uint32_t d, uint32_t a0, uint32_t b0, uint32_t wplane) {
-  constexpr uint32_t sbo = (uint32_t)(K * P::es / 16) * 128u;
-  constexpr uint32_t idesc = tc::instr_desc(P::kind, 128, N);
-  constexpr uint32_t aplane = 128u * 32u * P::es;
-  const uint32_t alo = tc::desc_lo(a0, 128u), blo = tc::desc_lo(b0, 128u);
-  bool first = true;
-#pragma unroll
-  for (int s = 0; s < K / P::kmma; ++s) {
-    const uint32_t off = (uint32_t)s * 256u;  // two 16-byte core-matrix columns per K step
-    // smallest part products first
-#pragma unroll
-    for (int sum = P::planes - 1; sum >= 0; --sum)
-#pragma unroll
-      for (int i = 0; i <= sum; ++i) {
-        const int jj = sum - i;
-        tc::mma_bf16(d, tc::desc_of(alo + ((i * aplane + off) >> 4), tc::desc_hi(sbo)),
-                     tc::desc_of(blo + ((jj * wplane + off) >> 4), tc::desc_hi(sbo)), idesc, first ? 0u : 1u);
-        first = false;
-      }
-  }
 }
 
 // Decoder weight gradients on the tensor core: D[64][N] (+)= sum over the tile's 128 samples
@@ -281,7 +248,9 @@ __device__ __forceinline__ void issue_mma_dw(uint32_t d, uint32_t a0, uint32_t a
   }
 }
 
-// The compact kernel's phase product: D[128][N] = A[128][K] B[N][K]^T, A in tensor memory
+// The compact kernel's phase product: D[128][N] = A[128][K] B[N][K]^T, A in tensor memory.  The operand
+// descriptors of a series are the first one's plus constants: built from their addresses each, the
+// issuing thread spent about 15 instructions per MMA, which the whole group waits for.
 template <class P, int N, int K>
 __device__ __forceinline__ void tile_mma(uint32_t d, uint32_t ta, uint32_t b0, uint32_t wplane) {
   constexpr uint32_t idesc = tc::instr_desc(P::kind, 128, N);
@@ -323,8 +292,6 @@ __device__ __forceinline__ void tile_mma_dw(uint32_t d, uint32_t a0, uint32_t b0
 
 // per-group MMA machinery
 struct Group {
-  uint8_t* a;  // A operand planes
-  uint8_t* b;  // partner planes of the weight-gradient products
   uint64_t* mbar;     // completion of the phase MMAs (issued by thread 0 of the group)
   uint64_t* mbar_dw;  // completion of the weight-gradient MMAs (issued by thread 32)
   int* abort;
@@ -655,21 +622,6 @@ __device__ __forceinline__ void scatter_direct(const GridDesc& g, float* grad, i
       if (e.any) f4fma(cv, dd[k], q4);
       red_add_f4(row[k & 3] + (k >> 2), cv);
     }
-  }
-}
-
-// All four levels by one warp (st: its kScatterStage floats)
-__device__ __forceinline__ void scatter_dz(const GridDesc& g, float* grad, const float x[3], const float dz[kZ],
-                                           bool valid, float* st, const float4* er = nullptr, long long es = 0) {
-  const unsigned active = __ballot_sync(0xffffffffu, valid);
-  if (active == 0) return;
-  const EikSeed e = eik_seed(er, es);
-#pragma unroll
-  for (int l = 0; l < kLevels; ++l) {
-    const float4 g4 = valid ? make_float4(dz[4 * l], dz[4 * l + 1], dz[4 * l + 2], dz[4 * l + 3])
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (l < 2) scatter_runs(g, grad, l, x, g4, valid, st, e);
-    else scatter_direct<false>(g, grad, l, x, g4, valid, e);
   }
 }
 
