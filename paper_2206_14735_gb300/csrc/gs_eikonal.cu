@@ -35,6 +35,13 @@
 //      about 3e10 16-byte reductions per second, and the fine levels need 16 per sample),
 //      so the deferred form leaves it the gathers and the tensor-core phases.
 // The loss is summed per CTA and combined in FP64 by the last CTA to finish.
+//
+// Both kernels are bound by their gathers, through L1, at 12 to 16 warps per SM.  The phases' A
+// operands lie in tensor memory: as shared-memory tiles they took 225 KB (this decoder) and 211 KB
+// (the paper's) of the SM's 256 KB that L1 shares, and every product read them through the data
+// path that the gathers load; only the weight-gradient products' operands are left there (165
+// and 192 KB).  Deferred form, room batch of 8192 x 96: 0.113 -> 0.065 ms a call (this decoder, the
+// division-free cells included); the paper's method at 8192 x 132: 1920 -> 1875 us a step.
 #include <algorithm>
 
 #include "gs_paper.cuh"
@@ -47,20 +54,20 @@ constexpr int kEtGroups = 4;                  // 16 warps per SM at one CTA per 
 constexpr int kEtThreads = kEtGroups * kGroupThreads;
 constexpr int kEtRunLevels = 2;               // levels scattered after a run reduction
 constexpr int kEtSt = 36;                     // staging row: 8 corner vectors | run key | pad
-constexpr uint32_t kZPlane = 128u * kZ * 2u;  // Z tile (K = 16), one bfloat16 part
 constexpr uint32_t kMTile = 128u * kH1 * 2u;  // mask tile (K = 32), exact in bfloat16
 constexpr uint32_t kJPlane = 128u * kZ * 2u;  // j tile (K = 16), one bfloat16 part
 constexpr uint32_t kStageBytes = 4u * 32u * kEtSt * 4u;
-// per group: Z (3 parts) | M | J (3 parts) | staging rows.  The M = 64 reads of the mask tile
+// per group: M | J (3 parts) | staging rows.  The M = 64 reads of the mask tile
 // run up to 512 bytes past its end, into the J tile (rows 32.. of C, which are not used).
-constexpr uint32_t oZ = 0, oM = oZ + 3u * kZPlane, oJ = oM + kMTile, oS = oJ + 3u * kJPlane;
+constexpr uint32_t oM = 0, oJ = oM + kMTile, oS = oJ + 3u * kJPlane;
 constexpr uint32_t kEtGroupBytes = oS + kStageBytes;
 constexpr uint32_t kW1Plane = kH1 * kZ * 2u;  // B of H = Z W1^T: {N = 32, K = 16}
 constexpr uint32_t kVPlane = kZ * kH1 * 2u;   // B of P = M V: {N = 16, K = 32}
 constexpr uint32_t oW1t = kEtGroups * kEtGroupBytes, oVt = oW1t + 3u * kW1Plane, oMisc = oVt + 3u * kVPlane;
-// tensor-memory columns of a group: H (N = 32), P (N = 16), C (M = 64 layout, N = 16)
-constexpr uint32_t cH = 0, cP = 32, cC = 48, kEtCols = 64;
-constexpr uint32_t kEtTmem = 256;  // a power of two >= kEtGroups * kEtCols
+// tensor-memory columns of a group: H (N = 32), P (N = 16), C (M = 64 layout, N = 16), the phases'
+// A operand (three parts of Z, or M)
+constexpr uint32_t cH = 0, cP = 32, cC = 48, cOp = 64, kEtCols = 88;
+constexpr uint32_t kEtTmem = 512;  // a power of two >= kEtGroups * kEtCols
 static_assert(kEtGroups * kEtCols <= kEtTmem, "tensor-memory columns");
 
 struct EtMisc {
@@ -137,39 +144,64 @@ __global__ void __launch_bounds__(kCompactThreads) eik_compact_kernel(const uint
     if (fs[k]) list[pos++] = (int)(s0 + k);
 }
 
-// D[128][N] (+)= sum of the part products A_i B_j^T (i < APL, j < BPL, i + j < SUM), smallest
-// first; A [128][K] and B [N][K] K-major without swizzle, parts `a_plane` / `b_plane` apart
-template <int APL, int BPL, int SUM, int N, int K>
-__device__ __forceinline__ void et_mma(uint32_t d, uint32_t a0, uint32_t a_plane, uint32_t b0, uint32_t b_plane) {
-  constexpr uint32_t sbo = (uint32_t)(K * 2 / 16) * 128u;
+// D[128][N] = sum of the part products A_i B_j^T (i < APL, j < BPL, i + j < 3), smallest first;
+// A [128][K] in tensor memory (part i in columns ta + i K / 2 ..), B [N][K] K-major without
+// swizzle, parts `b_plane` apart
+template <int APL, int BPL, int N, int K>
+__device__ __forceinline__ void et_mma(uint32_t d, uint32_t ta, uint32_t b0, uint32_t b_plane) {
   constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 128, N);
+  const uint32_t blo = tc::desc_lo(b0, 128u);
   bool first = true;
 #pragma unroll
-  for (int s = 0; s < K / 16; ++s) {
-    const uint32_t off = (uint32_t)s * 256u;
+  for (int s = 0; s < K / 16; ++s)
 #pragma unroll
-    for (int sum = SUM - 1; sum >= 0; --sum)
+    for (int sum = 2; sum >= 0; --sum)
 #pragma unroll
       for (int i = 0; i <= sum; ++i) {
         const int j = sum - i;
         if (i >= APL || j >= BPL) continue;
-        tc::mma_bf16(d, tc::smem_desc(a0 + i * a_plane + off, 128u, sbo), tc::smem_desc(b0 + j * b_plane + off, 128u, sbo),
-                     idesc, first ? 0u : 1u);
+        tc::mma_bf16_ta(d, ta + (uint32_t)(i * (K / 2) + s * 8),
+                        tc::desc_of(blo + ((j * b_plane + s * 256u) >> 4), tc::desc_hi(K * 16u)), idesc, first ? 0u : 1u);
         first = false;
       }
+}
+
+// This thread's row of an operand: its first TPL parts into tensor memory (ta: the warp's lanes, the
+// operand's first column; all lanes together), its first SPL parts into a shared-memory tile of
+// the weight-gradient products
+template <int TPL, int SPL, int K, uint32_t PLANE>
+__device__ __forceinline__ void put_row(uint32_t ta, uint8_t* planes, int row, const float* v) {
+  constexpr int PL = TPL > SPL ? TPL : SPL;
+  constexpr uint32_t sbo = (uint32_t)(K / 8) * 128u;
+#pragma unroll
+  for (int c = 0; c < K / 16; ++c) {
+    uint32_t w[PL][8];
+    split_words<PL, 8>(v + 16 * c, w);
+#pragma unroll
+    for (int pl = 0; pl < TPL; ++pl) tc::tmem_st(ta + (uint32_t)(pl * (K / 2) + 8 * c), w[pl]);
+#pragma unroll
+    for (int pl = 0; pl < SPL; ++pl)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<uint4*>(planes + pl * PLANE + tc::core_offset((uint32_t)row, (uint32_t)(2 * c + h), 128u, sbo)) =
+            make_uint4(w[pl][4 * h], w[pl][4 * h + 1], w[pl][4 * h + 2], w[pl][4 * h + 3]);
   }
 }
 
-// rows written by every thread of the group -> thread 0 issues `mma` and commits to G.mbar
+// operand rows written by every thread of the group -> one thread of its first warp (wu == 0)
+// issues `mma` and commits to G.mbar
 template <class F>
-__device__ __forceinline__ void et_phase(Group& G, F mma) {
-  tc::fence_smem_async();
+__device__ __forceinline__ void et_phase(Group& G, int wu, F mma) {
+  tc::tmem_st_wait();
   tc::fence_before_sync();
   group_sync(G.g);
   tc::fence_after_sync();
-  if (G.gt == 0) {
-    mma();
-    tc::mma_commit(G.mbar);
+  if (wu == 0) {
+    if (tc::elect_one()) {
+      mma();
+      tc::mma_commit(G.mbar);
+    }
+    __syncwarp();
   }
 }
 
@@ -260,23 +292,25 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
   __syncthreads();
   tc::fence_after_sync();
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // uniform
   const int gi = warp >> 2, warp_g = warp & 3;
   uint8_t* gb = base + gi * kEtGroupBytes;
   Group G;
   G.mbar = &ms.mbar[gi];
   G.mbar_dw = &ms.mbar_dw[gi];
   G.abort = &ms.abort[gi];
-  G.tcol = ms.tslot + gi * kEtCols;
+  G.tcol = __shfl_sync(0xffffffffu, ms.tslot, 0) + (uint32_t)gi * kEtCols;
   G.phase = G.phase_dw = 0;
   G.dw_pending = false;
   G.g = gi;
   G.gt = threadIdx.x & (kGroupThreads - 1);
   const int row = G.gt;
-  uint8_t* Zt = gb + oZ;
   uint8_t* Mt = gb + oM;
   uint8_t* Jt = gb + oJ;
   float* st = reinterpret_cast<float*>(gb + oS) + warp_g * 32 * kEtSt;
+  const uint32_t op = G.tcol + cOp, ta = lane_addr(G, cOp, warp_g);
+  const uint32_t sW1 = tc::smem_u32(W1t), sV = tc::smem_u32(Vt);
   const bool bwd = a.grad != nullptr;
   const int n_fs = a.counts[2];
   const float k_eik = n_fs > 0 ? a.dloss[0] * -2.0f / (float)n_fs : 0.0f;
@@ -342,11 +376,12 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
         z[4 * l + 2] = zz.z;
         z[4 * l + 3] = zz.w;
       }
-      store_row_planes<3, kZ, kZPlane>(Zt, row, z);
+      __syncwarp();
+      put_row<3, 0, kZ, 0>(ta, nullptr, row, z);
     }
     ray_of(s_nx, o_nx, r_nx, t_nx);  // the next tile's ray, in flight during the tensor-core phases
     // ---- 2. H = Z W1^T; the mask ----
-    et_phase(G, [&] { et_mma<3, 3, 3, kH1, kZ>(G.tcol + cH, tc::smem_u32(Zt), kZPlane, tc::smem_u32(W1t), kW1Plane); });
+    et_phase(G, warp_g, [&] { et_mma<3, 3, kH1, kZ>(G.tcol + cH, op, sW1, kW1Plane); });
     if (!(alive = mma_phase_wait(G))) break;
     {
       float h[kH1];
@@ -355,10 +390,11 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
 #pragma unroll
       for (int j = 0; j < kH1; ++j) h[j] = __fadd_rn(h[j], ms.b1[j]) > 0.f ? 1.f : 0.f;
       dw_wait(G);  // the mask and j tiles are free once the last C product has read them
-      store_row_planes<1, kH1, kMTile>(Mt, row, h);
+      __syncwarp();
+      put_row<1, 1, kH1, kMTile>(ta, Mt, row, h);
     }
     // ---- 3. P = M V ----
-    et_phase(G, [&] { et_mma<1, 3, 3, kZ, kH1>(G.tcol + cP, tc::smem_u32(Mt), kMTile, tc::smem_u32(Vt), kVPlane); });
+    et_phase(G, warp_g, [&] { et_mma<1, 3, kZ, kH1>(G.tcol + cP, op, sV, kVPlane); });
     if (!(alive = mma_phase_wait(G))) break;
     float p[kZ];
     tc::tmem_ld16(lane_addr(G, cP, warp_g), p);
@@ -406,10 +442,13 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
       tc::fence_before_sync();
       group_sync(gi);
       tc::fence_after_sync();
-      if (G.gt == 32) {
-        issue_mma_dw<1, 3, 3, kZ>(G.tcol + cC, tc::smem_u32(Mt), kMTile, 4u * 128u, tc::smem_u32(Jt), kJPlane, 2u * 128u,
-                                  dw_acc);
-        tc::mma_commit(G.mbar_dw);
+      if (warp_g == 1) {
+        if (tc::elect_one()) {
+          issue_mma_dw<1, 3, 3, kZ>(G.tcol + cC, tc::smem_u32(Mt), kMTile, 4u * 128u, tc::smem_u32(Jt), kJPlane,
+                                    2u * 128u, dw_acc);
+          tc::mma_commit(G.mbar_dw);
+        }
+        __syncwarp();
       }
       G.dw_pending = true;
       dw_acc = true;
@@ -496,19 +535,20 @@ constexpr int kEpGroups = 3;  // 12 warps per SM
 constexpr int kEpThreads = kEpGroups * kGroupThreads;
 constexpr uint32_t kQ32 = 128u * 32u * 2u;  // one part of a K = 32 tile
 constexpr uint32_t kQ16 = 128u * 16u * 2u;  // one part of a K = 16 tile
-// per group: R1 (Z, then A1, then VJ: 3 parts; the coarse scatter's staging while VJ runs) |
-// M2 (exact, 1 part) | PM (3 parts) | J (2 parts).  The M = 64 reads of M2 and PM run 512 bytes
-// past a part's end, into the next part or tile.
-constexpr uint32_t qR1 = 0, qM2 = 3 * kQ32, qPM = qM2 + kQ32, qJ = qPM + 3 * kQ32;
+// per group, the weight-gradient products' operands: VJ (3 parts; the coarse scatter's staging while
+// its product runs) | M2 (exact, 1 part) | PM (2 parts) | J (2 parts).  The M = 64 reads of M2 and
+// PM run 512 bytes past a part's end, into the next part or tile.
+constexpr uint32_t qR1 = 0, qM2 = 3 * kQ32, qPM = qM2 + kQ32, qJ = qPM + 2 * kQ32;
 constexpr uint32_t kEpGroupBytes = qJ + 2 * kQ16;
-static_assert(4u * 32u * kEtSt * 4u <= 3u * kQ32, "scatter staging fits in R1");
+static_assert(4u * 32u * kEtSt * 4u <= 3u * kQ32, "scatter staging fits in the VJ tile");
 // weight tiles {N, K}: gW1 32x16 | gW2 32x32 | V2 {k, j} 32x32 | gW1^T {k, j} 16x32; 3 parts
 constexpr uint32_t qW1 = 0, qW2 = qW1 + 32u * 16u * 2u, qV2 = qW2 + 32u * 32u * 2u, qW1T = qV2 + 32u * 32u * 2u,
                    kQW = qW1T + 16u * 32u * 2u;
 constexpr uint32_t oQW = kEpGroups * kEpGroupBytes, oQMisc = oQW + 3 * kQW;
-// tensor-memory columns of a group: phase outputs, C1 (N = 16), C2 (N = 32)
-constexpr uint32_t eH = 0, eC1 = 32, eC2 = 48, kEpCols = 80;
-static_assert(kEpGroups * kEpCols <= 256, "tensor-memory columns");
+// tensor-memory columns of a group: phase outputs, C1 (N = 16), C2 (N = 32), the phases' A operand
+constexpr uint32_t eH = 0, eC1 = 32, eC2 = 48, eOp = 80, kEpCols = 128;
+constexpr uint32_t kEpTmem = 512;  // a power of two >= kEpGroups * kEpCols
+static_assert(kEpGroups * kEpCols <= kEpTmem, "tensor-memory columns");
 
 struct EpMisc {
   float b1[32];
@@ -555,20 +595,21 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
     }
     tc::fence_mbar_init();
   }
-  if (threadIdx.x < 32) tc::tmem_alloc(&ms.tslot, 256);
+  if (threadIdx.x < 32) tc::tmem_alloc(&ms.tslot, kEpTmem);
   tc::fence_smem_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // uniform
   const int gi = warp >> 2, warp_g = warp & 3;
   uint8_t* gb = base + gi * kEpGroupBytes;
   Group G;
   G.mbar = &ms.mbar[gi];
   G.mbar_dw = &ms.mbar_dw[gi];
   G.abort = &ms.abort[gi];
-  G.tcol = ms.tslot + gi * kEpCols;
+  G.tcol = __shfl_sync(0xffffffffu, ms.tslot, 0) + (uint32_t)gi * kEpCols;
   G.phase = G.phase_dw = 0;
   G.dw_pending = false;
   G.g = gi;
@@ -579,6 +620,9 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
   uint8_t* PM = gb + qPM;
   uint8_t* Jt = gb + qJ;
   float* st = reinterpret_cast<float*>(R1) + warp_g * 32 * kEtSt;
+  const uint32_t op = G.tcol + eOp, ta = lane_addr(G, eOp, warp_g);
+  const uint32_t sW1 = tc::smem_u32(W + qW1), sW2 = tc::smem_u32(W + qW2), sV2 = tc::smem_u32(W + qV2),
+                 sW1T = tc::smem_u32(W + qW1T);
   const bool bwd = a.grad != nullptr;
   const int n_fs = a.counts[2];
   const float k_eik = n_fs > 0 ? a.dloss[0] * -2.0f / (float)n_fs : 0.0f;
@@ -640,13 +684,13 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
         z[4 * l + 2] = zz.z;
         z[4 * l + 3] = zz.w;
       }
-      dw_wait(G);  // the previous tile's C1, C2 products have read the tiles
-      store_row_planes<3, kZ, kQ32>(R1, row, z);
+      __syncwarp();
+      put_row<3, 0, kZ, 0>(ta, nullptr, row, z);
     }
     ray_of(s_nx, o_nx, r_nx, t_nx);  // the next tile's ray, in flight during the tensor-core phases
     uint32_t m1 = 0;
     // ---- H1 = Z gW1^T: layer 1 ----
-    et_phase(G, [&] { et_mma<3, 3, 3, kH, kZ>(G.tcol + eH, tc::smem_u32(R1), kQ32, tc::smem_u32(W + qW1), kQW); });
+    et_phase(G, warp_g, [&] { et_mma<3, 3, kH, kZ>(G.tcol + eH, op, sW1, kQW); });
     if (!(alive = mma_phase_wait(G))) break;
     {
       float v[32];
@@ -658,10 +702,10 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
         m1 |= (h > 0.f ? 1u : 0u) << j;
         v[j] = fmaxf(h, 0.f);
       }
-      store_row_planes<3, kH, kQ32>(R1, row, v);
+      put_row<3, 0, kH, 0>(ta, nullptr, row, v);
     }
     // ---- H2 = A1 gW2^T: the mask of layer 2 ----
-    et_phase(G, [&] { et_mma<3, 3, 3, kH, kH>(G.tcol + eH, tc::smem_u32(R1), kQ32, tc::smem_u32(W + qW2), kQW); });
+    et_phase(G, warp_g, [&] { et_mma<3, 3, kH, kH>(G.tcol + eH, op, sW2, kQW); });
     if (!(alive = mma_phase_wait(G))) break;
     uint32_t m2 = 0;
     {
@@ -674,10 +718,12 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
         m2 |= (on ? 1u : 0u) << j;
         v[j] = on ? 1.f : 0.f;
       }
-      store_row_planes<1, kH, kQ32>(M2, row, v);
+      dw_wait(G);  // the previous tile's C1, C2 products have read the tiles
+      __syncwarp();
+      put_row<1, 1, kH, kQ32>(ta, M2, row, v);
     }
     // ---- P1 = M2 V2, pm = m1 (.) P1 ----
-    et_phase(G, [&] { et_mma<1, 3, 3, kH, kH>(G.tcol + eH, tc::smem_u32(M2), kQ32, tc::smem_u32(W + qV2), kQW); });
+    et_phase(G, warp_g, [&] { et_mma<1, 3, kH, kH>(G.tcol + eH, op, sV2, kQW); });
     if (!(alive = mma_phase_wait(G))) break;
     {
       float v[32];
@@ -685,10 +731,10 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
       tc::tmem_ld_wait();
 #pragma unroll
       for (int j = 0; j < kH; ++j) v[j] = ((m1 >> j) & 1u) ? v[j] : 0.f;
-      store_row_planes<3, kH, kQ32>(PM, row, v);
+      put_row<3, 2, kH, kQ32>(ta, PM, row, v);
     }
     // ---- P = PM gW1: the sensitivity ----
-    et_phase(G, [&] { et_mma<3, 3, 3, kZ, kH>(G.tcol + eH, tc::smem_u32(PM), kQ32, tc::smem_u32(W + qW1T), kQW); });
+    et_phase(G, warp_g, [&] { et_mma<3, 3, kZ, kH>(G.tcol + eH, op, sW1T, kQW); });
     if (!(alive = mma_phase_wait(G))) break;
     float p[kZ];
     tc::tmem_ld16(lane_addr(G, eH, warp_g), p);
@@ -726,10 +772,11 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
         jv[4 * l + 2] = av[0] * d0.z + av[1] * d1.z + av[2] * d2.z;
         jv[4 * l + 3] = av[0] * d0.w + av[1] * d1.w + av[2] * d2.w;
       }
-      store_row_planes<2, kZ, kQ16>(Jt, row, jv);
+      __syncwarp();
+      put_row<2, 2, kZ, kQ16>(ta, Jt, row, jv);
     }
     // ---- VJ = J gW1^T (vj = m1 (.) VJ); the grid scatter meanwhile ----
-    et_phase(G, [&] { et_mma<2, 3, 3, kH, kZ>(G.tcol + eH, tc::smem_u32(Jt), kQ16, tc::smem_u32(W + qW1), kQW); });
+    et_phase(G, warp_g, [&] { et_mma<2, 3, kH, kZ>(G.tcol + eH, op, sW1, kQW); });
     if (a.eik == nullptr) eik_grid_scatter(a.g, a.grad, y, p, av, kk != 0.f, st, lane);
     if (!(alive = mma_phase_wait(G))) break;  // its barrier also ends every warp's use of the staging rows
     {
@@ -745,12 +792,15 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
     tc::fence_before_sync();
     group_sync(gi);
     tc::fence_after_sync();
-    if (G.gt == 32) {
-      issue_mma_dw<2, 2, 2, kZ>(G.tcol + eC1, tc::smem_u32(PM), kQ32, 4u * 128u, tc::smem_u32(Jt), kQ16, 2u * 128u,
-                                dw_acc);
-      issue_mma_dw<1, 3, 3, kH>(G.tcol + eC2, tc::smem_u32(M2), kQ32, 4u * 128u, tc::smem_u32(R1), kQ32, 4u * 128u,
-                                dw_acc);
-      tc::mma_commit(G.mbar_dw);
+    if (warp_g == 1) {
+      if (tc::elect_one()) {
+        issue_mma_dw<2, 2, 2, kZ>(G.tcol + eC1, tc::smem_u32(PM), kQ32, 4u * 128u, tc::smem_u32(Jt), kQ16, 2u * 128u,
+                                  dw_acc);
+        issue_mma_dw<1, 3, 3, kH>(G.tcol + eC2, tc::smem_u32(M2), kQ32, 4u * 128u, tc::smem_u32(R1), kQ32, 4u * 128u,
+                                  dw_acc);
+        tc::mma_commit(G.mbar_dw);
+      }
+      __syncwarp();
     }
     G.dw_pending = true;
     dw_acc = true;
@@ -789,7 +839,7 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
   __syncthreads();
   if (warp == 0) {
     tc::fence_after_sync();
-    tc::tmem_dealloc(ms.tslot, 256);
+    tc::tmem_dealloc(ms.tslot, kEpTmem);
   }
   if (!a.loss) return;
   if (threadIdx.x == 0) {
