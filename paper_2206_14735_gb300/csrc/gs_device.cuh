@@ -235,6 +235,52 @@ __device__ __forceinline__ Cell level_jacobian(const GridDesc& g, const float* _
   return c;
 }
 
+// z at y and J = d z / d y (4 features x 3 axes a level) from one pass over the corners
+__device__ __forceinline__ void features_jacobian(const GridDesc& g, const float* __restrict__ theta, const float y[3],
+                                                  float (&z)[kZ], float4 (&J)[kLevels][3]) {
+#pragma unroll
+  for (int l = 0; l < kLevels; ++l) {
+    const Cell c = locate(g, l, y);
+    float w[8], dw[8][3];
+    corner_weights(c.f, w);
+    corner_weight_grads(c.f, c.clamped, dw);
+    const float4* base = reinterpret_cast<const float4*>(theta + g.off[l]) + c.vtx;
+    float4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = __ldg(base + corner_offset(g, l, k));
+    float4 zz = make_float4(0.f, 0.f, 0.f, 0.f);
+    J[l][0] = J[l][1] = J[l][2] = zz;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      f4fma(zz, w[k], v[k]);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) f4fma(J[l][q], dw[k][q], v[k]);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) J[l][q] = f4scale(J[l][q], g.inv_voxel[l]);
+    z[4 * l] = zz.x;
+    z[4 * l + 1] = zz.y;
+    z[4 * l + 2] = zz.z;
+    z[4 * l + 3] = zz.w;
+  }
+}
+// W1's row j as four 16-byte broadcast reads; s + its product with v, in the order of v
+__device__ __forceinline__ void w1_row(const float* sm, int j, float (&w)[kZ]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float4 t = *reinterpret_cast<const float4*>(sm + sW1 + j * kZ + 4 * q);
+    w[4 * q] = t.x;
+    w[4 * q + 1] = t.y;
+    w[4 * q + 2] = t.z;
+    w[4 * q + 3] = t.w;
+  }
+}
+__device__ __forceinline__ float w1_dot(const float (&w)[kZ], const float (&v)[kZ], float s) {
+#pragma unroll
+  for (int k = 0; k < kZ; ++k) s = fmaf(w[k], v[k], s);
+  return s;
+}
+
 // warp reductions
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

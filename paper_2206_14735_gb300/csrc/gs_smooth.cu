@@ -6,8 +6,15 @@
 // For an adjoint a = dL/d(grad phi) at a point y:
 //   d/d theta_{l,c,k} = p_{l,k} (1/v_l) (a . dw_c/df)       (Supp. Eq. second_order_theta)
 //   d/d W1 = (m (.) W2[0,:]) j^T,  d/d W2[0,:] = m (.) (W1 j), j_k = a . d z_k / d x.
-// One lane per point; a warp stages its 32 points' vectors and reduces the decoder
-// gradients as 4x4 tiles, as the render kernel does.
+// One lane per evaluation; a warp stages its 32 evaluations' vectors and reduces the decoder
+// gradients as 4x4 tiles.
+//
+// Bound by latency: 4096 points are one pass of every warp, in the render kernel's shadow only where that
+// leaves SMs idle.  Hence one visit of the corners for z and dz/dx (three before: features, gradient
+// and adjoint each gathered again), W1's rows read once as 16-byte vectors for the unit, its mask
+// and its part of p, the points dealt over the blocks first, and nothing spilled (568 bytes of
+// stack a thread before).  Step of 1024 rays x 64 with its 1024 points: 130 -> 125 us; the query's
+// backward pass of 4096 points, cold: 28 -> 25 us.
 #include <algorithm>
 
 #include "gs_internal.h"
@@ -34,56 +41,6 @@ struct SmoothRunArgs {
 
 __device__ __forceinline__ float4 ldv(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-// z at y (all levels), values only
-__device__ __forceinline__ void features_only(const GridDesc& g, const float* __restrict__ theta, const float y[3],
-                                              float z[kZ]) {
-#pragma unroll
-  for (int l = 0; l < kLevels; ++l) {
-    const Cell c = locate(g, l, y);
-    float w[8];
-    corner_weights(c.f, w);
-    const float4* base = reinterpret_cast<const float4*>(theta + g.off[l]);
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) f4fma(acc, w[k], __ldg(base + c.vtx + corner_offset(g, l, k)));
-    z[4 * l] = acc.x;
-    z[4 * l + 1] = acc.y;
-    z[4 * l + 2] = acc.z;
-    z[4 * l + 3] = acc.w;
-  }
-}
-// ReLU mask m (bit j = unit j on), m (.) W2[0,:], and p = d phi / d z
-__device__ __forceinline__ unsigned phi_sensitivity(const float* sm, const float z[kZ], float mw2[kH1], float p[kZ]) {
-  unsigned mask = 0;
-#pragma unroll
-  for (int j = 0; j < kH1; ++j) {
-    float s = sm[sb1 + j];
-#pragma unroll
-    for (int k = 0; k < kZ; ++k) s = fmaf(sm[sW1 + j * 16 + k], z[k], s);
-    mw2[j] = s > 0.f ? sm[sW2 + j] : 0.f;
-    mask |= (s > 0.f ? 1u : 0u) << j;
-  }
-#pragma unroll
-  for (int k = 0; k < kZ; ++k) {
-    float s = 0.f;
-#pragma unroll
-    for (int j = 0; j < kH1; ++j) s = fmaf(sm[sW1 + j * 16 + k], mw2[j], s);
-    p[k] = s;
-  }
-  return mask;
-}
-
-// layer-1 ReLU output a1 = max(W1 z + b1, 0) of the SDF decoder
-__device__ __forceinline__ void sdf_layer1(const float* sm, const float z[kZ], float a1[kH1]) {
-#pragma unroll
-  for (int j = 0; j < kH1; ++j) {
-    float s = sm[sb1 + j];
-#pragma unroll
-    for (int k = 0; k < kZ; ++k) s = fmaf(sm[sW1 + j * 16 + k], z[k], s);
-    a1[j] = fmaxf(s, 0.f);
-  }
-}
-
 template <bool FWD, bool BWD>
 __global__ void __launch_bounds__(kSmoothWarps * 32, 1) smooth_kernel(SmoothRunArgs a) {
   __shared__ __align__(16) float sm[kSmemMlp];
@@ -107,29 +64,43 @@ __global__ void __launch_bounds__(kSmoothWarps * 32, 1) smooth_kernel(SmoothRunA
 
   // one lane per gradient evaluation: lanes 2q and 2q+1 evaluate point q at x and x + eps
 #pragma unroll 1
-  for (int base = (blockIdx.x * kSmoothWarps + warp) * 16; base < a.P; base += gridDim.x * kSmoothWarps * 16) {
+  for (int base = (warp * gridDim.x + blockIdx.x) * 16; base < a.P; base += gridDim.x * kSmoothWarps * 16) {
     const int p = base + (lane >> 1), e = lane & 1;
     const bool valid = p < a.P && a.valid[p];
     float y[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) y[k] = valid ? (e == 0 ? a.xs[3 * p + k] : __fadd_rn(a.xs[3 * p + k], a.eps[3 * p + k])) : 0.f;
-    float pz[kZ], mw2[kH1];
-    unsigned mask;
+    float4 J[kLevels][3];
+    float pz[kZ];           // p = d phi / d z
+    unsigned mask = 0;      // ReLU mask m (bit j = unit j on)
+    float* row = st + lane * kSt;
     {
       float z[kZ];
-      features_only(a.g, a.theta, y, z);
-      mask = phi_sensitivity(sm, z, mw2, pz);
+      features_jacobian(a.g, a.theta, y, z, J);
+#pragma unroll
+      for (int k = 0; k < kZ; ++k) pz[k] = 0.f;
+#pragma unroll 2
+      for (int j4 = 0; j4 < kH1; j4 += 4) {
+        float mw[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float w[kZ];
+          w1_row(sm, j4 + q, w);
+          const bool on = w1_dot(w, z, sm[sb1 + j4 + q]) > 0.f;
+          mw[q] = on ? sm[sW2 + j4 + q] : 0.f;
+          mask |= (on ? 1u : 0u) << (j4 + q);
+#pragma unroll
+          for (int k = 0; k < kZ; ++k) pz[k] = fmaf(w[k], mw[q], pz[k]);
+        }
+        if (BWD) *reinterpret_cast<float4*>(row + sMw2 + j4) = make_float4(mw[0], mw[1], mw[2], mw[3]);
+      }
     }
     float gq[3] = {0.f, 0.f, 0.f};  // grad_x phi = sum_l (dz_l/dx)^T p_l
 #pragma unroll
-    for (int l = 0; l < kLevels; ++l) {
-      float4 dl[3];
-      float dw[8][3];
-      level_jacobian(a.g, a.theta, l, y, dl, dw);
+    for (int l = 0; l < kLevels; ++l)
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        gq[q] += pz[4 * l] * dl[q].x + pz[4 * l + 1] * dl[q].y + pz[4 * l + 2] * dl[q].z + pz[4 * l + 3] * dl[q].w;
-    }
+        gq[q] += pz[4 * l] * J[l][q].x + pz[4 * l + 1] * J[l][q].y + pz[4 * l + 2] * J[l][q].z + pz[4 * l + 3] * J[l][q].w;
     float dg[3];  // g(x) - g(x + eps), on both lanes of the pair
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -141,18 +112,21 @@ __global__ void __launch_bounds__(kSmoothWarps * 32, 1) smooth_kernel(SmoothRunA
     const float sgn = e == 0 ? 1.f : -1.f;
     const float av[3] = {valid ? sgn * k_sm * dg[0] : 0.f, valid ? sgn * k_sm * dg[1] : 0.f,
                          valid ? sgn * k_sm * dg[2] : 0.f};
-    // per level: j_l = a . dz_l/dx, and the direct term d/d theta_{l,c,k} = p_{l,k} (1/v_l) (a . dw_c/df)
-    float jv[kZ];
+    float jv[kZ];  // j_l = a . dz_l/dx
 #pragma unroll
     for (int l = 0; l < kLevels; ++l) {
-      float4 dl[3];
-      float dw[8][3];
-      const Cell c = level_jacobian(a.g, a.theta, l, y, dl, dw);
-      jv[4 * l] = av[0] * dl[0].x + av[1] * dl[1].x + av[2] * dl[2].x;
-      jv[4 * l + 1] = av[0] * dl[0].y + av[1] * dl[1].y + av[2] * dl[2].y;
-      jv[4 * l + 2] = av[0] * dl[0].z + av[1] * dl[1].z + av[2] * dl[2].z;
-      jv[4 * l + 3] = av[0] * dl[0].w + av[1] * dl[1].w + av[2] * dl[2].w;
-      if (valid) {
+      const float4 d0 = J[l][0], d1 = J[l][1], d2 = J[l][2];
+      jv[4 * l] = av[0] * d0.x + av[1] * d1.x + av[2] * d2.x;
+      jv[4 * l + 1] = av[0] * d0.y + av[1] * d1.y + av[2] * d2.y;
+      jv[4 * l + 2] = av[0] * d0.z + av[1] * d1.z + av[2] * d2.z;
+      jv[4 * l + 3] = av[0] * d0.w + av[1] * d1.w + av[2] * d2.w;
+    }
+    if (valid) {  // the direct term d/d theta_{l,c,k} = p_{l,k} (1/v_l) (a . dw_c/df)
+#pragma unroll
+      for (int l = 0; l < kLevels; ++l) {
+        const Cell c = locate(a.g, l, y);
+        float dw[8][3];
+        corner_weight_grads(c.f, c.clamped, dw);
         const float iv = a.g.inv_voxel[l];
         const float4 p4 = make_float4(pz[4 * l], pz[4 * l + 1], pz[4 * l + 2], pz[4 * l + 3]);
 #pragma unroll
@@ -162,22 +136,21 @@ __global__ void __launch_bounds__(kSmoothWarps * 32, 1) smooth_kernel(SmoothRunA
         }
       }
     }
-    float* row = st + lane * kSt;
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      *reinterpret_cast<float4*>(row + sMw2 + 4 * q) = make_float4(mw2[4 * q], mw2[4 * q + 1], mw2[4 * q + 2], mw2[4 * q + 3]);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       *reinterpret_cast<float4*>(row + sJ + 4 * q) = make_float4(jv[4 * q], jv[4 * q + 1], jv[4 * q + 2], jv[4 * q + 3]);
     // d/d W2[0][j] = m_j (W1 j)_j
+#pragma unroll 2
+    for (int j4 = 0; j4 < kH1; j4 += 4) {
+      float u[4];
 #pragma unroll
-    for (int j = 0; j < kH1; ++j) {
-      float u = 0.f;
-      if ((mask >> j) & 1u) {
-#pragma unroll
-        for (int k = 0; k < kZ; ++k) u = fmaf(sm[sW1 + j * 16 + k], jv[k], u);
+      for (int q = 0; q < 4; ++q) {
+        float w[kZ];
+        w1_row(sm, j4 + q, w);
+        u[q] = w1_dot(w, jv, 0.f);
+        if (!((mask >> (j4 + q)) & 1u)) u[q] = 0.f;
       }
-      row[sU + j] = u;
+      *reinterpret_cast<float4*>(row + sU + j4) = make_float4(u[0], u[1], u[2], u[3]);
     }
     __syncwarp();
     {  // dW1[32][16] += mw2 (x) j over the warp's 32 evaluations
@@ -261,22 +234,44 @@ __global__ void __launch_bounds__(kSmoothWarps * 32) query_backward_kernel(Query
     float av[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) av[k] = (valid && a.dgrad) ? a.dgrad[3 * p + k] : 0.f;
-    float z[kZ], a1[kH1], mw2[kH1], pz[kZ];
-    features_only(a.g, a.theta, y, z);
-    sdf_layer1(sm, z, a1);
-    const unsigned mask = phi_sensitivity(sm, z, mw2, pz);
-    float jv[kZ];
+    float z[kZ], jv[kZ], pz[kZ];
+    {
+      float4 J[kLevels][3];
+      features_jacobian(a.g, a.theta, y, z, J);
 #pragma unroll
-    for (int l = 0; l < kLevels; ++l) {
-      float4 dl[3];
-      float dw[8][3], w[8];
-      const Cell c = level_jacobian(a.g, a.theta, l, y, dl, dw);
-      corner_weights(c.f, w);
-      jv[4 * l] = av[0] * dl[0].x + av[1] * dl[1].x + av[2] * dl[2].x;
-      jv[4 * l + 1] = av[0] * dl[0].y + av[1] * dl[1].y + av[2] * dl[2].y;
-      jv[4 * l + 2] = av[0] * dl[0].z + av[1] * dl[1].z + av[2] * dl[2].z;
-      jv[4 * l + 3] = av[0] * dl[0].w + av[1] * dl[1].w + av[2] * dl[2].w;
-      if (valid) {
+      for (int l = 0; l < kLevels; ++l) {
+        const float4 d0 = J[l][0], d1 = J[l][1], d2 = J[l][2];
+        jv[4 * l] = av[0] * d0.x + av[1] * d1.x + av[2] * d2.x;
+        jv[4 * l + 1] = av[0] * d0.y + av[1] * d1.y + av[2] * d2.y;
+        jv[4 * l + 2] = av[0] * d0.z + av[1] * d1.z + av[2] * d2.z;
+        jv[4 * l + 3] = av[0] * d0.w + av[1] * d1.w + av[2] * d2.w;
+        pz[4 * l] = pz[4 * l + 1] = pz[4 * l + 2] = pz[4 * l + 3] = 0.f;
+      }
+    }
+    float* row = st + lane * kSt;
+#pragma unroll 2
+    for (int j4 = 0; j4 < kH1; j4 += 4) {
+      float mw[4], u[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float w[kZ];
+        w1_row(sm, j4 + q, w);
+        const float s = w1_dot(w, z, sm[sb1 + j4 + q]), wj = w1_dot(w, jv, 0.f);
+        mw[q] = s > 0.f ? sm[sW2 + j4 + q] : 0.f;
+        u[q] = fmaf(ds, fmaxf(s, 0.f), s > 0.f ? wj : 0.f);
+#pragma unroll
+        for (int k = 0; k < kZ; ++k) pz[k] = fmaf(w[k], mw[q], pz[k]);
+      }
+      *reinterpret_cast<float4*>(row + sMw2 + j4) = make_float4(mw[0], mw[1], mw[2], mw[3]);
+      *reinterpret_cast<float4*>(row + sU + j4) = make_float4(u[0], u[1], u[2], u[3]);
+    }
+    if (valid) {
+#pragma unroll
+      for (int l = 0; l < kLevels; ++l) {
+        const Cell c = locate(a.g, l, y);
+        float dw[8][3], w[8];
+        corner_weights(c.f, w);
+        corner_weight_grads(c.f, c.clamped, dw);
         const float iv = a.g.inv_voxel[l];
         const float4 p4 = make_float4(pz[4 * l], pz[4 * l + 1], pz[4 * l + 2], pz[4 * l + 3]);
 #pragma unroll
@@ -286,24 +281,11 @@ __global__ void __launch_bounds__(kSmoothWarps * 32) query_backward_kernel(Query
         }
       }
     }
-    float* row = st + lane * kSt;
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      *reinterpret_cast<float4*>(row + sMw2 + 4 * q) = make_float4(mw2[4 * q], mw2[4 * q + 1], mw2[4 * q + 2], mw2[4 * q + 3]);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       *reinterpret_cast<float4*>(row + sJ + 4 * q) =
           make_float4(fmaf(ds, z[4 * q], jv[4 * q]), fmaf(ds, z[4 * q + 1], jv[4 * q + 1]),
                       fmaf(ds, z[4 * q + 2], jv[4 * q + 2]), fmaf(ds, z[4 * q + 3], jv[4 * q + 3]));
-#pragma unroll
-    for (int j = 0; j < kH1; ++j) {
-      float u = 0.f;
-      if ((mask >> j) & 1u) {
-#pragma unroll
-        for (int k = 0; k < kZ; ++k) u = fmaf(sm[sW1 + j * 16 + k], jv[k], u);
-      }
-      row[sU + j] = fmaf(ds, a1[j], u);
-    }
     row[80] = ds;
     db2 += ds;
     __syncwarp();
