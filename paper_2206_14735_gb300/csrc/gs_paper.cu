@@ -148,24 +148,10 @@ __device__ __forceinline__ void write_partials(const Args& a, const float* sG, c
 // p = gW1^T pm, pm = m1 (.) gW2^T e, e = m2 (.) gw3 (masks m1, m2 of the two hidden layers);
 // e and pm are staged in the lane's row (fields A2, A1) for grad_phi_adjoint.
 __device__ __forceinline__ void grad_phi_fwd(const Args& a, const float* sW, float* my, const float y[3],
-                                             unsigned& m1, unsigned& m2, float pz[kZ], float g[3]) {
-    // z; the x-derivatives dz/dx are gathered again level by level where they are used
-    // (keeping all 48 of them in registers beside the decoder sensitivities spills)
+                                             unsigned& m1, unsigned& m2, float pz[kZ], float g[3],
+                                             float4 (&J)[kLevels][3]) {
     float z[kZ];
-#pragma unroll
-    for (int l = 0; l < kLevels; ++l) {
-      const Cell c = locate(a.g, l, y);
-      float wv[8];
-      corner_weights(c.f, wv);
-      const float4* lv = reinterpret_cast<const float4*>(a.theta + a.g.off[l]);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) f4fma(acc, wv[k], __ldg(lv + c.vtx + corner_offset(a.g, l, k)));
-      z[4 * l] = acc.x;
-      z[4 * l + 1] = acc.y;
-      z[4 * l + 2] = acc.z;
-      z[4 * l + 3] = acc.w;
-    }
+    features_jacobian(a.g, a.theta, y, z, J);
     // forward masks; the layer-1 activations go through the lane's row (field R1, free until
     // grad_phi_adjoint) instead of 32 registers
     m1 = 0u;
@@ -190,34 +176,35 @@ __device__ __forceinline__ void grad_phi_fwd(const Args& a, const float* sW, flo
       }
       st4(my + fR1 + 4 * j4, hv[0], hv[1], hv[2], hv[3]);
     }
-#pragma unroll 1
-    for (int j = 0; j < kH; ++j) {
-      float v = sW[S_gb2 + j];
-#pragma unroll
-      for (int k4 = 0; k4 < 8; ++k4) {
-        const float4 wv = ld4(sW + S_gW2 + j * kH + 4 * k4), hv = ld4(my + fR1 + 4 * k4);
-        v = fmaf(wv.x, hv.x, v);
-        v = fmaf(wv.y, hv.y, v);
-        v = fmaf(wv.z, hv.z, v);
-        v = fmaf(wv.w, hv.w, v);
-      }
-      m2 |= (v > 0.f ? 1u : 0u) << j;
-    }
-    // e = m2 (.) gw3 (row field A2), pm = m1 (.) gW2^T e (row field A1), p = gW1^T pm
+    // layer 2's mask, e = m2 (.) gw3 (row field A2), pm = m1 (.) gW2^T e (row field A1) from one read
+    // of gW2's rows; then p = gW1^T pm
     {
+      float4 hr[8];
       float pm[kH];
 #pragma unroll
+      for (int k4 = 0; k4 < 8; ++k4) hr[k4] = ld4(my + fR1 + 4 * k4);
+#pragma unroll
       for (int k = 0; k < kH; ++k) pm[k] = 0.f;
-#pragma unroll 1
+#pragma unroll 2
       for (int j = 0; j < kH; ++j) {
-        const float e = (m2 >> j) & 1u ? sW[S_gw3 + j] : 0.f;
+        float4 wv[8];
+        float v = sW[S_gb2 + j];
 #pragma unroll
         for (int k4 = 0; k4 < 8; ++k4) {
-          const float4 wv = ld4(sW + S_gW2 + j * kH + 4 * k4);
-          pm[4 * k4] = fmaf(wv.x, e, pm[4 * k4]);
-          pm[4 * k4 + 1] = fmaf(wv.y, e, pm[4 * k4 + 1]);
-          pm[4 * k4 + 2] = fmaf(wv.z, e, pm[4 * k4 + 2]);
-          pm[4 * k4 + 3] = fmaf(wv.w, e, pm[4 * k4 + 3]);
+          wv[k4] = ld4(sW + S_gW2 + j * kH + 4 * k4);
+          v = fmaf(wv[k4].x, hr[k4].x, v);
+          v = fmaf(wv[k4].y, hr[k4].y, v);
+          v = fmaf(wv[k4].z, hr[k4].z, v);
+          v = fmaf(wv[k4].w, hr[k4].w, v);
+        }
+        m2 |= (v > 0.f ? 1u : 0u) << j;
+        const float e = v > 0.f ? sW[S_gw3 + j] : 0.f;
+#pragma unroll
+        for (int k4 = 0; k4 < 8; ++k4) {
+          pm[4 * k4] = fmaf(wv[k4].x, e, pm[4 * k4]);
+          pm[4 * k4 + 1] = fmaf(wv[k4].y, e, pm[4 * k4 + 1]);
+          pm[4 * k4 + 2] = fmaf(wv[k4].z, e, pm[4 * k4 + 2]);
+          pm[4 * k4 + 3] = fmaf(wv[k4].w, e, pm[4 * k4 + 3]);
         }
       }
 #pragma unroll
@@ -232,29 +219,28 @@ __device__ __forceinline__ void grad_phi_fwd(const Args& a, const float* sW, flo
             (m2 >> (b + 2)) & 1u ? w3.z : 0.f, (m2 >> (b + 3)) & 1u ? w3.w : 0.f);
         st4(my + fA1 + b, pm[b], pm[b + 1], pm[b + 2], pm[b + 3]);
       }
+#pragma unroll 1
+      for (int j4 = 0; j4 < kH / 4; ++j4) {
+        const float4 p4 = ld4(my + fA1 + 4 * j4);
+        const float pj[4] = {p4.x, p4.y, p4.z, p4.w};
 #pragma unroll
-      for (int j = 0; j < kH; ++j) {
-        const float pj = pm[j];
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) {
-          const float4 wv = ld4(sW + S_gW1 + j * kZ + 4 * k4);
-          pz[4 * k4] = fmaf(wv.x, pj, pz[4 * k4]);
-          pz[4 * k4 + 1] = fmaf(wv.y, pj, pz[4 * k4 + 1]);
-          pz[4 * k4 + 2] = fmaf(wv.z, pj, pz[4 * k4 + 2]);
-          pz[4 * k4 + 3] = fmaf(wv.w, pj, pz[4 * k4 + 3]);
-        }
+          for (int k4 = 0; k4 < 4; ++k4) {
+            const float4 wv = ld4(sW + S_gW1 + (4 * j4 + q) * kZ + 4 * k4);
+            pz[4 * k4] = fmaf(wv.x, pj[q], pz[4 * k4]);
+            pz[4 * k4 + 1] = fmaf(wv.y, pj[q], pz[4 * k4 + 1]);
+            pz[4 * k4 + 2] = fmaf(wv.z, pj[q], pz[4 * k4 + 2]);
+            pz[4 * k4 + 3] = fmaf(wv.w, pj[q], pz[4 * k4 + 3]);
+          }
       }
     }
     g[0] = g[1] = g[2] = 0.f;
 #pragma unroll
-    for (int l = 0; l < kLevels; ++l) {
-      float4 dl[3];
-      float dw[8][3];
-      level_jacobian(a.g, a.theta, l, y, dl, dw);
+    for (int l = 0; l < kLevels; ++l)
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        g[q] += pz[4 * l] * dl[q].x + pz[4 * l + 1] * dl[q].y + pz[4 * l + 2] * dl[q].z + pz[4 * l + 3] * dl[q].w;
-    }
+        g[q] += pz[4 * l] * J[l][q].x + pz[4 * l + 1] * J[l][q].y + pz[4 * l + 2] * J[l][q].z + pz[4 * l + 3] * J[l][q].w;
 }
 
 // The second-order adjoint (Supp. Sec. 1) of sum over the warp's lanes of a . grad_x phi(y)
@@ -264,38 +250,47 @@ __device__ __forceinline__ void grad_phi_fwd(const Args& a, const float* sW, flo
 // calls it (a lane with av = 0 adds nothing); its row holds e and pm from grad_phi_fwd.
 __device__ __forceinline__ void grad_phi_adjoint(const Args& a, const float* sW, float* sG, const float* wr, float* my,
                                                  int lane, const float y[3], bool do_grid, const float av[3],
-                                                 unsigned m1, unsigned m2, const float pz[kZ]) {
+                                                 unsigned m1, unsigned m2, const float pz[kZ],
+                                                 const float4 (&J)[kLevels][3]) {
     float jv[kZ];  // j_k = a . dz_k/dx
 #pragma unroll
     for (int l = 0; l < kLevels; ++l) {
-      float4 dl[3];
-      float dw[8][3];
-      level_jacobian(a.g, a.theta, l, y, dl, dw);
-      jv[4 * l] = av[0] * dl[0].x + av[1] * dl[1].x + av[2] * dl[2].x;
-      jv[4 * l + 1] = av[0] * dl[0].y + av[1] * dl[1].y + av[2] * dl[2].y;
-      jv[4 * l + 2] = av[0] * dl[0].z + av[1] * dl[1].z + av[2] * dl[2].z;
-      jv[4 * l + 3] = av[0] * dl[0].w + av[1] * dl[1].w + av[2] * dl[2].w;
+      jv[4 * l] = av[0] * J[l][0].x + av[1] * J[l][1].x + av[2] * J[l][2].x;
+      jv[4 * l + 1] = av[0] * J[l][0].y + av[1] * J[l][1].y + av[2] * J[l][2].y;
+      jv[4 * l + 2] = av[0] * J[l][0].z + av[1] * J[l][1].z + av[2] * J[l][2].z;
+      jv[4 * l + 3] = av[0] * J[l][0].w + av[1] * J[l][1].w + av[2] * J[l][2].w;
     }
 #pragma unroll
     for (int k4 = 0; k4 < kZ / 4; ++k4) st4(my + fZ + 4 * k4, jv[4 * k4], jv[4 * k4 + 1], jv[4 * k4 + 2], jv[4 * k4 + 3]);
     // vj = m1 (.) gW1 j (row field R1);  w3g = m2 (.) gW2 vj (row field R2)
-    {
-      float vj[kH];
+#pragma unroll 1
+    for (int j4 = 0; j4 < kH / 4; ++j4) {
+      float vj[4];
 #pragma unroll
-      for (int j = 0; j < kH; ++j) {
+      for (int q = 0; q < 4; ++q) {
         float v = 0.f;
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4) {
-          const float4 wv = ld4(sW + S_gW1 + j * kZ + 4 * k4);
+          const float4 wv = ld4(sW + S_gW1 + (4 * j4 + q) * kZ + 4 * k4);
           v = fmaf(wv.x, jv[4 * k4], v);
           v = fmaf(wv.y, jv[4 * k4 + 1], v);
           v = fmaf(wv.z, jv[4 * k4 + 2], v);
           v = fmaf(wv.w, jv[4 * k4 + 3], v);
         }
-        vj[j] = (m1 >> j) & 1u ? v : 0.f;
+        vj[q] = (m1 >> (4 * j4 + q)) & 1u ? v : 0.f;
       }
+      st4(my + fR1 + 4 * j4, vj[0], vj[1], vj[2], vj[3]);
+    }
+    {
+      float vj[kH];
 #pragma unroll
-      for (int j4 = 0; j4 < kH / 4; ++j4) st4(my + fR1 + 4 * j4, vj[4 * j4], vj[4 * j4 + 1], vj[4 * j4 + 2], vj[4 * j4 + 3]);
+      for (int j4 = 0; j4 < kH / 4; ++j4) {
+        const float4 t = ld4(my + fR1 + 4 * j4);
+        vj[4 * j4] = t.x;
+        vj[4 * j4 + 1] = t.y;
+        vj[4 * j4 + 2] = t.z;
+        vj[4 * j4 + 3] = t.w;
+      }
 #pragma unroll 1
       for (int j4 = 0; j4 < kH / 4; ++j4) {
         float vv[4];
@@ -351,6 +346,9 @@ __device__ __forceinline__ void grad_phi_adjoint(const Args& a, const float* sW,
 // The adjoint a = dL/dg gives the grid term p_{l,f} (1/v_l) (a . dw_c/df) and the decoder
 // terms gW1 += pm j^T, gW2 += e vj^T, gw3 += m2 (.) gW2 vj with j_k = a . dz_k/dx,
 // pm = m1 (.) gW2^T e, e = m2 (.) gw3, vj = m1 (.) gW1 j (biases get none).
+// Latency-bound like the compact decoder's: one visit of the corners for z and dz/dx instead of three,
+// gW2's rows read once for layer 2 and its adjoint, groups of points dealt over the blocks first.
+// 4096 points, cold: 66 -> 45 us; the step of 8192 x 96: 830 -> 825 us.
 __global__ void __launch_bounds__(kThreads, 1) paper_smooth_kernel(Args a) {
   extern __shared__ __align__(16) float smem[];
   float* sW = smem;
@@ -369,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, 1) paper_smooth_kernel(Args a) {
   const float w4 = a.dloss[4] + a.lam[4] * a.dloss[5];
   const int ev = lane >> 4;
   float lsum = 0.f;
-  for (int grp = blockIdx.x * kWarps + wid; grp * 16 < a.P; grp += gridDim.x * kWarps) {
+  for (int grp = wid * gridDim.x + blockIdx.x; grp * 16 < a.P; grp += gridDim.x * kWarps) {  // over the blocks first
     const int p = grp * 16 + (lane & 15);
     const bool ok = p < a.P && a.valid[p] != 0;
     float y[3] = {0.f, 0.f, 0.f};
@@ -379,7 +377,8 @@ __global__ void __launch_bounds__(kThreads, 1) paper_smooth_kernel(Args a) {
     }
     unsigned m1, m2;
     float pz[kZ], g[3];
-    grad_phi_fwd(a, sW, my, y, m1, m2, pz, g);
+    float4 J[kLevels][3];
+    grad_phi_fwd(a, sW, my, y, m1, m2, pz, g, J);
     float dg[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -394,7 +393,7 @@ __global__ void __launch_bounds__(kThreads, 1) paper_smooth_kernel(Args a) {
 #pragma unroll
       for (int q = 0; q < 3; ++q) av[q] = sc * dg[q];
     }
-    grad_phi_adjoint(a, sW, sG, wr, my, lane, y, ok && n_g > 0, av, m1, m2, pz);
+    grad_phi_adjoint(a, sW, sG, wr, my, lane, y, ok && n_g > 0, av, m1, m2, pz, J);
   }
   const float v = warp_sum(lsum);
   if (lane == 0) atomicAdd(sL + 4, v);
@@ -518,13 +517,14 @@ __global__ void __launch_bounds__(kThreads, 1) paper_query_backward_kernel(Args 
     if (dgrad) {  // second-order term
       unsigned m1, m2;
       float pz[kZ], g[3];
-      grad_phi_fwd(a, sW, my, y, m1, m2, pz, g);
+      float4 J[kLevels][3];
+      grad_phi_fwd(a, sW, my, y, m1, m2, pz, g, J);
       float av[3] = {0.f, 0.f, 0.f};
       if (ok) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) av[c] = dgrad[3 * p + c];
       }
-      grad_phi_adjoint(a, sW, sG, wr, my, lane, y, ok, av, m1, m2, pz);
+      grad_phi_adjoint(a, sW, sG, wr, my, lane, y, ok, av, m1, m2, pz, J);
     }
     if (dsdf) {  // first-order term: phi = gw3 . a2 + gb3, a2 = relu(gW2 a1 + gb2), a1 = relu(gW1 z + gb1)
       float z[kZ], cf[kC];
