@@ -39,6 +39,7 @@ using paper::kC;
 using paper::kH;
 using paper::kU;
 using P3 = PrecBF16x3;
+constexpr int kPaperSums = kSums + 1;  // and the SDF seeds' (the output layer's bias)
 
 // weight (B) tiles {N, K}:
 //   0 gW1 32x16 | 1 cW1 32x16 (cols 9.. zero) | 2 gW2 32x32 | 3 cW2 32x32
@@ -251,8 +252,8 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
   float4* rays0 = xch0 + (size_t)kPGroups * NCH * 128;
   float* sc = reinterpret_cast<float*>(rays0 + kPGroups * 20);
   float* kc = sc + kScal;     // loss scales of rgb, depth, sdf, fs; sharpness
-  float* sums0 = kc + 8;      // [kPGroups][4][kSums]: a compositing warp's running sums
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sums0 + kPGroups * 4 * kSums);
+  float* sums0 = kc + 8;      // [kPGroups][4][kPaperSums]: a compositing warp's running sums
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sums0 + kPGroups * 4 * kPaperSums);
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
     else if (i == sc_kappa) v = mlp[A_kappa];
     sc[i] = v;
   }
-  if (tid < kPGroups * 4 * kSums) sums0[tid] = 0.f;
+  if (tid < kPGroups * 4 * kPaperSums) sums0[tid] = 0.f;
   if (w8 == 0 && lane == 0) {
     tc::mbar_init(&T.bars->done, 1);
     tc::mbar_init(&T.bars->dw, 2);
@@ -513,7 +514,8 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
         }
       }
       const float4 in4 = *tint;
-      composite_ray<NCH, FWD, BWD>(a, ray, has_ray, tt, ph, col, clv, in4, kc, xch + row, sums0 + (gi * 4 + wq) * kSums);
+      composite_ray<NCH, FWD, BWD, kPaperSums>(a, ray, has_ray, tt, ph, col, clv, in4, kc, xch + row,
+                                               sums0 + (gi * 4 + wq) * kPaperSums);
     }
     if constexpr (!BWD) continue;
     group_sync<kTileThreads>(gi);  // the reverse pass's seeds
@@ -731,7 +733,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
   auto total = [&](int k) {  // running sum k over the compositing warps
     float v = 0.f;
 #pragma unroll
-    for (int q = 0; q < kPGroups * 4; ++q) v += sums0[q * kSums + k];
+    for (int q = 0; q < kPGroups * 4; ++q) v += sums0[q * kPaperSums + k];
     return v;
   };
   for (int i = tid; i < kPart; i += blockDim.x) {
@@ -749,7 +751,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
 template <int NCH>
 constexpr size_t paper_tc_smem() {
   constexpr size_t b = 128 + (size_t)kPGroups * kPGroupBytes + 3 * kTW + (size_t)kPGroups * NCH * 128 * 16 +
-                       kPGroups * 20 * 16 + sizeof(float) * (kScal + 8 + kPGroups * 4 * kSums) + 16;
+                       kPGroups * 20 * 16 + sizeof(float) * (kScal + 8 + kPGroups * 4 * kPaperSums) + 16;
   static_assert(b <= 227u * 1024u, "shared memory per CTA");
   return b;
 }

@@ -90,7 +90,7 @@ __host__ __device__ constexpr uint32_t tmem_cols(uint32_t columns) {
 
 constexpr int kGroupThreads = 128;  // a tile group of one thread per tile row
 constexpr int kTileThreads = 256;   // the compact render kernel's tile group: two threads per tile row
-constexpr int kSums = 9;            // running sums of a compositing warp: 4 losses, kappa, the colour and SDF seeds
+constexpr int kSums = 8;            // running sums of a compositing warp: 4 losses, kappa, the colour seeds
 constexpr uint32_t kMbarLimit = 1u << 20;  // bounded MMA-completion wait (tries of up to 2 us: ~2 s)
 
 // Shared memory per tile group: adjoint tile | partner planes of the weight-gradient products (an
@@ -694,8 +694,9 @@ __device__ __forceinline__ void get_planes(const StoreRef& s, int first, bool ge
 // NeuS compositing of one ray by one warp (lane = sample within the chunk), the losses of Sec.
 // 3.2-3.4 and, with BWD, the adjoint down to each sample's seeds: dL/d(colour pre-activations)
 // and dL/dphi into xch[128 j] of chunk j.  kc: the loss terms' scales (rgb, depth, sdf, fs) and
-// the sharpness; sums: the warp's running sums (kSums: the four losses, dL/dkappa, the seeds').
-template <int NCH, bool FWD, bool BWD, class Args>
+// the sharpness; sums: the warp's NS running sums (the four losses, dL/dkappa, the colour seeds';
+// a ninth, the SDF seeds', is only the paper architecture's).
+template <int NCH, bool FWD, bool BWD, int NS, class Args>
 __device__ __forceinline__ void composite_ray(const Args& a, int ray, bool has_ray, const float (&tt)[NCH],
                                               const float (&ph)[NCH], const float (&col)[NCH][3],
                                               const int (&clv)[NCH], const float4& seen, const float* kc, float4* xch,
@@ -858,12 +859,12 @@ __device__ __forceinline__ void composite_ray(const Args& a, int ray, bool has_r
   }
   }  // BWD
   {
-    float q[kSums] = {l_rgb, l_d, l_sdf, l_fs, g_kappa, db4[0], db4[1], db4[2], sum_d};
+    float q[9] = {l_rgb, l_d, l_sdf, l_fs, g_kappa, db4[0], db4[1], db4[2], sum_d};
 #pragma unroll
-    for (int k = 0; k < kSums; ++k) q[k] = warp_sum(q[k]);
+    for (int k = 0; k < NS; ++k) q[k] = warp_sum(q[k]);
     if (lane == 0) {
 #pragma unroll
-      for (int k = 0; k < kSums; ++k) sums[k] += q[k];
+      for (int k = 0; k < NS; ++k) sums[k] += q[k];
     }
   }
 }
@@ -1143,7 +1144,8 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       }
     }
     const float4 in4 = *tint;
-    composite_ray<NCH, FWD, BWD>(a, ray, has_ray, tt, ph, col, clv, in4, kc, xch + row, sums0 + (gi * 4 + wq) * kSums);
+    composite_ray<NCH, FWD, BWD, kSums>(a, ray, has_ray, tt, ph, col, clv, in4, kc, xch + row,
+                                        sums0 + (gi * 4 + wq) * kSums);
     }  // lower half
     if constexpr (!BWD) continue;
     group_sync<kTileThreads>(gi);  // the reverse pass's seeds
