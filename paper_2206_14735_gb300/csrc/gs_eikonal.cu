@@ -390,7 +390,6 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
 #pragma unroll
       for (int j = 0; j < kH1; ++j) h[j] = __fadd_rn(h[j], ms.b1[j]) > 0.f ? 1.f : 0.f;
       dw_wait(G);  // the mask and j tiles are free once the last C product has read them
-      __syncwarp();
       put_row<1, 1, kH1, kMTile>(ta, Mt, row, h);
     }
     // ---- 3. P = M V ----
@@ -719,7 +718,6 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
         v[j] = on ? 1.f : 0.f;
       }
       dw_wait(G);  // the previous tile's C1, C2 products have read the tiles
-      __syncwarp();
       put_row<1, 1, kH, kQ32>(ta, M2, row, v);
     }
     // ---- P1 = M2 V2, pm = m1 (.) P1 ----

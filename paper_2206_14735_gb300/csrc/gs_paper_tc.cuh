@@ -744,6 +744,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
     a.mlp_part[(size_t)blockIdx.x * kPart + i] = v;
   }
   if (tid < kLossPad) a.loss_part[(size_t)blockIdx.x * kLossPad + tid] = tid < 4 ? total(tid) : 0.f;
+  __syncwarp();
   if (warp == 0) tc::tmem_dealloc(*tslot, kPTmem);
 }
 #pragma nv_diag_default 128

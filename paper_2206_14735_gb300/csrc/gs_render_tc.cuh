@@ -122,8 +122,11 @@ struct TcLayout {
   static constexpr uint32_t row_stride(int K) { return (uint32_t)side * (uint32_t)K * 16u; }  // per 8 rows
 };
 
+// Lanes come here from polls and branches of their own (a phase's one polling lane, lane 0's sums);
+// bar.sync is an .aligned instruction, which a whole warp has to execute together.
 template <int T = kGroupThreads>
 __device__ __forceinline__ void group_sync(int g) {
+  __syncwarp();
   asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(T) : "memory");
 }
 
@@ -368,12 +371,14 @@ __device__ __forceinline__ bool phase_wait(Tile& T) {
   tc::fence_after_sync();
   return *reinterpret_cast<volatile int*>(&T.bars->abort) == 0;
 }
-// no weight-gradient product reads the tiles
+// no weight-gradient product reads the tiles.  Every lane polls by itself and may leave at another
+// try than its neighbours; the warp goes on together, as the tcgen05 instructions that follow require.
 __device__ __forceinline__ void tiles_free(Tile& T) {
   if (T.dw_pending) {
     if (!tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit)) *reinterpret_cast<volatile int*>(&T.bars->abort) = 1;
     T.ph_dw ^= 1u;
     T.dw_pending = false;
+    __syncwarp();
     tc::fence_after_sync();
   }
 }
@@ -384,6 +389,7 @@ __device__ __forceinline__ void dw_wait(Group& G) {
   if (!tc::mbar_wait(G.mbar_dw, G.phase_dw, kMbarLimit)) *reinterpret_cast<volatile int*>(G.abort) = 1;
   G.phase_dw ^= 1u;
   G.dw_pending = false;
+  __syncwarp();
   tc::fence_after_sync();
 }
 // the issuing thread waits for the MMA (bounded) while the other threads of the group park on
@@ -1371,6 +1377,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
     }
     a.mlp_part[(size_t)blockIdx.x * kMlpPad + i] = v;
   }
+  __syncwarp();
   if (warp == 0) tc::tmem_dealloc(*tslot, tmem_cols(GR * kGroupCols<BWD>));
 }
 #pragma nv_diag_default 128
