@@ -456,12 +456,14 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
     }
   }
 
-  if (!alive && G.gt == 0) {
-    atomicOr(a.status, kStatusEikonal);
-    tc::mbar_wait(G.mbar, G.phase ^ 1u, kMbarLimit);  // let an MMA in flight finish
-  }
   dw_wait(G);
   group_sync(gi);
+  if (G.gt == 0 && *reinterpret_cast<volatile int*>(G.abort) != 0) {  // a bounded wait ran out, the last one included
+    atomicOr(a.status, kStatusEikonal);
+    tc::mbar_wait(G.mbar, G.phase ^ 1u, kMbarLimit);  // let the products in flight finish
+    tc::mbar_wait(G.mbar_dw, G.phase_dw ^ 1u, kMbarLimit);
+  }
+  __syncwarp();
   // ---- epilogue: C -> dW1 = diag(w2) C and dW2[0,:] = rowsum(W1 (.) C) ----
   if (bwd && alive && dw_acc && *reinterpret_cast<volatile int*>(G.abort) == 0) {
     float c[kZ];
@@ -804,12 +806,14 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
     dw_acc = true;
   }
 
-  if (!alive && G.gt == 0) {
-    atomicOr(a.status, kStatusEikonal);
-    tc::mbar_wait(G.mbar, G.phase ^ 1u, kMbarLimit);  // let an MMA in flight finish
-  }
   dw_wait(G);
   group_sync(gi);
+  if (G.gt == 0 && *reinterpret_cast<volatile int*>(G.abort) != 0) {  // a bounded wait ran out, the last one included
+    atomicOr(a.status, kStatusEikonal);
+    tc::mbar_wait(G.mbar, G.phase ^ 1u, kMbarLimit);  // let the products in flight finish
+    tc::mbar_wait(G.mbar_dw, G.phase_dw ^ 1u, kMbarLimit);
+  }
+  __syncwarp();
   // ---- epilogue: dgW1 = C1, dgW2 = diag(gw3) C2, dgw3 = rowsum(gW2 (.) C2) ----
   if (bwd && alive && dw_acc && *reinterpret_cast<volatile int*>(G.abort) == 0) {
     float c1[16], c2[32];

@@ -179,7 +179,7 @@ __device__ __forceinline__ void phase2(Tile& T, F mma, Fg dwg, Fc dwc) {
     }
     __syncwarp();
   } else if (DW && (T.w8 == 4 || T.w8 == 5)) {
-    if (tc::elect_one()) {
+    if (!failed(T) && tc::elect_one()) {
       if (T.w8 == 4) dwg();
       else dwc();
       tc::mma_commit(&T.bars->dw);
@@ -695,8 +695,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
   }
 
   // ---- epilogue: loss sums, decoder-gradient partial row, tensor memory ----
-  tiles_free(T);
-  if (!alive && w8 == 0 && lane == 0) atomicOr(a.status, kStatusPaperRender);
+  const bool done = tile_end(T, a.status, kStatusPaperRender);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -704,7 +703,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
   for (int i = tid; i < kPart; i += blockDim.x) prow[i] = 0.f;
   __syncthreads();
   if (BWD) {
-    if (dw_acc && *reinterpret_cast<volatile int*>(&T.bars->abort) == 0) {
+    if (dw_acc && done) {
       // warp w (mod 4) holds rows 16 w .. 16 w + 15 of every M = 64 product in its lanes 0..15
       const int m = 16 * wq + lane, n1 = half ? kU : kZ;
       float d[32];

@@ -130,8 +130,6 @@ __global__ void voxel_index_kernel(GridDesc g, const float* __restrict__ xq, int
 
 using namespace gs;
 
-static_assert(kStatusRender == 2, "render_tc_kernel reports a bounded wait that ran out as bit 1 (value 2)");
-
 gs_status gs_launch_render(const gs_ctx* ctx, const float* theta, const uint16_t* theta_bf16, const gs_batch* b,
                            const float* dloss, float* grad, float* rgb_hat, float* d_hat, float* wsum, int mode,
                            cudaStream_t st) {

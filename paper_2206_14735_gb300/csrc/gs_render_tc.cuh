@@ -306,7 +306,9 @@ struct Group {
 };
 
 // ---- the compact render kernel's tile groups ------------------------------------------------
-// A tile group's barriers: the phase's products done, its weight-gradient products done
+// A tile group's barriers: the phase's products done, its weight-gradient products done; and which
+// bounded waits ran out: on `done`, on `dw` at parity 0 or 1 (kAbortDw << parity)
+constexpr int kAbortDone = 1, kAbortDw = 2;
 struct TileBars {
   uint64_t done, dw;
   int abort;
@@ -336,6 +338,10 @@ struct Tile {
   uint32_t ph_done, ph_dw;  // parities of the next completions
   bool dw_pending;          // weight-gradient products may still read the tiles
 };
+// A bounded wait of the group ran out (every thread reads the same between two group barriers).  The
+// group then issues no further weight-gradient products (a second completion owed would make the
+// parities ambiguous) and leaves its loop at the next phase_wait.
+__device__ __forceinline__ bool failed(const Tile& T) { return *reinterpret_cast<volatile int*>(&T.bars->abort) != 0; }
 // Operand rows of this warp written -> once all warps have met, one thread of warp 0 issues the
 // phase's products and (adjoint phases) one of warp 4 the weight-gradient products that
 // read the same tiles.
@@ -353,7 +359,7 @@ __device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa,
     }
     __syncwarp();
   } else if (TYPE >= 3 && T.w8 == 4) {
-    if (tc::elect_one()) {
+    if (!failed(T) && tc::elect_one()) {
       issue_phase_dw<P, TYPE>(tcol, sa, dw_acc);
       tc::mma_commit(&T.bars->dw);
     }
@@ -365,22 +371,41 @@ __device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa,
 // barrier; false (for every thread) if they never complete
 __device__ __forceinline__ bool phase_wait(Tile& T) {
   if (T.w8 == 1 && tc::elect_one() && !tc::mbar_wait(&T.bars->done, T.ph_done, kMbarLimit))
-    *reinterpret_cast<volatile int*>(&T.bars->abort) = 1;
+    atomicOr(&T.bars->abort, kAbortDone);
   T.ph_done ^= 1u;
   group_sync<kTileThreads>(T.g);
   tc::fence_after_sync();
-  return *reinterpret_cast<volatile int*>(&T.bars->abort) == 0;
+  return !failed(T);
 }
 // no weight-gradient product reads the tiles.  Every lane polls by itself and may leave at another
 // try than its neighbours; the warp goes on together, as the tcgen05 instructions that follow require.
 __device__ __forceinline__ void tiles_free(Tile& T) {
   if (T.dw_pending) {
-    if (!tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit)) *reinterpret_cast<volatile int*>(&T.bars->abort) = 1;
+    if (!tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit)) atomicOr(&T.bars->abort, kAbortDw << T.ph_dw);
     T.ph_dw ^= 1u;
     T.dw_pending = false;
     __syncwarp();
     tc::fence_after_sync();
   }
+}
+// The end of a group's work, called by all of its threads: no product of the group is in flight any
+// more.  After a bounded wait that ran out, the status word takes `bit` and one thread waits once
+// more (bounded) for the products that may still run: what follows reuses the tiles' space and
+// releases the tensor memory that they read and write.  The CTA meets after this call and before
+// either.  false if a wait ran out.
+__device__ __forceinline__ bool tile_end(Tile& T, int* status, int bit) {
+  tiles_free(T);
+  group_sync<kTileThreads>(T.g);
+  if (!failed(T)) return true;
+  if (T.w8 == 0 && tc::elect_one()) {
+    atomicOr(status, bit);
+    tc::mbar_wait(&T.bars->done, T.ph_done ^ 1u, kMbarLimit);
+    const int why = *reinterpret_cast<volatile int*>(&T.bars->abort);
+    for (uint32_t parity = 0; parity < 2; ++parity)
+      if (why & (kAbortDw << parity)) tc::mbar_wait(&T.bars->dw, parity, kMbarLimit);
+  }
+  __syncwarp();
+  return false;
 }
 
 // every thread of the group: bounded wait until the weight-gradient MMAs are done with the tiles
@@ -1303,9 +1328,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
   }
 
   // ---- epilogue: loss and decoder-gradient partials, tensor memory ----
-  tiles_free(T);
-  if (!alive && w8 == 0 && lane == 0) atomicOr(a.status, 2);
-
+  const bool done = tile_end(T, a.status, kStatusRender);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -1315,7 +1338,7 @@ __global__ void __launch_bounds__(GR * kTileThreads, 1) render_tc_kernel(const _
       reinterpret_cast<float*>(gbase + (size_t)(i / kMlpPad) * L::group_bytes)[i % kMlpPad] = 0.f;
     __syncthreads();
     float* macc = reinterpret_cast<float*>(tileA);
-    if (half == 0 && dw_acc && *reinterpret_cast<volatile int*>(&T.bars->abort) == 0) {
+    if (half == 0 && dw_acc && done) {
       // The weight-gradient accumulators: warp w holds rows 16 w .. 16 w + 15 of every M = 64
       // product in its lanes 0..15.  Rows 32 .. 63 of dW1 and dW3 (16 .. 31 of dW2) are the
       // adjoints' second parts; without one they mean nothing.

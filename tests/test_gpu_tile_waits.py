@@ -82,3 +82,64 @@ int main() {
 
 def test_a_warp_leaves_the_tile_wait_together(tmp_path):
     run_program(tmp_path, CONVERGE)
+
+
+DRAIN = COMMON + r"""
+// what the group saw: threads with true, with false, whether the late arrival had come, the status word
+struct Seen { int good, bad, arrived, status; };
+// scenario 0: every product complete; 1: the weight-gradient products never do; 2: a phase wait ran out
+// before, its products complete 1 ms late; 3: weight-gradient products 1 ms late, within the wait; 4: a
+// wait for the weight-gradient products ran out before, they complete 1 ms late
+__global__ void run(int scenario, Seen* out) {
+  __shared__ TileBars bars;
+  __shared__ volatile int came;
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&bars.done, 1);
+    tc::mbar_init(&bars.dw, 1);
+    tc::fence_mbar_init();
+    bars.abort = scenario == 2 ? kAbortDone : scenario == 4 ? kAbortDw : 0;
+    came = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x >= kTileThreads) {  // the ninth warp
+    if (threadIdx.x == kTileThreads && scenario >= 2) {
+      pause(2000000);
+      came = 1;
+      __threadfence_block();
+      arrive(scenario == 2 ? &bars.done : &bars.dw);
+    }
+    return;
+  }
+  Tile T;
+  T.bars = &bars;
+  T.g = 0;
+  T.w8 = threadIdx.x >> 5;
+  T.ph_done = scenario == 2 ? 1u : 0u;  // a phase wait flips it, also when it runs out
+  T.ph_dw = scenario == 4 ? 1u : 0u;
+  T.dw_pending = scenario == 1 || scenario == 3;
+  const bool ok = tile_end(T, &out->status, 64);
+  group_sync<kTileThreads>(0);  // the caller's barrier
+  atomicAdd(ok ? &out->good : &out->bad, 1);
+  if (threadIdx.x == 0) out->arrived = came;
+}
+int main() {
+  const int want[5][4] = {{256, 0, 0, 0}, {0, 256, 0, 64}, {0, 256, 1, 64}, {256, 0, 1, 0}, {0, 256, 1, 64}};
+  Seen* d;
+  if (cudaMalloc(&d, sizeof(Seen)) != cudaSuccess) return 2;
+  for (int s = 0; s < 5; ++s) {
+    Seen h;
+    cudaMemset(d, 0, sizeof(Seen));
+    run<<<1, kTileThreads + 32>>>(s, d);
+    if (cudaMemcpy(&h, d, sizeof(Seen), cudaMemcpyDeviceToHost) != cudaSuccess) return 3;
+    const int got[4] = {h.good, h.bad, h.arrived, h.status};
+    printf("%d: %d %d %d %d\n", s, got[0], got[1], got[2], got[3]);
+    for (int k = 0; k < 4; ++k)
+      if (got[k] != want[s][k]) return 1;
+  }
+  return 0;
+}
+"""
+
+
+def test_a_wait_that_runs_out_is_reported_and_drained(tmp_path):
+    run_program(tmp_path, DRAIN)
