@@ -401,9 +401,11 @@ __global__ void __launch_bounds__(kThreads, 1) paper_smooth_kernel(Args a) {
   write_partials(a, sG, sL);
 }
 
-// phi(x) and (grad != nullptr) grad_x phi(x) of the geometry decoder, one thread per point
-__global__ void __launch_bounds__(128) paper_query_kernel(GridDesc g, const float* __restrict__ theta,
-                                                          const float* __restrict__ xq, int P, float* sdf,
+// phi(x) and (grad != nullptr) grad_x phi(x) of the geometry decoder, one thread per point.  Large
+// calls wait for their corner loads: four blocks per SM.  Left alone, the compiler takes 143 registers,
+// three blocks, and 300000 points take 87 us (with the gradient 126) for 76 (107).
+__global__ void __launch_bounds__(128, 4) paper_query_kernel(GridDesc g, const float* __restrict__ theta,
+                                                             const float* __restrict__ xq, int P, float* sdf,
                                                           float* grad) {
   __shared__ __align__(16) float sg[kGeoPad];
   __shared__ float hs[128][kH + 1];  // each thread's layer-1 activations (stride 33: conflict-free)

@@ -206,17 +206,21 @@ constexpr int kSensFloats = kPaper ? paper::S_gb3 : oW2 + kH1;
 // p = d phi / d z at z (sd: the decoder floats above in shared memory; hs: 64 floats of the
 // calling thread's shared scratch for the paper decoder's hidden layers)
 template <bool kPaper>
-__device__ __forceinline__ void dphi_dz(const float* sd, const float z[kZ], float* hs, float p[kZ]) {
-  float e[kH1];  // d phi / d (layer-1 output), masked
-  if constexpr (!kPaper) {
+__device__ __forceinline__ void dphi_dz(const float* sd, const float (&z)[kZ], float* hs, float (&p)[kZ]) {
+  if constexpr (!kPaper) {  // a unit and its part of p from one read of W1's row
+    static_assert(oW1 == sW1, "w1_row reads this copy's rows");
 #pragma unroll
+    for (int k = 0; k < kZ; ++k) p[k] = 0.f;
+#pragma unroll 4
     for (int j = 0; j < kH1; ++j) {
-      float y = sd[ob1 + j];
+      float w[kZ];
+      w1_row(sd, j, w);
+      const float e = w1_dot(w, z, sd[ob1 + j]) > 0.f ? sd[oW2 + j] : 0.f;
 #pragma unroll
-      for (int k = 0; k < kZ; ++k) y = fmaf(sd[oW1 + j * kZ + k], z[k], y);
-      e[j] = y > 0.f ? sd[oW2 + j] : 0.f;
+      for (int k = 0; k < kZ; ++k) p[k] = fmaf(w[k], e, p[k]);
     }
   } else {
+    float e[paper::kH];  // d phi / d (layer-1 output), masked
     unsigned m1 = 0;
 #pragma unroll
     for (int j = 0; j < paper::kH; ++j) {
@@ -242,13 +246,13 @@ __device__ __forceinline__ void dphi_dz(const float* sd, const float z[kZ], floa
       for (int j = 0; j < paper::kH; ++j) v = fmaf(sd[paper::S_gW2 + j * paper::kH + i], e2[j], v);
       e[i] = ((m1 >> i) & 1u) ? v : 0.f;
     }
-  }
 #pragma unroll
-  for (int k = 0; k < kZ; ++k) {
-    float s = 0.f;
+    for (int k = 0; k < kZ; ++k) {
+      float s = 0.f;
 #pragma unroll
-    for (int j = 0; j < kH1; ++j) s = fmaf(sd[oW1 + j * kZ + k], e[j], s);
-    p[k] = s;
+      for (int j = 0; j < paper::kH; ++j) s = fmaf(sd[paper::S_gW1 + j * kZ + k], e[j], s);
+      p[k] = s;
+    }
   }
 }
 
@@ -274,9 +278,11 @@ struct EikPoseArgs {
 // ray's sums to its frame's six derivatives
 // kRec: the batch's Eikonal records hold the sensitivity; without the decoder's evaluation the
 // kernel takes 64 registers for 168 (the paper's decoder), and its corner loads get more than twice
-// the warps: 146 us for 8192 x 132, now 74
+// the warps: 146 us for 8192 x 132, now 74.  Without records the compact decoder's rows are read once, for
+// the unit and its part of p: with every weight in flight the kernel took 190 registers, two blocks
+// per SM for four, and 111 us for 8192 x 96; now 91
 template <bool kPaper, bool kRec>
-__global__ void __launch_bounds__(128, kRec ? 8 : (kPaper ? 3 : 0)) eikonal_pose_kernel(EikPoseArgs a) {
+__global__ void __launch_bounds__(128, kRec ? 8 : (kPaper ? 3 : 4)) eikonal_pose_kernel(EikPoseArgs a) {
   __shared__ __align__(16) float sd[kRec ? 4 : kSensFloats<kPaper>];
   __shared__ __align__(16) float sp[128][kZ];  // this thread's p, read level by level
   __shared__ float sh[kPaper && !kRec ? 128 : 1][kPaper && !kRec ? 65 : 1];  // the paper decoder's hidden layers
