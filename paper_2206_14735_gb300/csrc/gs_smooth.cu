@@ -206,6 +206,11 @@ struct QueryBwdArgs {
   float* grad;
 };
 
+// Large calls are bound by the reductions, 32 of 16 bytes a point, most of all by the ones that meet on
+// the few vertices of the coarse levels.  Those come last, when the warps have drifted apart, and five
+// CTAs per SM share them: 40000 / 300000 points of the room 101 / 515 us with the coarse levels first
+// and eight CTAs, now 87 / 486; of the cube, whose levels are all crowded, 105 / 508, now 99 / 511.
+constexpr int kQueryBwdCtasPerSm = 5;
 __global__ void __launch_bounds__(kSmoothWarps * 32) query_backward_kernel(QueryBwdArgs a) {
   __shared__ __align__(16) float sm[kSmemMlp];
   __shared__ __align__(16) float acc[kH1 * kZ + kH1 + kH1 + 4];  // dW1 | db1 | dW2[0,:] | db2[0]
@@ -267,7 +272,7 @@ __global__ void __launch_bounds__(kSmoothWarps * 32) query_backward_kernel(Query
     }
     if (valid) {
 #pragma unroll
-      for (int l = 0; l < kLevels; ++l) {
+      for (int l = kLevels - 1; l >= 0; --l) {  // the crowded coarse levels last
         const Cell c = locate(a.g, l, y);
         float dw[8][3], w[8];
         corner_weights(c.f, w);
@@ -346,7 +351,7 @@ gs_status gs_launch_query_backward(const gs_ctx* ctx, const float* theta, const 
   a.dgrad = dgrad;
   a.grad = grad;
   const int per = kSmoothWarps * 32;
-  const int blocks = (int)std::min<long long>(((long long)P + per - 1) / per, 8LL * ctx->num_sms);
+  const int blocks = (int)std::min<long long>(((long long)P + per - 1) / per, (long long)kQueryBwdCtasPerSm * ctx->num_sms);
   query_backward_kernel<<<blocks, per, 0, st>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
