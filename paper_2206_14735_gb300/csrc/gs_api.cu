@@ -238,6 +238,9 @@ static gs_status render_common(gs_ctx* ctx, const char* who, const float* theta,
   cudaStream_t st = (cudaStream_t)stream;
   ctx->last_stream = st;
   const float* dl = dloss ? dloss : ctx->default_dloss;
+  // written as 16-byte vectors
+  if ((mode & 2) && batch->R > 0 && batch->dz && !aligned16(batch->dz))
+    return fail(ctx, GS_ERR_ALIGN, "batch dz is not 16-byte aligned");
   if (ctx->cfg.arch == GS_ARCH_PAPER) {
     if (batch->dz && (reinterpret_cast<uintptr_t>(batch->dz) & 15u)) return fail(ctx, GS_ERR_ALIGN, "batch dz is not 16-byte aligned");
     if (gs_launch_paper(ctx, theta, batch, dl, grad, loss, rgb_hat, d_hat, wsum, mode, st) != GS_OK)
