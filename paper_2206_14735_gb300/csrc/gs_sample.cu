@@ -94,7 +94,9 @@ __global__ void __launch_bounds__(128) sample_smooth_kernel(SmoothArgs a) {
 // words at 8192 rays.
 // The two sorted lists merge by rank: a stratified sample follows the guided ones below it, a
 // guided one the stratified ones up to it (ties stratified first), so a sample's place is its own
-// index plus one binary search in the other list.
+// index plus one binary search in the other list.  Both searches ask the merge's own question,
+// "stratified <= guided", so the places are all different for any depths (an infinite guide_half
+// makes the guided ones NaN, which go first).
 constexpr int kSampleWarps = 16;
 __global__ void __launch_bounds__(kSampleWarps * 32) sample_rays_kernel(SampleArgs a, SmoothArgs sm, int ray_blocks) {
   __shared__ float list[kSampleWarps][GS_MAX_SAMPLES];
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(kSampleWarps * 32) sample_rays_kernel(SampleAr
         const int base = lo;
         while (lo < hi) {
           const int m = (lo + hi) >> 1;
-          if (strat ? l[m] < tk : l[m] <= tk) lo = m + 1;
+          if (strat ? !(tk <= l[m]) : l[m] <= tk) lo = m + 1;
           else hi = m;
         }
         const int at = (strat ? k : k - a.Ns) + lo - base;
