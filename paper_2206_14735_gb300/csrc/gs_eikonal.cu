@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kCompactThreads) eik_compact_kernel(const uint
 // swizzle, parts `b_plane` apart
 template <int APL, int BPL, int N, int K>
 __device__ __forceinline__ void et_mma(uint32_t d, uint32_t ta, uint32_t b0, uint32_t b_plane) {
-  constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 128, N);
+  constexpr uint32_t idesc = tc::instr_desc(128, N);
   const uint32_t blo = tc::desc_lo(b0, 128u);
   bool first = true;
 #pragma unroll
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kEtThreads, 1) eikonal_tc_kernel(EikArgs a) {
         }
         store_row_planes<3, kZ, kJPlane>(Jt, row, jv);
       }
-      // C += M^T J over the tile's 128 samples, issued by thread 32 of the group; the scatter
+      // C += M^T J over the tile's 128 samples, issued by a lane of the second warp; the scatter
       // below runs meanwhile and the tiles are rewritten only after dw_wait
       tc::fence_smem_async();
       tc::fence_before_sync();
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(kEpThreads, 1) eikonal_paper_tc_kernel(EikArgs
       for (int j = 0; j < kH; ++j) v[j] = ((m1 >> j) & 1u) ? v[j] : 0.f;
       store_row_planes<3, kH, kQ32>(R1, row, v);
     }
-    // C1 += PM^T J and C2 += M2^T VJ, issued by thread 32 of the group
+    // C1 += PM^T J and C2 += M2^T VJ, issued by a lane of the second warp
     tc::fence_smem_async();
     tc::fence_before_sync();
     group_sync(gi);

@@ -193,7 +193,7 @@ __device__ __forceinline__ void phase2(Tile& T, F mma, Fg dwg, Fc dwc) {
 // and 1 from tensor memory (ta), part 2 from the A tile at a0, B's parts kTW apart
 template <int N, int K>
 __device__ __forceinline__ void mma3(uint32_t d, uint32_t ta, uint32_t a0, uint32_t b0) {
-  constexpr uint32_t sbo = K * 16u, idesc = tc::instr_desc(tc::KIND_BF16, 128, N);
+  constexpr uint32_t sbo = K * 16u, idesc = tc::instr_desc(128, N);
   const uint32_t alo = tc::desc_lo(a0 + 2 * kAP, 128u), blo = tc::desc_lo(b0, 128u);
   bool first = true;
 #pragma unroll

@@ -413,7 +413,7 @@ template <int K>
 __device__ __forceinline__ bool tc_phase(uint32_t tcol, const uint8_t* A, const uint8_t* B, uint64_t* mbar,
                                          uint32_t& phase, int* abort) {
   constexpr uint32_t sbo = (uint32_t)(K * 2 / 16) * 128u;
-  constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 128, 32);
+  constexpr uint32_t idesc = tc::instr_desc(128, 32);
   tc::fence_smem_async();
   tc::fence_before_sync();
   __syncthreads();

@@ -42,13 +42,11 @@ namespace gs {
 // FP32 by the tensor core: 6 MMAs per K step give FP32-grade products (the dropped terms
 // are below 2^-24 relative), 1 MMA per step is the plain BF16 form.
 struct PrecBF16x3 {
-  static constexpr int kind = tc::KIND_BF16;
   static constexpr int es = 2;      // bytes per operand element
   static constexpr int kmma = 16;   // K per MMA instruction
   static constexpr int planes = 3;
 };
 struct PrecBF16 {
-  static constexpr int kind = tc::KIND_BF16;
   static constexpr int es = 2;
   static constexpr int kmma = 16;
   static constexpr int planes = 1;
@@ -232,7 +230,7 @@ __device__ __forceinline__ void store_w(uint8_t* planes, uint32_t wplane, int K,
 template <int APL, int BPL, int SUM, int N>
 __device__ __forceinline__ void issue_mma_dw(uint32_t d, uint32_t a0, uint32_t a_plane, uint32_t a_kstride,
                                              uint32_t b0, uint32_t b_plane, uint32_t b_kstride, bool acc) {
-  constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 64, N) | (1u << 15) | (1u << 16);
+  constexpr uint32_t idesc = tc::instr_desc(64, N) | (1u << 15) | (1u << 16);
   uint32_t alo = tc::desc_lo(a0, a_kstride), blo = tc::desc_lo(b0, b_kstride);
 #pragma unroll 2
   for (int s = 0; s < 8; ++s) {  // K = 128 samples, 16 per MMA
@@ -256,7 +254,7 @@ __device__ __forceinline__ void issue_mma_dw(uint32_t d, uint32_t a0, uint32_t a
 // issuing thread spent about 15 instructions per MMA, which the whole group waits for.
 template <class P, int N, int K>
 __device__ __forceinline__ void tile_mma(uint32_t d, uint32_t ta, uint32_t b0, uint32_t wplane) {
-  constexpr uint32_t idesc = tc::instr_desc(P::kind, 128, N);
+  constexpr uint32_t idesc = tc::instr_desc(128, N);
   const uint32_t blo = tc::desc_lo(b0, 128u);
   bool first = true;
 #pragma unroll
@@ -280,7 +278,7 @@ __device__ __forceinline__ void tile_mma(uint32_t d, uint32_t ta, uint32_t b0, u
 template <class P, int N, int KA>
 __device__ __forceinline__ void tile_mma_dw(uint32_t d, uint32_t a0, uint32_t b0, bool acc) {
   using L = TcLayout<P>;
-  constexpr uint32_t idesc = tc::instr_desc(tc::KIND_BF16, 64, N) | (1u << 15) | (1u << 16);
+  constexpr uint32_t idesc = tc::instr_desc(64, N) | (1u << 15) | (1u << 16);
   constexpr uint32_t ra = L::row_stride(KA), rb = N * 16u;
   const uint32_t alo = tc::desc_lo(a0, ra), blo = tc::desc_lo(b0, rb);
 #pragma unroll
@@ -295,8 +293,8 @@ __device__ __forceinline__ void tile_mma_dw(uint32_t d, uint32_t a0, uint32_t b0
 
 // per-group MMA machinery
 struct Group {
-  uint64_t* mbar;     // completion of the phase MMAs (issued by thread 0 of the group)
-  uint64_t* mbar_dw;  // completion of the weight-gradient MMAs (issued by thread 32)
+  uint64_t* mbar;     // completion of the phase MMAs (issued by a lane of the group's first warp)
+  uint64_t* mbar_dw;  // completion of the weight-gradient MMAs (a lane of its second warp)
   int* abort;
   uint32_t tcol;      // tensor-memory address of this group's column 0
   uint32_t phase;     // parity of the next completion on mbar

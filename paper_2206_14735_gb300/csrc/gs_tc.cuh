@@ -40,14 +40,12 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo) { retu
 __host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
 __device__ __forceinline__ uint64_t desc_of(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 
-enum Kind { KIND_TF32 = 0, KIND_BF16 = 1 };
-
-// Instruction descriptor for kind::tf32 / kind::f16: D = F32, A and B K-major,
+// Instruction descriptor for kind::f16 on bfloat16 operands: D = F32, A and B K-major,
 // N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-__host__ __device__ constexpr uint32_t instr_desc(int kind, int M, int N) {
-  return (1u << 4)                                                   // D format F32
-         | ((kind == KIND_TF32 ? 2u : 1u) << 7)                      // A format: TF32 = 2, BF16 = 1
-         | ((kind == KIND_TF32 ? 2u : 1u) << 10)                     // B format
+__host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
+  return (1u << 4)     // D format F32
+         | (1u << 7)   // A format BF16
+         | (1u << 10)  // B format BF16
          | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
