@@ -600,7 +600,9 @@ __global__ void __launch_bounds__(128) prop_backward_tc_kernel(PropBwdArgs a, in
   // holds rows 4 i .. 4 i + 3 of dW2's columns 8 c .. and of dW1's columns 3 c .. (the twelfth is
   // nobody's), every lane its b1 and b2 rows, lane j entry j of w3.  A lane per row took 47 words
   // from shared memory per bin (one 32-column row, broadcast) where the tiles take 21: 217 us for
-  // 16384 rays, now 191.
+  // 16384 rays, now 191.  A ray's 32 bins are summed by themselves and then added: one FP32 chain over
+  // all bins of all rays, whose terms cancel within a ray, errs the more the more rays there are (and
+  // costs the same).
   const int i0 = 4 * (lane >> 2), c0 = lane & 3;
   float gW2[4][8], gW1[4][3], gb1[4], gb2[4], gw3 = 0.f, gb3 = 0.f;
 #pragma unroll
@@ -673,6 +675,7 @@ __global__ void __launch_bounds__(128) prop_backward_tc_kernel(PropBwdArgs a, in
     for (int k = 0; k < kPIn; ++k) row[rU + k] = u[k];
     row[rDl] = dl;
     __syncwarp();
+    float tW2[4][8] = {}, tW1[4][3] = {}, tb1[4] = {}, tb2[4] = {}, tw3 = 0.f, tb3 = 0.f;  // this ray's
 #pragma unroll 2
     for (int s2 = 0; s2 < 32; ++s2) {  // sums over the warp's 32 bin rows
       const float* rw = st + s2 * kRow;
@@ -685,16 +688,27 @@ __global__ void __launch_bounds__(128) prop_backward_tc_kernel(PropBwdArgs a, in
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) gW2[x][q] = fmaf(x2[x], y[q], gW2[x][q]);
+        for (int q = 0; q < 8; ++q) tW2[x][q] = fmaf(x2[x], y[q], tW2[x][q]);
 #pragma unroll
-        for (int q = 0; q < 3; ++q) gW1[x][q] = fmaf(x1[x], ui[q], gW1[x][q]);
-        gb2[x] += x2[x];
-        gb1[x] += x1[x];
+        for (int q = 0; q < 3; ++q) tW1[x][q] = fmaf(x1[x], ui[q], tW1[x][q]);
+        tb2[x] += x2[x];
+        tb1[x] += x1[x];
       }
       const float dls = rw[rDl];
-      gw3 = fmaf(dls, rw[rA2 + lane], gw3);
-      gb3 += dls;
+      tw3 = fmaf(dls, rw[rA2 + lane], tw3);
+      tb3 += dls;
     }
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) gW2[x][q] += tW2[x][q];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) gW1[x][q] += tW1[x][q];
+      gb1[x] += tb1[x];
+      gb2[x] += tb2[x];
+    }
+    gw3 += tw3;
+    gb3 += tb3;
     __syncwarp();
   }
 #pragma unroll
