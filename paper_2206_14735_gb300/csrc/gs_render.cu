@@ -65,8 +65,10 @@ __global__ void __launch_bounds__(256) finalize_kernel(const float* loss_part, c
 // SDF query and cell lookup
 // ------------------------------------------------------------------------------------
 // Bound by the latency of its gathers; W1's rows are read once, as 16-byte vectors, for a unit and its
-// part of p, and 64-thread blocks spread small batches: 4096 points, cold, 18.8 -> 15.0 us.
-__global__ void __launch_bounds__(64) query_kernel(GridDesc g, const float* __restrict__ theta, const float* __restrict__ xq, int P,
+// part of p.  Room, 4096 / 40000 / 300000 points with the gradient: 23 / 50 / 167 us with a read per use
+// and 1.5 KB of spills, now 17 / 21 / 60 (blocks of 64 threads, each with its own copy of the decoder,
+// took 19 / 23 / 66).
+__global__ void __launch_bounds__(128) query_kernel(GridDesc g, const float* __restrict__ theta, const float* __restrict__ xq, int P,
                              float* sdf, float* grad) {
   __shared__ __align__(16) float sm[sb2 + 1];
   const float* mlp = theta + g.n_grid;
@@ -195,7 +197,7 @@ gs_status gs_launch_finalize(const gs_ctx* ctx, const gs_batch* b, float* loss, 
 
 gs_status gs_launch_query(const gs_ctx* ctx, const float* theta, const float* x, int P, float* sdf, float* grad,
                           cudaStream_t st) {
-  if (P > 0) query_kernel<<<(P + 63) / 64, 64, 0, st>>>(ctx->grid, theta, x, P, sdf, grad);
+  if (P > 0) query_kernel<<<(P + 127) / 128, 128, 0, st>>>(ctx->grid, theta, x, P, sdf, grad);
   return cudaPeekAtLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
