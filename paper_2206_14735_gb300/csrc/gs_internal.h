@@ -14,9 +14,25 @@ constexpr int kRenderCtasPerSm = 1;  // persistent render CTAs per SM
 constexpr int kStoreFloatsPerSample = 100;  // stored activations: z 16, a1 32, (phi, h) 16, a2 32, c 3 + 1 pad
 constexpr int kPaperStoreFloatsPerSample = 156;  // paper architecture: z 16, cf 6 + phi + pad, c 3 + pad, 4 x 32 hidden
 // Tile groups (8 warps) per CTA of the compact render kernel.  With a reverse pass two of 128
-// registers a thread; a forward-only call holds less per thread, and its third group at 80
-// registers fills the waits of the other two: 8192 rays x 132, 197 us with two, 187 us with three.
+// registers a thread; a forward-only call holds less per thread, and a third group at 80 registers
+// fills the waits of the other two, where there is work for it.
 constexpr int kRenderGroups = 2, kForwardGroups = 3;
+// The forward-only form's groups.  A round of ray-quads over all groups takes longer with three (each
+// has fewer registers, and they share the data path): 1.1 to 1.2 times with few of them resident, 1.4
+// times with all, so three have to save a quarter of the rounds; a single chunk's state fits their
+// registers, and they never lose.  Without store, two against three groups, FP32 / BF16: 300 x 96 (one
+// round) 36 against 37 / 31 against 36 us, 1300 x 96 (two against one) 52 against 44 / 46 against 40,
+// 2000 x 132 (two each) 74 against 83 / 64 against 76, 4000 x 96 (four against three) 85 against 83 / 70
+// against 72, 8192 x 132 195 against 187 / 165 against 167, 32768 x 96 427 against 394 / 337 against 320.
+// Three chunks with the activation store spill most, 1.5 to 1.6 times a round: 32768 x 96 500 against 511
+// / 429 against 463, so there three have to halve the rounds (1300 x 96 56 against 48 / 50 against 47).
+inline int forward_groups(int rays, int ctas, int chunks, bool stored) {
+  const long long quads = ((long long)rays + 3) / 4;
+  auto rounds = [&](int groups) { return (quads + (long long)groups * ctas - 1) / ((long long)groups * ctas); };
+  const long long three = rounds(kForwardGroups), two = rounds(kRenderGroups);
+  const bool pays = chunks == 1 || (stored && chunks == 3 ? 5 * three < 3 * two : 4 * three <= 3 * two);
+  return pays ? kForwardGroups : kRenderGroups;
+}
 // Bits of the context's device status word: a kernel sets its bit when a bounded wait for its
 // tensor-core products ran out (it then stops early; that call's outputs are incomplete)
 constexpr int kStatusRender = 2, kStatusProposal = 4, kStatusEikonal = 8, kStatusPaperRender = 16,

@@ -23,11 +23,14 @@
 // before the operands moved to tensor memory, in bursts: the phases of a group load it in turn)
 // and each group's serial chain; DRAM and the tensor cores are below 20 %.  Hence two threads per
 // row (half the chain at the same shared and tensor memory), the phases' A operands in tensor
-// memory, two groups of 128 registers without spills (three at 80 registers measured slower
-// with a reverse pass: 607 against 476 us, at the same data path), the weight gradients' part pairs in as few products
-// as the tile layout allows.  Render call, 8192 x 96, stored: one thread per row and three groups
-// 523 us, two threads and two groups 476 us, A operands in tensor memory 451 us; forward only,
-// 8192 x 132: 251, 223, 197 us, and 187 us with three groups, which only that form has.
+// memory, two groups of 128 registers (three at 80 registers measured slower with a reverse pass: 607
+// against 476 us, at the same data path), the weight gradients' part pairs in as few products as the
+// tile layout allows.  What does not fit 128 registers goes to local memory, through the same data
+// path: with a reverse pass 62 bytes stored and 168 loaded a thread at three chunks, 230 and 412 at
+// five (the BF16 form 44 and 96 at three); forward only with two groups 0 to 8, with three at 80
+// registers 68 and 76 at three chunks, 124 and 140 at five.  Render call, 8192 x 96, stored: one thread
+// per row and three groups 523 us, two threads and two groups 476 us, A operands in tensor memory 451 us;
+// forward only, 8192 x 132: 251, 223, 195 us, and 187 us with three groups (forward_groups says when).
 #pragma once
 #include "gs_internal.h"
 #include <cuda_bf16.h>
@@ -1425,7 +1428,10 @@ gs_status launch_tc_t(const gs_ctx* ctx, RenderTcArgs& a, cudaStream_t st) {
 template <class P, int NCH>
 gs_status launch_tc_n(const gs_ctx* ctx, RenderTcArgs& a, int mode, cudaStream_t st) {
   constexpr int GR = kRenderGroups;  // tile groups in one CTA per SM
-  if (mode == 1) return launch_tc_t<P, NCH, kForwardGroups, true, false>(ctx, a, st);
+  if (mode == 1)
+    return forward_groups(a.R, ctx->render_ctas, NCH, a.store != nullptr) == kForwardGroups
+               ? launch_tc_t<P, NCH, kForwardGroups, true, false>(ctx, a, st)
+               : launch_tc_t<P, NCH, kRenderGroups, true, false>(ctx, a, st);
   if (mode == 2) return launch_tc_t<P, NCH, GR, false, true>(ctx, a, st);
   return launch_tc_t<P, NCH, GR, true, true>(ctx, a, st);
 }

@@ -75,10 +75,12 @@ def test_ragged_rays_render_as_whole_chunks(form, rays, n):
 
 
 @pytest.mark.parametrize("form", FORMS)
-def test_forward_of_more_rays_than_one_round(form):
+@pytest.mark.parametrize("n", [5, 33])
+def test_forward_of_more_rays_than_one_round(form, n):
     """Each tile group of the forward-only kernel takes several ray-quads here; in pieces of 1200 rays
-    it takes at most one.  A ray's outputs are the same bits."""
-    R, n, piece = 8 * 4 * torch.cuda.get_device_properties(0).multi_processor_count + 3, 5, 1200
+    it takes at most one, and from two chunks on the compact kernel has two groups for three then.  A
+    ray's outputs are the same bits."""
+    R, piece = 8 * 4 * torch.cuda.get_device_properties(0).multi_processor_count + 3, 1200
     w = _workload(form, R, n)
     p = Problem(w)
     th, mirror = _params(form, w, p)
