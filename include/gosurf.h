@@ -203,8 +203,10 @@ gs_status gs_forward(gs_ctx* ctx, const float* theta, const uint16_t* theta_bf16
  * gs_forward_backward) are read: that call must have seen the same theta and batch, and
  * GS_ERR_INVALID_ARG is returned when no forward pass of a batch with this R, N and t
  * pointer came first.  Otherwise everything is recomputed from theta.  Grid
- * gradients are accumulated with FP32 atomics (summation order not deterministic); decoder
- * gradients are reduced in a fixed order.  With batch->eik set, the grid gradient also
+ * gradients are accumulated with FP32 atomics (summation order not deterministic).  The
+ * decoder gradients' per-CTA sums are combined in a fixed order; inside a CTA several warps
+ * add to an entry in the order they arrive, so its last bits may differ from call to call.
+ * With batch->eik set, the grid gradient also
  * receives the deferred Eikonal term of every free-space sample (records written by
  * gs_eikonal on this batch before this call; see there). */
 gs_status gs_backward(gs_ctx* ctx, const float* theta, const uint16_t* theta_bf16, const gs_batch* batch,

@@ -81,7 +81,8 @@ inline void set_voxel(GridDesc& g, int l, float voxel) {
 // and a select in place of a division's reciprocal, its own steps and its range check with the
 // branch behind it; a sample needs 24 of them.  The power of two is exact, and keeps the
 // products clear of overflow; a quotient beyond 2^100 (or not finite) is left as it is: the
-// caller clamps it to the grid.
+// caller clamps it to the grid.  A quotient below about 2^-90, whose residuals underflow, lies on the
+// grid's face and may differ in its last bits.
 __host__ __device__ __forceinline__ float cell_coord(float d, float scale, float voxel, float recip) {
   const float a = d * scale;
   const float q0 = a * recip;

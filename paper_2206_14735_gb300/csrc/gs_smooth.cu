@@ -12,9 +12,10 @@
 // Bound by latency: 4096 points are one pass of every warp, in the render kernel's shadow only where that
 // leaves SMs idle.  Hence one visit of the corners for z and dz/dx (three before: features, gradient
 // and adjoint each gathered again), W1's rows read once as 16-byte vectors for the unit, its mask
-// and its part of p, the points dealt over the blocks first, and nothing spilled (568 bytes of
-// stack a thread before).  Step of 1024 rays x 64 and 4096 points: 130 -> 125 us; the query's
-// backward pass of 4096 points, cold: 28 -> 25 us.
+// and its part of p, and the points dealt over the blocks first; 230 registers, no spill.  The term by
+// itself, forward and backward, 300 / 4096 / 20000 / 100000 points: 43 / 49 / 133 / 507 us with three
+// visits (192 registers), now 36 / 44 / 96 / 330; forward only, where that form spilled 948 bytes, 35 /
+// 36 / 92 / 342 and now 27 / 27 / 49 / 140.
 #include <algorithm>
 
 #include "gs_internal.h"
