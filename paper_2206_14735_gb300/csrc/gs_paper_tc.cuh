@@ -179,7 +179,7 @@ __device__ __forceinline__ void phase2(Tile& T, F mma, Fg dwg, Fc dwc) {
     }
     __syncwarp();
   } else if (DW && (T.w8 == 4 || T.w8 == 5)) {
-    if (!failed(T) && tc::elect_one()) {
+    if (tc::elect_one()) {
       if (T.w8 == 4) dwg();
       else dwc();
       tc::mma_commit(&T.bars->dw);
@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(kPThreads, 1) paper_tc_kernel(const __grid_con
   }
 
   // ---- epilogue: loss sums, decoder-gradient partial row, tensor memory ----
-  const bool done = tile_end(T, a.status, kStatusPaperRender);
+  const bool done = tile_end(T, a.status, kStatusPaperRender) && alive;
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();

@@ -307,9 +307,8 @@ struct Group {
 };
 
 // ---- the compact render kernel's tile groups ------------------------------------------------
-// A tile group's barriers: the phase's products done, its weight-gradient products done; and which
-// bounded waits ran out: on `done`, on `dw` at parity 0 or 1 (kAbortDw << parity)
-constexpr int kAbortDone = 1, kAbortDw = 2;
+// A tile group's barriers: the phase's products done, its weight-gradient products done; and whether a
+// bounded wait ran out
 struct TileBars {
   uint64_t done, dw;
   int abort;
@@ -339,9 +338,8 @@ struct Tile {
   uint32_t ph_done, ph_dw;  // parities of the next completions
   bool dw_pending;          // weight-gradient products may still read the tiles
 };
-// A bounded wait of the group ran out (every thread reads the same between two group barriers).  The
-// group then issues no further weight-gradient products (a second completion owed would make the
-// parities ambiguous) and leaves its loop at the next phase_wait.
+// A bounded wait of the group ran out (every thread reads the same between two group barriers): the
+// group leaves its loop at the next phase_wait.
 __device__ __forceinline__ bool failed(const Tile& T) { return *reinterpret_cast<volatile int*>(&T.bars->abort) != 0; }
 // Operand rows of this warp written -> once all warps have met, one thread of warp 0 issues the
 // phase's products and (adjoint phases) one of warp 4 the weight-gradient products that
@@ -360,7 +358,7 @@ __device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa,
     }
     __syncwarp();
   } else if (TYPE >= 3 && T.w8 == 4) {
-    if (!failed(T) && tc::elect_one()) {
+    if (tc::elect_one()) {
       issue_phase_dw<P, TYPE>(tcol, sa, dw_acc);
       tc::mma_commit(&T.bars->dw);
     }
@@ -372,7 +370,7 @@ __device__ __forceinline__ void phase_issue(Tile& T, uint32_t tcol, uint32_t sa,
 // barrier; false (for every thread) if they never complete
 __device__ __forceinline__ bool phase_wait(Tile& T) {
   if (T.w8 == 1 && tc::elect_one() && !tc::mbar_wait(&T.bars->done, T.ph_done, kMbarLimit))
-    atomicOr(&T.bars->abort, kAbortDone);
+    atomicOr(&T.bars->abort, 1);
   T.ph_done ^= 1u;
   group_sync<kTileThreads>(T.g);
   tc::fence_after_sync();
@@ -382,7 +380,7 @@ __device__ __forceinline__ bool phase_wait(Tile& T) {
 // try than its neighbours; the warp goes on together, as the tcgen05 instructions that follow require.
 __device__ __forceinline__ void tiles_free(Tile& T) {
   if (T.dw_pending) {
-    if (!tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit)) atomicOr(&T.bars->abort, kAbortDw << T.ph_dw);
+    if (!tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit)) atomicOr(&T.bars->abort, 1);
     T.ph_dw ^= 1u;
     T.dw_pending = false;
     __syncwarp();
@@ -394,6 +392,9 @@ __device__ __forceinline__ void tiles_free(Tile& T) {
 // more (bounded) for the products that may still run: what follows reuses the tiles' space and
 // releases the tensor memory that they read and write.  The CTA meets after this call and before
 // either.  false if a wait ran out.
+// Weight-gradient products may be owed twice: the wait that ran out before a phase, and that phase's
+// own.  Then the first has parity ph_dw (the parity flips at every wait) and the second the other one;
+// owed once, only the other one blocks.  What is not owed runs to its limit.
 __device__ __forceinline__ bool tile_end(Tile& T, int* status, int bit) {
   tiles_free(T);
   group_sync<kTileThreads>(T.g);
@@ -401,9 +402,8 @@ __device__ __forceinline__ bool tile_end(Tile& T, int* status, int bit) {
   if (T.w8 == 0 && tc::elect_one()) {
     atomicOr(status, bit);
     tc::mbar_wait(&T.bars->done, T.ph_done ^ 1u, kMbarLimit);
-    const int why = *reinterpret_cast<volatile int*>(&T.bars->abort);
-    for (uint32_t parity = 0; parity < 2; ++parity)
-      if (why & (kAbortDw << parity)) tc::mbar_wait(&T.bars->dw, parity, kMbarLimit);
+    tc::mbar_wait(&T.bars->dw, T.ph_dw, kMbarLimit);
+    tc::mbar_wait(&T.bars->dw, T.ph_dw ^ 1u, kMbarLimit);
   }
   __syncwarp();
   return false;

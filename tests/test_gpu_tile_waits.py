@@ -89,7 +89,8 @@ DRAIN = COMMON + r"""
 struct Seen { int good, bad, arrived, status; };
 // scenario 0: every product complete; 1: the weight-gradient products never do; 2: a phase wait ran out
 // before, its products complete 1 ms late; 3: weight-gradient products 1 ms late, within the wait; 4: a
-// wait for the weight-gradient products ran out before, they complete 1 ms late
+// wait for the weight-gradient products ran out before, they complete 1 ms late; 5: and so did the wait
+// for the next phase's, both come late, one after the other
 __global__ void run(int scenario, Seen* out) {
   __shared__ TileBars bars;
   __shared__ volatile int came;
@@ -97,16 +98,18 @@ __global__ void run(int scenario, Seen* out) {
     tc::mbar_init(&bars.done, 1);
     tc::mbar_init(&bars.dw, 1);
     tc::fence_mbar_init();
-    bars.abort = scenario == 2 ? kAbortDone : scenario == 4 ? kAbortDw : 0;
+    bars.abort = scenario == 2 || scenario >= 4;
     came = 0;
   }
   __syncthreads();
   if (threadIdx.x >= kTileThreads) {  // the ninth warp
     if (threadIdx.x == kTileThreads && scenario >= 2) {
-      pause(2000000);
-      came = 1;
-      __threadfence_block();
-      arrive(scenario == 2 ? &bars.done : &bars.dw);
+      for (int k = 0; k < (scenario == 5 ? 2 : 1); ++k) {
+        pause(2000000);
+        came = k + 1;
+        __threadfence_block();
+        arrive(scenario == 2 ? &bars.done : &bars.dw);
+      }
     }
     return;
   }
@@ -115,7 +118,7 @@ __global__ void run(int scenario, Seen* out) {
   T.g = 0;
   T.w8 = threadIdx.x >> 5;
   T.ph_done = scenario == 2 ? 1u : 0u;  // a phase wait flips it, also when it runs out
-  T.ph_dw = scenario == 4 ? 1u : 0u;
+  T.ph_dw = scenario == 4 ? 1u : 0u;  // a wait flips it, also when it runs out
   T.dw_pending = scenario == 1 || scenario == 3;
   const bool ok = tile_end(T, &out->status, 64);
   group_sync<kTileThreads>(0);  // the caller's barrier
@@ -123,10 +126,10 @@ __global__ void run(int scenario, Seen* out) {
   if (threadIdx.x == 0) out->arrived = came;
 }
 int main() {
-  const int want[5][4] = {{256, 0, 0, 0}, {0, 256, 0, 64}, {0, 256, 1, 64}, {256, 0, 1, 0}, {0, 256, 1, 64}};
+  const int want[6][4] = {{256, 0, 0, 0}, {0, 256, 0, 64}, {0, 256, 1, 64}, {256, 0, 1, 0}, {0, 256, 1, 64}, {0, 256, 2, 64}};
   Seen* d;
   if (cudaMalloc(&d, sizeof(Seen)) != cudaSuccess) return 2;
-  for (int s = 0; s < 5; ++s) {
+  for (int s = 0; s < 6; ++s) {
     Seen h;
     cudaMemset(d, 0, sizeof(Seen));
     run<<<1, kTileThreads + 32>>>(s, d);
